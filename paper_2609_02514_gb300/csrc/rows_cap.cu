@@ -81,7 +81,13 @@ constexpr int HEADROOM = 256;       // of them above the sample's max at least
 constexpr int SKG = 16384;          // sketch entries (group maxima, as 16-bit order keys)
 constexpr int PCAP = 1024;          // ids at or above the payload's last value
 constexpr int GCAP = 1024;          // sketch groups re-read
-constexpr int SMEM_BF = HW * 4 + SKG * 2 + PCAP * 8;
+// Values below the counted ones go to one of HPAD counters just below them,
+// lane l's to the l-th: every lane adds to some counter, so that counting
+// takes no branch (a predicated reduction on shared memory is compiled into
+// one: 18.3 instructions a logit on flat rows) and no two lanes of a warp
+// add to the same dummy.  Counters below the final limit are never read.
+constexpr int HPAD = 32;
+constexpr int SMEM_BF = (HPAD + HW) * 4 + SKG * 2 + PCAP * 8;
 // sketch-led pass: a row is short when at most SHORT_IDS ids reach its
 // crossing (top_p = 1: when k <= SHORT_IDS); later rows take the pass when
 // at least SHORT_NUM / SHORT_DEN of the finished rows were short.  Its areas
@@ -159,20 +165,30 @@ __device__ __forceinline__ unsigned long long ex2_pair(unsigned long long z2, un
 }
 
 // Max of one chunk, as a packed pair (bfloat16: the max of its even and of
-// its odd elements; float32: the max of elements 0,2 and of 1,3).
+// its odd elements, NaN when one is NaN; float32: the max of all four).
 template <int DT>
 __device__ __forceinline__ uint32_t chunk_max2(const uint4 &w) {
     if (DT == ACES_BF16) {
-        const __nv_bfloat162 a = __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&w.x),
-                                         *reinterpret_cast<const __nv_bfloat162 *>(&w.y));
-        const __nv_bfloat162 b = __hmax2(*reinterpret_cast<const __nv_bfloat162 *>(&w.z),
-                                         *reinterpret_cast<const __nv_bfloat162 *>(&w.w));
-        const __nv_bfloat162 m = __hmax2(a, b);
+        const __nv_bfloat162 a = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&w.x),
+                                             *reinterpret_cast<const __nv_bfloat162 *>(&w.y));
+        const __nv_bfloat162 b = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&w.z),
+                                             *reinterpret_cast<const __nv_bfloat162 *>(&w.w));
+        const __nv_bfloat162 m = __hmax2_nan(a, b);
         return *reinterpret_cast<const uint32_t *>(&m);
     } else {
         return __float_as_uint(fmaxf(fmaxf(__uint_as_float(w.x), __uint_as_float(w.y)),
                                      fmaxf(__uint_as_float(w.z), __uint_as_float(w.w))));
     }
+}
+// the max of two such maxima
+template <int DT>
+__device__ __forceinline__ uint32_t max2(uint32_t x, uint32_t y) {
+    if (DT == ACES_BF16) {
+        const __nv_bfloat162 m = __hmax2_nan(*reinterpret_cast<const __nv_bfloat162 *>(&x),
+                                             *reinterpret_cast<const __nv_bfloat162 *>(&y));
+        return *reinterpret_cast<const uint32_t *>(&m);
+    }
+    return __float_as_uint(fmaxf(__uint_as_float(x), __uint_as_float(y)));
 }
 template <int DT>
 __device__ __forceinline__ float max2_value(uint32_t m2) {
@@ -221,6 +237,22 @@ __device__ __forceinline__ float chunks_expsum(const uint4 (&w)[UC], float c, fl
     return acc_total(acc0, acc1);
 }
 
+// maxima of chunks 0..3 and 4..7 (bfloat16: packed over all their pairs,
+// unpacked once); returns the packed max of both
+template <int DT>
+__device__ __forceinline__ uint32_t group_maxima(const uint4 (&w)[UC], float &g0, float &g1) {
+    uint32_t p[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        p[h] = chunk_max2<DT>(w[h * (UC / 2)]);
+#pragma unroll
+        for (int u = 1; u < UC / 2; ++u) p[h] = max2<DT>(p[h], chunk_max2<DT>(w[h * (UC / 2) + u]));
+    }
+    g0 = max2_value<DT>(p[0]);
+    g1 = max2_value<DT>(p[1]);
+    return max2<DT>(p[0], p[1]);
+}
+
 // element e of a chunk (e may be a run-time index)
 template <int DT>
 __device__ __forceinline__ float chunk_elem(const uint4 &w, int e) {
@@ -234,31 +266,9 @@ __device__ __forceinline__ float chunk_elem(const uint4 &w, int e) {
     }
 }
 
-// bits of the chunk's elements >= th (bfloat16: th is a bfloat16 value)
-template <int DT>
-__device__ __forceinline__ uint32_t chunk_hits(const uint4 &w, float th) {
-    if (DT == ACES_BF16) {
-        const __nv_bfloat162 t2 = __floats2bfloat162_rn(th, th);
-        const uint32_t wd[4] = {w.x, w.y, w.z, w.w};
-        uint32_t hm = 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t m = __hge2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&wd[q]), t2);
-            hm |= ((m & 1u) | ((m >> 15) & 2u)) << (2 * q);
-        }
-        return hm;
-    } else {
-        return (uint32_t)(__uint_as_float(w.x) >= th) | (uint32_t)(__uint_as_float(w.y) >= th) << 1 |
-               (uint32_t)(__uint_as_float(w.z) >= th) << 2 | (uint32_t)(__uint_as_float(w.w) >= th) << 3;
-    }
-}
-
-// adds 1 to the shared-memory counter at address addr when x < lim (one
-// predicated reduction: no branch)
-__device__ __forceinline__ void red_inc_lt(uint32_t addr, uint32_t x, uint32_t lim) {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %1, %2;\n\t@q red.shared.add.u32 [%0], 1;\n\t}"
-        :: "r"(addr), "r"(x), "r"(lim) : "memory");
+// adds 1 to the shared-memory counter at address addr
+__device__ __forceinline__ void red_inc(int addr) {
+    asm volatile("red.shared.add.u32 [%0], 1;" :: "r"(addr) : "memory");
 }
 
 // bfloat16 order key of a bfloat16 bit pattern (keys sort like values, -0
@@ -335,12 +345,12 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
     constexpr int EPC = E::EPC;
     constexpr bool BF = DT == ACES_BF16;
     extern __shared__ __align__(16) unsigned char smem[];
-    // bfloat16: [value counts: HW u32 | sketch: SKG u16 | ids >= the payload's
-    //           last value: PCAP u64]; the list of re-read groups reuses the
-    //           counts, the ordered ids the sketch, once each is read
-    uint32_t *hist = reinterpret_cast<uint32_t *>(smem);
-    uint16_t *sk = reinterpret_cast<uint16_t *>(smem + HW * 4);
-    unsigned long long *pay = reinterpret_cast<unsigned long long *>(smem + HW * 4 + SKG * 2);
+    // bfloat16: [HPAD dummies, value counts: HW u32 | sketch: SKG u16 | ids >=
+    //           the payload's last value: PCAP u64]; the list of re-read groups
+    //           reuses the counts, the ordered ids the sketch, once each is read
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem) + HPAD;
+    uint16_t *sk = reinterpret_cast<uint16_t *>(smem + (HPAD + HW) * 4);
+    unsigned long long *pay = reinterpret_cast<unsigned long long *>(smem + (HPAD + HW) * 4 + SKG * 2);
     uint32_t *glist = hist;
     unsigned long long *sorted = reinterpret_cast<unsigned long long *>(sk);
     // float32:  [records: CREC x (16 + 4) bytes | list: LCAP u64 | bin counts:
@@ -425,50 +435,35 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
     // ---- stream ----
     float k_t = -1e30f, m_t = -INFINITY, s_t = 0.f, e_t = 0.f;
     uint4 w[UC];
-    int tile0 = (int)(((long long)wid * a.pstride) % ntile);  // tile of (iteration 0, u = 0)
+    // this lane's byte offset of (iteration, u = 0): tile * 512 + lane * 16;
+    // the next chunk's is one addition and one unsigned min away (a tile
+    // index past ntile wraps around: off - tile_end is huge before that)
+    uint32_t off0 = (uint32_t)(((long long)wid * a.pstride) % ntile) * (TCH * 16) + lane * 16;
+    const uint32_t off_w = (uint32_t)a.pstride_w * (TCH * 16), off_it = (uint32_t)a.pstride_it * (TCH * 16);
+    const uint32_t tile_end = (uint32_t)ntile * (TCH * 16);
+    auto wrap = [&](uint32_t off) -> uint32_t { return min(off, off - tile_end); };
     // (iterations whose tiles all exist and are whole load without checks:
     // only the last iteration can hold fewer tiles, and only the row's last
     // tile can be partial)
-    // chunk u of iteration it, starting at tile `tile` (checked: bounds tested)
-    auto load_chunk = [&](int it, int u, int tile, bool checked) {
-        const int t = it * TPI + u * NWC + wid;
-        const int c = tile * TCH + lane;
-        w[u] = (!checked || (t < ntile && c < nch)) ? ldg16(row + (size_t)c * 16) : make_uint4(NI, NI, NI, NI);
-    };
     auto load = [&](int it) {
-        int tile = tile0;
-        const bool checked = (it + 1) * TPI > ntile || it == a.it_partial;
+        uint32_t off = off0;
+        if ((it + 1) * TPI > ntile || it == a.it_partial) {
 #pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            load_chunk(it, u, tile, checked);
-            tile += a.pstride_w;
-            if (tile >= ntile) tile -= ntile;
+            for (int u = 0; u < UC; ++u) {
+                const int t = it * TPI + u * NWC + wid;
+                w[u] = (t < ntile && off < (uint32_t)nch * 16u) ? ldg16(row + off) : make_uint4(NI, NI, NI, NI);
+                off = wrap(off + off_w);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < UC; ++u) {
+                w[u] = ldg16(row + off);
+                off = wrap(off + off_w);
+            }
         }
     };
-    // bit u: chunk u holds an id >= th
-    auto mask_of = [&](float th) -> uint32_t {
-        uint32_t hb = 0u;
-#pragma unroll
-        for (int u = 0; u < UC; ++u) hb |= (uint32_t)(max2_value<DT>(chunk_max2<DT>(w[u])) >= th) << u;
-        return hb;
-    };
-    // max and exp-sum of this iteration; returns mask_of(th), the iteration's
-    // max in im and the maxima of chunks 0..3 and 4..7 in g0, g1
-    // the iteration's maxima and the reference k_t raised to them; returns
-    // mask_of(th), the iteration's max in im and the maxima of chunks 0..3
-    // and 4..7 in g0, g1
-    auto head = [&](float th, float &im, float &g0, float &g1) -> uint32_t {
-        uint32_t hb = 0u;
-        g0 = -INFINITY;
-        g1 = -INFINITY;
-#pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            const float cmx = max2_value<DT>(chunk_max2<DT>(w[u]));
-            if (u < UC / 2) g0 = fmaxf(g0, cmx);
-            else g1 = fmaxf(g1, cmx);
-            hb |= (uint32_t)(cmx >= th) << u;
-        }
-        im = fmaxf(g0, g1);
+    // the iteration's max im raises m_t and the reference k_t
+    auto raise_ref = [&](float im) {
         m_t = fmaxf(m_t, im);
         const float gk = im * a.c;
         if (gk > k_t) {
@@ -478,7 +473,6 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             e_t *= sc;
             k_t = nk;
         }
-        return hb;
     };
     auto add_sum = [&](float gs) {
         const float t = s_t + gs;  // Neumaier
@@ -486,23 +480,20 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
         else e_t += (gs - t) + s_t;
         s_t = t;
     };
-    // max and exp-sum of this iteration (head, then the sum)
-    auto math = [&](float th, float &im, float &g0, float &g1) -> uint32_t {
-        const uint32_t hb = head(th, im, g0, g1);
-        add_sum(chunks_expsum<DT>(w, a.c, -k_t));
-        return hb;
-    };
     // the running max of the CTA (a lower bound of the row max at any time)
     auto publish_max = [&](float im) {
-        const float wm = warp_max(im);
-        if (lane == 0 && wm > -INFINITY) atomicMax(&s_mr, fkey(wm));
+        const uint32_t wm = __reduce_max_sync(0xffffffffu, fkey(im));
+        if (lane == 0 && wm > fkey(-INFINITY)) atomicMax(&s_mr, wm);
     };
     auto running_max = [&]() -> float { return fkey_inv(*reinterpret_cast<volatile uint32_t *>(&s_mr)); };
 
     // iteration 0: a strided sample (1/8 to 1/16 of a large row, spread over it)
     float im, g0, g1;
     load(0);
-    math(INFINITY, im, g0, g1);
+    uint32_t im2 = group_maxima<DT>(w, g0, g1);
+    im = fmaxf(g0, g1);
+    raise_ref(im);
+    if (!BF) add_sum(chunks_expsum<DT>(w, a.c, -k_t));  // (bfloat16: with the counting, below)
     // D: how far below the row max the nucleus crossing (top_p = 1: the
     // payload's end) can lie.  Rows of this call that have finished published
     // their depths (in bins of T/4 below their max); the HINT_Q quantile of
@@ -637,68 +628,97 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             b = b > thb0 ? b : thb0;
             return b < thb0 + HW ? b : thb0 + HW;
         };
-        // (the counts' shared-memory address, offset so that a value's bit
-        // pattern times 4 indexes its counter)
-        const uint32_t hbase = (uint32_t)__cvta_generic_to_shared(hist) - thb0 * 4u;
-        // counts the ids of chunk u that reach thb (every lane checks every
-        // element: the callers' branches are warp-uniform)
-        auto count_chunk = [&](int u, uint32_t thb) {
-            const uint32_t span = thb0 + HW - thb;
-            const uint32_t wd[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+        // counts the ids of a chunk that reach value thb in the counters of
+        // values thb0 ... (no id of it lies above the window)
+        auto count_chunk = [&](const uint4 &ch, uint32_t thb) {
+            const uint32_t wd[4] = {ch.x, ch.y, ch.z, ch.w};
+            // (the counts' shared-memory address, offset so that a value's
+            // float bits >> 14, its bfloat16 pattern times 4, index its counter)
+            const int hbase = (int)__cvta_generic_to_shared(hist) - (int)thb0 * 4;
+            const int dummy = hbase + (int)thb * 4 - 4 - 4 * lane;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t lo = wd[q] & 0xFFFFu, hi = wd[q] >> 16;
+            for (int e = 0; e < EPC; ++e) {
+                const int v = (int)((e & 1) ? wd[e >> 1] & 0xFFFF0000u : wd[e >> 1] << 16);
+                const int at = max((v >> 14) + hbase, dummy);
 #ifdef ACES_CHECKED
-                if (lo - thb < span && ACES_IN(lo - thb0, HW)) atomicAdd(&hist[lo - thb0], 1u);
-                if (hi - thb < span && ACES_IN(hi - thb0, HW)) atomicAdd(&hist[hi - thb0], 1u);
+                if (ACES_IN((at - hbase) / 4 - (int)thb0 + HPAD, HPAD + HW)) red_inc(at);
 #else
-                red_inc_lt(hbase + lo * 4u, lo - thb, span);
-                red_inc_lt(hbase + hi * 4u, hi - thb, span);
+                red_inc(at);
 #endif
             }
         };
+        const uint32_t topp = (thb0 + HW) | (thb0 + HW) << 16;  // the value above the window (at most +inf)
+        const __nv_bfloat162 top2 = *reinterpret_cast<const __nv_bfloat162 *>(&topp);
         const int gpi = a.sk_gpi, ish = a.sk_ish;
-        uint32_t gacc = 0u;
+        float gacc = -INFINITY;
+        // the sketch holds bfloat16 bit patterns (as signed 16-bit integers
+        // those of positive values sort like the values, above all others)
         auto sketch_put = [&](int it) {
-            const uint32_t k0 = key16(__float_as_uint(g0) >> 16), k1 = key16(__float_as_uint(g1) >> 16);
             if (gpi == 2) {
                 const int s2 = it * NTC + tid;
-                if (ACES_IN(2 * s2 + 1, SKG)) reinterpret_cast<uint32_t *>(sk)[s2] = k0 | (k1 << 16);
+                if (ACES_IN(2 * s2 + 1, SKG))
+                    reinterpret_cast<uint32_t *>(sk)[s2] = __byte_perm(__float_as_uint(g0), __float_as_uint(g1), 0x7632);
             } else {
-                gacc = max(gacc, max(k0, k1));
+                gacc = fmaxf(gacc, fmaxf(g0, g1));
                 if (((it + 1) & ((1 << ish) - 1)) == 0 || it == nit - 1) {
                     const int s1 = (it >> ish) * NTC + tid;
-                    if (ACES_IN(s1, SKG)) sk[s1] = (uint16_t)gacc;
-                    gacc = 0u;
+                    if (ACES_IN(s1, SKG)) sk[s1] = (uint16_t)(__float_as_uint(gacc) >> 16);
+                    gacc = -INFINITY;
                 }
             }
         };
-        {
-            uint32_t thb = count_on ? lim_of(m1) : 0u;
-            float thf = count_on ? __uint_as_float(thb << 16) : INFINITY;
-            uint32_t hb = mask_of(thf);  // (iteration 0 is loaded and summed)
+        // The counting loop is bound by issue slots: 14.3 warp instructions
+        // per 32 logits on flat rows (whole kernel, ncu; 20.5 with a predicated
+        // reduction, maxima per chunk and a divided tile order), 224 us against
+        // 282 us for the call on 128 x 17 rows of 128256.  Without counting it
+        // is 7.2 (8.7): there HBM and the row's other phases bound it, and
+        // fewer instructions still (or L2 prefetches of the next iterations or
+        // of the row one wave on) change nothing.
+        auto stream = [&](auto counting) {
+            constexpr bool COUNT = decltype(counting)::value;
             for (int it = 0; it < nit; ++it) {
-                if (it > 0) {
-                    tile0 += a.pstride_it;
-                    if (tile0 >= ntile) tile0 -= ntile;
+                uint32_t thb = 0u;
+                if (it > 0) {  // (iteration 0 is loaded, its maxima known)
+                    off0 = wrap(off0 + off_it);
                     load(it);
-                    if (count_on) {
-                        thb = lim_of(running_max());
-                        thf = __uint_as_float(thb << 16);
-                    }
-                    hb = math(thf, im, g0, g1);
-                    publish_max(im);
                 }
-                if (count_on) {
-                    // chunk positions where some lane of the warp reaches thb
-                    const uint32_t any = __reduce_or_sync(0xffffffffu, hb);
+                if (COUNT) thb = lim_of(running_max());
+                if (it > 0) {
+                    im2 = group_maxima<DT>(w, g0, g1);
+                    im = fmaxf(g0, g1);
+                    raise_ref(im);
+                    if (COUNT) publish_max(im);
+                }
+                uint32_t any = 0u;  // chunk positions where some lane of the warp reaches thb
+                if (COUNT) {
+                    uint32_t hb = 0u;
+                    const uint32_t thp = thb | thb << 16;
+                    const __nv_bfloat162 t2 = *reinterpret_cast<const __nv_bfloat162 *>(&thp);
 #pragma unroll
-                    for (int u = 0; u < UC; ++u)
-                        if ((any >> u) & 1u) count_chunk(u, thb);
+                    for (int u = 0; u < UC; ++u) {
+                        const uint32_t cm = chunk_max2<DT>(w[u]);
+                        hb |= (uint32_t)(__hge2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&cm), t2) != 0u) << u;
+                    }
+                    // a value above the window (the row is counted again) or a
+                    // NaN (it is not a distribution): this iteration need not
+                    // be counted, nor may it be
+                    if (__hlt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&im2), top2) != 0xFFFFFFFFu) hb |= 1u << UC;
+                    any = __reduce_or_sync(0xffffffffu, hb);
+                    if (any >> UC) any = 0u;
                 }
+                const unsigned long long c2 = pack2(a.c, a.c), nk2 = pack2(-k_t, -k_t);
+                unsigned long long acc0 = 0ull, acc1 = 0ull;
+#pragma unroll
+                for (int u = 0; u < UC; ++u) {
+                    if (COUNT && ((any >> u) & 1u)) count_chunk(w[u], thb);  // (warp-uniform)
+                    acc_pair(u, chunk_expsum2<DT>(w[u], c2, nk2), acc0, acc1);
+                }
+                add_sum(acc_total(acc0, acc1));
                 sketch_put(it);
             }
-        }
+        };
+        if (count_on) stream(std::true_type());
+        else stream(std::false_type());
         if (finish_sums()) return;
         const uint32_t km = __float_as_uint(m) >> 16;
         if (a.force_fb || !(m > 0.0f)) {
@@ -865,16 +885,16 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             if (lane == 31 && inc > 0) base = atomicAdd(ctr, inc);
             return __shfl_sync(0xffffffffu, base, 31) + inc - cnt;
         };
-        // lists in gl the slots whose group max (16-bit order key) reaches
-        // key; returns their count (all threads)
-        auto compact = [&](uint32_t key, uint32_t *gl) -> int {
+        // lists in gl the slots whose group max reaches the positive value of
+        // bit pattern vb; returns their count (all threads)
+        auto compact = [&](uint32_t vb, uint32_t *gl) -> int {
             if (tid == 0) s_ng = 0;
             __syncthreads();
             const int per_t = ng_all / NTC;  // (at most 64: slot i * NTC + tid)
             unsigned long long hm = 0ull;
             for (int i = 0; i < per_t; ++i) {
                 const int slot = i * NTC + tid;
-                if (ACES_IN(slot, SKG) && sk[slot] >= key) hm |= 1ull << i;
+                if (ACES_IN(slot, SKG) && (int)(int16_t)sk[slot] >= (int)vb) hm |= 1ull << i;
             }
             int at = warp_place(__popcll(hm), &s_ng);
             __syncthreads();  // (gl may overlap slots of the sketch read above)
@@ -957,7 +977,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
                 thb0 = lb > kfull ? lb : kfull;
             }
             uint32_t *gls = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(sk) + SK_TMP);
-            const int nc = compact(0x8000u + thb0, gls);  // (ends with a barrier)
+            const int nc = compact(thb0, gls);  // (ends with a barrier)
             if (nc > GCAP) return 1;
             if (tid == 0) s_npay = 0;
             __syncthreads();
@@ -1007,7 +1027,6 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             thb0 = km > (uint32_t)(HW - 1) ? km - (uint32_t)(HW - 1) : 1u;
             for (int i = tid; i < HW; i += NTC) hist[i] = 0u;
             __syncthreads();
-            const uint32_t span = km + 1u - thb0;
             for (int c0 = 0; c0 < nch; c0 += NTC * UC) {
 #pragma unroll
                 for (int u = 0; u < UC; ++u) {
@@ -1015,15 +1034,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
                     w[u] = c < nch ? ldg16(row + (size_t)c * 16) : make_uint4(NI, NI, NI, NI);
                 }
 #pragma unroll
-                for (int u = 0; u < UC; ++u) {
-                    const uint32_t wd[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint32_t lo = (wd[q] & 0xFFFFu) - thb0, hi = (wd[q] >> 16) - thb0;
-                        if (lo < span && ACES_IN(lo, HW)) atomicAdd(&hist[lo], 1u);
-                        if (hi < span && ACES_IN(hi, HW)) atomicAdd(&hist[hi], 1u);
-                    }
-                }
+                for (int u = 0; u < UC; ++u) count_chunk(w[u], thb0);
             }
             __syncthreads();
             if (tid == 0) atomicAdd(&a.ws.fb_count[10], 1);
@@ -1041,7 +1052,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             // ---- the ids at or above value vr, then ordered ----
             const uint32_t vrb = thb0 + (uint32_t)vr;  // its bit pattern
             if (!pay_ready) {
-                const int ng = compact(0x8000u + vrb, glist);
+                const int ng = compact(vrb, glist);
                 if (ng > GCAP) {
                     if (tid == 0) fallback_row(a, r, m, kref, S);
                     return;
@@ -1201,12 +1212,12 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
         // records the chunks in hb (those holding an id >= the capture
         // threshold): one vote per iteration, one warp-aggregated atomic per
         // chunk position that has any; the ids are extracted after the stream
-        auto record_hits = [&](uint32_t hb) {
-            if (!__any_sync(0xffffffffu, hb != 0u)) return;
-            int tile = tile0;
+        auto record_hits = [&](float th) {
+            if (!__any_sync(0xffffffffu, im >= th)) return;
+            uint32_t off = off0;
 #pragma unroll
             for (int u = 0; u < UC; ++u) {
-                const bool hit = (hb >> u) & 1u;
+                const bool hit = max2_value<DT>(chunk_max2<DT>(w[u])) >= th;
                 const unsigned bal = __ballot_sync(0xffffffffu, hit);
                 if (bal != 0u) {
                     const int lead = __ffs(bal) - 1;
@@ -1217,27 +1228,27 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
                         const int at = base + __popc(bal & ((1u << lane) - 1u));
                         if (at < CREC && ACES_IN(at, CREC)) {
                             rec_dat[at] = w[u];
-                            rec_idx[at] = (uint32_t)(tile * TCH + lane);
+                            rec_idx[at] = off >> 4;
                         }
                     }
                 }
-                tile += a.pstride_w;
-                if (tile >= ntile) tile -= ntile;
+                off = wrap(off + off_w);
             }
         };
         {
             float th = hinted ? m1 - D : thlo;
-            uint32_t hb = mask_of(th);  // (iteration 0 is loaded and summed)
             for (int it = 0; it < nit; ++it) {
-                if (it > 0) {
-                    tile0 += a.pstride_it;
-                    if (tile0 >= ntile) tile0 -= ntile;
+                if (it > 0) {  // (iteration 0 is loaded and summed)
+                    off0 = wrap(off0 + off_it);
                     load(it);
                     if (hinted) th = running_max() - D;
-                    hb = math(th, im, g0, g1);
+                    group_maxima<DT>(w, g0, g1);
+                    im = fmaxf(g0, g1);
+                    raise_ref(im);
+                    add_sum(chunks_expsum<DT>(w, a.c, -k_t));
                     if (hinted) publish_max(im);
                 }
-                record_hits(hb);
+                record_hits(th);
             }
         }
         if (finish_sums()) return;
