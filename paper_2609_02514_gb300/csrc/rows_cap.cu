@@ -33,7 +33,7 @@
 //             values: a second counting pass over the row; a capacity
 //             exceeded: the exact general kernel):
 //             bfloat16  (sketch-led: the groups reaching row max - D are read
-//                       back and their ids counted first) one warp scans the
+//                       back and their ids counted first) the CTA scans the
 //                       value counts for the crossing value, the number j of
 //                       its ids inside the nucleus and the payload's last
 //                       value; the sketch's groups whose max reaches that
@@ -64,11 +64,9 @@
 
 namespace aces {
 
-constexpr int NTC = 256;            // threads per CTA
-constexpr int NWC = NTC / 32;
 constexpr int UC = 8;               // 16-byte chunks per thread and iteration
 constexpr int TCH = 32;             // chunks per tile
-constexpr int TPI = NWC * UC;       // tiles per iteration
+constexpr int SAMPLE = 64;          // tiles of the sample: the first of the row's order
 constexpr int NSB = 40;             // depth bins (of T/SPB) of the hints; D before any hint
 constexpr int SPB = 4;              // depth bins per temperature
 constexpr int MARGIN_BINS = 2;      // float32 first rows: theta below the sample's crossing
@@ -92,11 +90,10 @@ constexpr int SMEM_BF = (HPAD + HW) * 4 + SKG * 2 + PCAP * 8;
 // crossing (top_p = 1: when k <= SHORT_IDS); later rows take the pass when
 // at least SHORT_NUM / SHORT_DEN of the finished rows were short.  Its areas
 // inside the sketch's (in 8-byte units): the ordered ids [0, 1024), the
-// groups read back, then the kept ids [2048, 3072), the per-value masses
-// [3072, 4096)
+// groups read back, then the kept ids [2048, 3072)
 constexpr int SHORT_IDS = 256;
 constexpr int SHORT_NUM = 49, SHORT_DEN = 50;
-constexpr int SK_TMP = 2048, SK_EMASS = 3072;
+constexpr int SK_TMP = 2048;
 // float32
 constexpr int CREC = 1536;          // recorded chunks (16-byte chunk + its index) per row
 constexpr int LCAP = 2048;          // listed ids, expanded from the records after the stream
@@ -116,9 +113,8 @@ struct F32Caps {
 constexpr int RANK_MAX = 512;       // ids ordered by direct ranking (more: bitonic sort)
 static_assert(WS_DEPTH + NSB <= WS_COUNTERS / 4, "the depth histogram fits the counters area");
 static_assert(4 * NUC_CAP * 8 <= SMEM_BF && 4 * NUC_CAP * 8 <= SMEM_F32, "the draw's scratch fits");
-static_assert(GCAP * 4 <= HW * 4 && PCAP * 8 <= SKG * 2 && HW <= PCAP, "the aliased areas fit");
-static_assert(PCAP <= SK_TMP && GCAP * 4 <= (SK_EMASS - SK_TMP) * 8 && PCAP <= SK_EMASS - SK_TMP &&
-                  SK_EMASS + HW <= SKG / 4, "the sketch-led areas fit");
+static_assert(GCAP * 4 <= HW * 4 && PCAP * 8 <= SKG * 2 && "the aliased areas fit");
+static_assert(PCAP <= SK_TMP && SK_TMP + GCAP / 2 <= SKG / 4 && SK_TMP + PCAP <= SKG / 4, "the sketch-led areas fit");
 static_assert(WCAP * 8 <= CREC * 20 && RANK_MAX * 2 <= LCAP, "the float32 work areas fit");
 static_assert(F32Caps<2>::WC * 8 <= F32Caps<2>::CR * 20 && RANK_MAX * 2 <= F32Caps<2>::LC &&
                   2 * (F32Caps<2>::SMEM + 1024) <= 228 * 1024,
@@ -228,12 +224,13 @@ __device__ __forceinline__ float acc_total(unsigned long long acc0, unsigned lon
 }
 
 // sum over the chunks of 2^(z*c - k), two logits per instruction
-template <int DT>
+// (chunks U0 <= j < U1)
+template <int DT, int U0, int U1>
 __device__ __forceinline__ float chunks_expsum(const uint4 (&w)[UC], float c, float nk) {
     const unsigned long long c2 = pack2(c, c), nk2 = pack2(nk, nk);
     unsigned long long acc0 = 0ull, acc1 = 0ull;
 #pragma unroll
-    for (int j = 0; j < UC; ++j) acc_pair(j, chunk_expsum2<DT>(w[j], c2, nk2), acc0, acc1);
+    for (int j = U0; j < U1; ++j) acc_pair(j - U0, chunk_expsum2<DT>(w[j], c2, nk2), acc0, acc1);
     return acc_total(acc0, acc1);
 }
 
@@ -286,10 +283,11 @@ __device__ __forceinline__ float val16(uint32_t k) {
 // The CTA that finishes the last row of a sequence (rows handed to the
 // general kernel are never counted) draws the sequence's token from the
 // stored nucleus, so most sequences need no separate resolve launch.
+template <int NTC>
 __device__ void row_finished(const RowArgs &a, int r, unsigned char *scratch) {
     if (a.ws.seqcnt == nullptr) return;  // sparsify
     __shared__ int s_last;
-    __shared__ unsigned long long s_red[NWC];
+    __shared__ unsigned long long s_red[NTC / 32];
     __shared__ DrawShared s_draw;
     const int b = r / (a.K + 1);
     __syncthreads();  // every thread's writes of this row are issued
@@ -337,8 +335,13 @@ __device__ __forceinline__ unsigned long long id_fx(float v, float c, float kref
     return to_fx(ex2(fmaf(v, c, -kref)));
 }
 
-template <int DT, int W>
-__global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
+// NTC: threads per CTA, 1024 / NTC CTAs per SM
+template <int DT, int W, int NTC>
+__global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
+    constexpr int NWC = NTC / 32;
+    constexpr int TPI = NWC * UC;         // tiles per iteration
+    constexpr int UCS = SAMPLE / NWC;     // this thread's chunks of iteration 0 that are in the sample
+    static_assert(UCS >= 1 && UCS <= UC && HW % NTC == 0, "the sample lies in iteration 0");
     constexpr int CREC = F32Caps<W>::CR, LCAP = F32Caps<W>::LC, WCAP = F32Caps<W>::WC;
     constexpr int MARGIN_BINS = F32Caps<W>::MARGIN;
     using E = Elem<DT>;
@@ -363,19 +366,20 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
 
     __shared__ uint32_t sbin[NWC][NSB];  // float32 estimate: per warp, below the sample max
     __shared__ float redf[NWC], redk[NWC], redh[NWC], redl[NWC];
-    __shared__ int s_nrec, s_nl, s_fb, s_n, s_bsel, s_nstar, s_L, s_npay, s_ng, s_nge, s_j, s_vs, s_vk, s_nnuc;
+    __shared__ int s_nrec, s_nl, s_fb, s_n, s_bsel, s_nstar, s_L, s_npay, s_ng, s_nge, s_j, s_vs, s_vk;
     __shared__ float s_thlo, s_zx;
     __shared__ int s_dbins, s_xb;  // s_dbins: D in depth bins (-1: no hints yet)
     __shared__ int s_skm;          // bfloat16: the sketch-led pass (no counting while streaming)
     __shared__ uint32_t s_mr;  // order key of the running max
     __shared__ double s_Snuc;
     __shared__ float s_inv_S;
-    __shared__ unsigned long long s_cut, s_cumL_fx;
-    __shared__ unsigned long long s_redu[NWC];
+    __shared__ unsigned long long s_cut, s_cumL_fx, s_tg;
+    __shared__ unsigned long long s_redu[NWC], s_above, s_evs;
+    __shared__ uint32_t s_redc[NWC], s_cab, s_cnvs;
 
     const int r = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (a.stagger_ns > 0 && r < 4 * a.nsm) {
+    if (NTC == 256 && a.stagger_ns > 0 && r < 4 * a.nsm) {
         // the j-th CTA an SM starts with (blocks are placed on the SMs in
         // turn) waits j times stagger_ns on the global timer (bounded: at
         // most 3 x stagger_ns)
@@ -487,13 +491,20 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
     };
     auto running_max = [&]() -> float { return fkey_inv(*reinterpret_cast<volatile uint32_t *>(&s_mr)); };
 
-    // iteration 0: a strided sample (1/8 to 1/16 of a large row, spread over it)
+    // iteration 0 begins with a strided sample (1/8 to 1/16 of a large row,
+    // spread over it): chunks u < UCS
     float im, g0, g1;
     load(0);
-    uint32_t im2 = group_maxima<DT>(w, g0, g1);
-    im = fmaxf(g0, g1);
-    raise_ref(im);
-    if (!BF) add_sum(chunks_expsum<DT>(w, a.c, -k_t));  // (bfloat16: with the counting, below)
+    {
+        uint32_t sm2 = chunk_max2<DT>(w[0]);
+#pragma unroll
+        for (int u = 1; u < UCS; ++u) sm2 = max2<DT>(sm2, chunk_max2<DT>(w[u]));
+        im = max2_value<DT>(sm2);
+    }
+    if (!BF) {  // (bfloat16: with the other iterations, below)
+        raise_ref(im);
+        add_sum(chunks_expsum<DT, 0, UCS>(w, a.c, -k_t));
+    }
     // D: how far below the row max the nucleus crossing (top_p = 1: the
     // payload's end) can lie.  Rows of this call that have finished published
     // their depths (in bins of T/4 below their max); the HINT_Q quantile of
@@ -531,12 +542,14 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
     int lazy = 0;
     int nnuc = -1;  // nucleus ids written to the row's list (-1: none)
     float m = -INFINITY, kref = -1e30f;
-    double S = 0.0;
+    double S = 0.0;  // (thread 0)
     float v_need = 0.0f;  // the crossing (top_p = 1: the payload's end), for the hints
     bool short_row = false;  // (bfloat16) few ids reach the crossing: published for later rows' pass
 
-    // reduces the row max, the reference and the exp-sum (fp32 two-sum tree,
-    // fp64 in warp 0); true when the row is not a distribution (handled)
+    // reduces the row max, the reference and the exp-sum S (fp32 two-sum tree,
+    // fp64 in thread 0 only, which also leaves the nucleus target in s_tg:
+    // valid after the next barrier); true when the row is not a distribution
+    // (handled)
     auto finish_sums = [&]() -> bool {
         if (a.K > 0) {
             bq = r / (a.K + 1);
@@ -571,28 +584,47 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
         }
         __syncthreads();
         // every thread combines the warps' parts (fp64, exact rescales)
-        m = redf[0];
-        kref = redk[0];
-#pragma unroll
-        for (int i = 1; i < NWC; ++i) {
-            m = fmaxf(m, redf[i]);
-            kref = fmaxf(kref, redk[i]);
-        }
         // (fp32 two-sums over exact power-of-two rescales: fp64 is slow here)
         float sh = 0.0f, sl = 0.0f;
+        if constexpr (NWC <= 8) {
+            m = redf[0];
+            kref = redk[0];
 #pragma unroll
-        for (int i = 0; i < NWC; ++i) {
-            const float f = pow2_int(fmaxf(redk[i] - kref, -1000.0f));  // (an integer <= 0)
-            float sm, er;
-            two_sum(sh, redh[i] * f, sm, er);
-            sl += er + redl[i] * f;
-            sh = sm;
+            for (int i = 1; i < NWC; ++i) {
+                m = fmaxf(m, redf[i]);
+                kref = fmaxf(kref, redk[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < NWC; ++i) {
+                const float f = pow2_int(fmaxf(redk[i] - kref, -1000.0f));  // (an integer <= 0)
+                float sm, er;
+                two_sum(sh, redh[i] * f, sm, er);
+                sl += er + redl[i] * f;
+                sh = sm;
+            }
+        } else {  // one warp's part per lane, the same tree in every warp
+            const int i = lane % NWC;
+            m = warp_max(redf[i]);
+            kref = warp_max(redk[i]);
+            const float f = pow2_int(fmaxf(redk[i] - kref, -1000.0f));
+            sh = redh[i] * f;
+            sl = redl[i] * f;
+            for (int o = NWC / 2; o > 0; o >>= 1) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, sh, o);
+                const float l2 = __shfl_xor_sync(0xffffffffu, sl, o);
+                float sm, er;
+                two_sum(sh, h2, sm, er);
+                sl = sl + l2 + er;
+                sh = sm;
+            }
         }
-        const double Sa = (double)sh + (double)sl;
-        S = Sa;
-        if (!(S > 0.0 && S < 1e300) || !(m < INFINITY) || !(kref < 1e30f)) {
+        if (tid == 0) {
+            S = (double)sh + (double)sl;
+            s_tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
+        }
+        if (!(sh > 0.0f && sh < INFINITY) || !(m < INFINITY) || !(kref < 1e30f)) {
             nonfinite_row<NTC>(a, r);
-            row_finished(a, r, smem);
+            row_finished<NTC>(a, r, smem);
             return true;
         }
         return false;
@@ -678,17 +710,15 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             constexpr bool COUNT = decltype(counting)::value;
             for (int it = 0; it < nit; ++it) {
                 uint32_t thb = 0u;
-                if (it > 0) {  // (iteration 0 is loaded, its maxima known)
+                if (it > 0) {  // (iteration 0 is loaded)
                     off0 = wrap(off0 + off_it);
                     load(it);
                 }
                 if (COUNT) thb = lim_of(running_max());
-                if (it > 0) {
-                    im2 = group_maxima<DT>(w, g0, g1);
-                    im = fmaxf(g0, g1);
-                    raise_ref(im);
-                    if (COUNT) publish_max(im);
-                }
+                const uint32_t im2 = group_maxima<DT>(w, g0, g1);
+                im = fmaxf(g0, g1);
+                raise_ref(im);
+                if (COUNT) publish_max(im);
                 uint32_t any = 0u;  // chunk positions where some lane of the warp reaches thb
                 if (COUNT) {
                     uint32_t hb = 0u;
@@ -726,150 +756,126 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             return;
         }
         auto vmass = [&](int idx) { return id_fx(val16(0x8000u + thb0 + (uint32_t)idx), a.c, kref); };
-        unsigned long long *emass = pay;  // (until the re-read) the mass of one id of each counted value
         // ---- the crossing, the payload's end and the values to re-read,
-        // from the counts of values thc..m (warp 0).  Returns 0, or 1 when
-        // they lie below the counted values, 2 when more ids than the
-        // re-read keeps share the payload's last value ----
+        // from the counts of values thc..m (all threads, VPT consecutive
+        // values each, from the top).  Returns 0, or 1 when they lie below
+        // the counted values, 2 when more ids than the re-read keeps share
+        // the payload's last value ----
+        // (L, vs, vr, j, n_nuc and nge are set when it returns 0)
+        int vs = -1, vr = -1, j = 0, n_nuc = -1, nge = 0;
         auto scan = [&](uint32_t thc) -> int {
-            if (wid == 0) {
-                const unsigned long long tg =
-                    all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
-                const int top = (int)(km - thb0), lo = (int)(thc - thb0);
-                const int per = (top - lo + 32) >> 5;
-                const int b0 = top - lane * per;  // this lane's values: b0, b0 - 1, ... (>= lo)
-                unsigned long long lm = 0ull, lc = 0ull;
-                for (int i = 0; i < per; ++i) {
-                    const int idx = b0 - i;
-                    if (idx < lo) break;
-                    const uint32_t cn = hist[idx];
-                    if (cn) {
-                        const unsigned long long e1 = vmass(idx);
-                        if (ACES_IN(idx, PCAP)) emass[idx] = e1;
-                        lm += (unsigned long long)cn * e1;
-                        lc += cn;
-                    }
+            constexpr int VPT = HW / NTC;
+            const int top = (int)(km - thb0) - VPT * tid, lo = (int)(thc - thb0);
+            uint32_t cn[VPT];
+            unsigned long long e1[VPT], lm = 0ull;
+            uint32_t lc = 0u;
+#pragma unroll
+            for (int i = 0; i < VPT; ++i) {
+                cn[i] = top - i >= lo ? hist[top - i] : 0u;
+                e1[i] = cn[i] ? vmass(top - i) : 0ull;
+                lm += (unsigned long long)cn[i] * e1[i];
+                lc += cn[i];
+            }
+            unsigned long long incm = lm;
+            uint32_t incc = lc;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long tm = __shfl_up_sync(0xffffffffu, incm, o);
+                const uint32_t tc = __shfl_up_sync(0xffffffffu, incc, o);
+                if (lane >= o) {
+                    incm += tm;
+                    incc += tc;
                 }
-                unsigned long long incm = lm, incc = lc;
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long tm = __shfl_up_sync(0xffffffffu, incm, o);
-                    const unsigned long long tc = __shfl_up_sync(0xffffffffu, incc, o);
-                    if (lane >= o) {
-                        incm += tm;
-                        incc += tc;
-                    }
+            }
+            if (lane == 31) {
+                s_redu[wid] = incm;
+                s_redc[wid] = incc;
+            }
+            if (tid == 0) {
+                s_vs = -1;
+                s_j = 0;
+                s_cab = s_cnvs = 0u;
+                s_above = s_evs = 0ull;
+            }
+            __syncthreads();
+            uint32_t totc = 0u;
+#pragma unroll
+            for (int i = 0; i < NWC; ++i) {
+                if (i < wid) {
+                    incm += s_redu[i];
+                    incc += s_redc[i];
                 }
-                const unsigned long long exm = incm - lm, exc = incc - lc;
-                const unsigned long long totc = __shfl_sync(0xffffffffu, incc, 31);
-                int fail = 0, vs = -1, jj = 0;
-                unsigned long long above = 0ull, cab = 0ull, cnvs = 0ull;
-                if (!all_in) {
-                    if (exm < tg && incm >= tg) {
-                        unsigned long long cm = exm, cc = exc;
-                        for (int i = 0; i < per; ++i) {
-                            const int idx = b0 - i;
-                            if (idx < lo) break;
-                            const uint32_t cn = hist[idx];
-                            if (!cn) continue;
-                            const unsigned long long e1 = emass[idx];
-                            const unsigned long long mm = (unsigned long long)cn * e1;
-                            if (cm + mm >= tg) {
-                                vs = idx;
-                                above = cm;
-                                cab = cc;
-                                cnvs = cn;
-                                // the fewest ids of this value reaching the target
-                                const unsigned long long rem = tg - cm;
-                                unsigned long long q = (unsigned long long)((float)rem / (float)e1);
-                                while (q * e1 < rem) ++q;
-                                while (q > 1ull && (q - 1ull) * e1 >= rem) --q;
-                                jj = (int)q;
-                                break;
-                            }
-                            cm += mm;
-                            cc += cn;
-                        }
+                totc += s_redc[i];
+            }
+            const unsigned long long exm = incm - lm, tg = s_tg;
+            const uint32_t exc = incc - lc;
+            if (!all_in && exm < tg && incm >= tg) {  // (at most one thread)
+                unsigned long long cm = exm;
+                uint32_t cc = exc;
+#pragma unroll
+                for (int i = 0; i < VPT; ++i) {
+                    const unsigned long long mm = (unsigned long long)cn[i] * e1[i];
+                    if (cm < tg && cm + mm >= tg) {
+                        s_vs = top - i;
+                        s_above = cm;
+                        s_cab = cc;
+                        s_cnvs = cn[i];
+                        s_evs = e1[i];
+                        // the fewest ids of this value reaching the target
+                        const unsigned long long rem = tg - cm;
+                        unsigned long long q = (unsigned long long)((float)rem / (float)e1[i]);
+                        while (q * e1[i] < rem) ++q;
+                        while (q > 1ull && (q - 1ull) * e1[i] >= rem) --q;
+                        s_j = (int)q;
                     }
-                    const unsigned bal = __ballot_sync(0xffffffffu, vs >= 0);
-                    if (bal) {
-                        const int src = __ffs(bal) - 1;
-                        vs = __shfl_sync(0xffffffffu, vs, src);
-                        jj = __shfl_sync(0xffffffffu, jj, src);
-                        above = __shfl_sync(0xffffffffu, above, src);
-                        cab = __shfl_sync(0xffffffffu, cab, src);
-                        cnvs = __shfl_sync(0xffffffffu, cnvs, src);
-                    } else {
-                        fail = 1;
-                    }
+                    cm += mm;
+                    cc += cn[i];
                 }
-                const unsigned long long nn = all_in ? (unsigned long long)a.V : cab + (unsigned long long)jj;
-                const int Lw = fail ? 0 : (int)(nn < (unsigned long long)a.k ? nn : (unsigned long long)a.k);
-                if (!fail && (unsigned long long)Lw > totc) fail = 1;  // (top_p = 1) the payload reaches below them
-                int vk = -1;
-                unsigned long long cabk = 0ull, mabk = 0ull, cnk = 0ull;
-                if (!fail && Lw > 0) {
-                    const unsigned long long Lu = (unsigned long long)Lw;
-                    if (exc < Lu && incc >= Lu) {
-                        unsigned long long cm = exm, cc = exc;
-                        for (int i = 0; i < per; ++i) {
-                            const int idx = b0 - i;
-                            if (idx < lo) break;
-                            const uint32_t cn = hist[idx];
-                            if (!cn) continue;
-                            if (cc + cn >= Lu) {
-                                vk = idx;
-                                cabk = cc;
-                                mabk = cm;
-                                cnk = cn;
-                                break;
-                            }
-                            cc += cn;
-                            cm += (unsigned long long)cn * emass[idx];
-                        }
+            }
+            const uint32_t ku = (uint32_t)a.k;
+            if (exc < ku && incc >= ku) {  // the value of the k-th id (one thread)
+                unsigned long long cm = exm;
+                uint32_t cc = exc;
+#pragma unroll
+                for (int i = 0; i < VPT; ++i) {
+                    if (cc < ku && cc + cn[i] >= ku) {
+                        s_vk = top - i;
+                        s_nge = (int)(cc + cn[i]);
+                        s_cumL_fx = cm + (unsigned long long)(ku - cc) * e1[i];
                     }
-                    const unsigned bal = __ballot_sync(0xffffffffu, vk >= 0);
-                    const int src = bal ? __ffs(bal) - 1 : 0;
-                    vk = __shfl_sync(0xffffffffu, vk, src);
-                    cabk = __shfl_sync(0xffffffffu, cabk, src);
-                    mabk = __shfl_sync(0xffffffffu, mabk, src);
-                    cnk = __shfl_sync(0xffffffffu, cnk, src);
-                    if (vk < 0) fail = 1;
-                }
-                // the values to re-read: down to the crossing value when the
-                // nucleus is short (then it is kept and the cut is exact),
-                // else down to the payload's last value
-                int vr = -1;
-                unsigned long long nge = 0ull;
-                if (!fail) {
-                    if (!all_in && cab + cnvs <= (unsigned long long)PCAP && nn <= (unsigned long long)NUC_CAP) {
-                        vr = vs;
-                        nge = cab + cnvs;
-                    } else if (Lw > 0) {
-                        vr = vk;
-                        nge = cabk + cnk;
-                        if (nge > (unsigned long long)PCAP) fail = 2;
-                    }
-                }
-                if (lane == 0) {
-                    s_fb = fail;
-                    s_vs = vs;
-                    s_vk = vr;
-                    s_j = jj;
-                    s_L = Lw;
-                    s_nnuc = all_in ? -1 : (int)(nn < (unsigned long long)INT_MAX ? nn : (unsigned long long)INT_MAX);
-                    s_nge = (int)nge;
-                    s_ng = 0;
-                    s_npay = 0;
-                    if (!fail) {
-                        const unsigned long long ek = vk >= 0 ? emass[vk] : 0ull;
-                        s_cumL_fx = mabk + ((unsigned long long)Lw - cabk) * ek;
-                        s_Snuc = all_in ? S : (double)(above + (unsigned long long)jj * emass[vs]) * FX_INV;
-                        s_inv_S = inv_mass(s_Snuc);
-                    }
+                    cm += (unsigned long long)cn[i] * e1[i];
+                    cc += cn[i];
                 }
             }
             __syncthreads();
-            return s_fb;
+            // (the same in every thread)
+            vs = s_vs;
+            j = s_j;
+            if (!all_in && vs < 0) return 1;
+            const uint32_t nn = all_in ? (uint32_t)a.V : s_cab + (uint32_t)j;  // (at most V)
+            const unsigned long long nuc = s_above + (unsigned long long)j * s_evs;
+            n_nuc = all_in ? -1 : (int)nn;
+            L = min((int)nn, a.k);
+            if ((uint32_t)L > totc) return 1;  // (top_p = 1) the payload reaches below them
+            // the values to re-read: down to the crossing value when the
+            // nucleus is short (then it is kept and the cut is exact), else
+            // down to the payload's last value
+            vr = -1;
+            if (!all_in && s_cab + s_cnvs <= (uint32_t)PCAP && nn <= (uint32_t)NUC_CAP) {
+                vr = vs;
+                nge = (int)(s_cab + s_cnvs);
+            } else if (L > 0) {
+                const bool at_k = nn > ku;  // else the payload ends with the nucleus
+                vr = at_k ? s_vk : vs;
+                nge = at_k ? s_nge : (int)(s_cab + s_cnvs);
+                if (nge > PCAP) return 2;
+            }
+            if (tid == 0) {  // (read after later barriers)
+                if (nn <= ku) s_cumL_fx = nuc;
+                if (ku == 0u) s_cumL_fx = 0ull;
+                s_Snuc = all_in ? S : (double)nuc * FX_INV;
+                s_inv_S = inv_mass(s_Snuc);
+            }
+            return 0;
         };
         // ---- reading groups of the sketch back ----
         const int ng_all = gpi == 2 ? nit * NTC * 2 : ((nit + (1 << ish) - 1) >> ish) * NTC;
@@ -890,18 +896,29 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
         auto compact = [&](uint32_t vb, uint32_t *gl) -> int {
             if (tid == 0) s_ng = 0;
             __syncthreads();
-            const int per_t = ng_all / NTC;  // (at most 64: slot i * NTC + tid)
+            // this thread's slots: pairs 2 (i * NTC + tid) + {0, 1}, bits 2 i and
+            // 2 i + 1 (at most 64 slots; without pairs slot i * NTC + tid)
             unsigned long long hm = 0ull;
-            for (int i = 0; i < per_t; ++i) {
-                const int slot = i * NTC + tid;
-                if (ACES_IN(slot, SKG) && (int)(int16_t)sk[slot] >= (int)vb) hm |= 1ull << i;
+            if (gpi == 2) {
+                for (int i = 0; i < nit; ++i) {
+                    const int s2 = i * NTC + tid;
+                    const uint32_t g = ACES_IN(2 * s2 + 1, SKG) ? reinterpret_cast<const uint32_t *>(sk)[s2] : 0u;
+                    if ((int)(g << 16) >= (int)(vb << 16)) hm |= 1ull << (2 * i);
+                    if ((int)g >= (int)(vb << 16)) hm |= 2ull << (2 * i);
+                }
+            } else {
+                for (int i = 0; i < ng_all / NTC; ++i) {
+                    const int slot = i * NTC + tid;
+                    if (ACES_IN(slot, SKG) && (int)(int16_t)sk[slot] >= (int)vb) hm |= 1ull << i;
+                }
             }
             int at = warp_place(__popcll(hm), &s_ng);
             __syncthreads();  // (gl may overlap slots of the sketch read above)
             while (hm) {
                 const int i = __ffsll((long long)hm) - 1;
                 hm &= hm - 1ull;
-                if (at < GCAP && ACES_IN(at, GCAP)) gl[at] = (uint32_t)(i * NTC + tid);
+                const int slot = gpi == 2 ? 2 * ((i >> 1) * NTC + tid) + (i & 1) : i * NTC + tid;
+                if (at < GCAP && ACES_IN(at, GCAP)) gl[at] = (uint32_t)slot;
                 ++at;
             }
             __syncthreads();
@@ -988,22 +1005,22 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             });
             const int nall = s_npay;
             if (nall > PCAP) return 1;
-            emass = reinterpret_cast<unsigned long long *>(sk) + SK_EMASS;
+            if (tid == 0) s_ng = 0;  // (the scan's barriers come before its next use)
             const int f = scan(thb0);
             if (f != 0) return f;
             // keep in pay the ids >= the scan's vr
-            if (s_vk >= 0) {
-                const uint32_t kr = fkey(val16(0x8000u + thb0 + (uint32_t)s_vk));
+            if (vr >= 0) {
+                const uint32_t kr = fkey(val16(0x8000u + thb0 + (uint32_t)vr));
                 unsigned long long *tmp = reinterpret_cast<unsigned long long *>(sk) + SK_TMP;
                 for (int i0 = 0; i0 < nall; i0 += NTC) {  // warp-uniform rounds
                     const int i = i0 + tid;
                     const unsigned long long o = i < nall ? pay[i] : 0ull;
                     const bool keep = i < nall && (uint32_t)(o >> 32) >= kr;
-                    const int at = warp_place(keep ? 1 : 0, &s_npay);
+                    const int at = warp_place(keep ? 1 : 0, &s_ng);
                     if (keep && ACES_IN(at, PCAP)) tmp[at] = o;
                 }
                 __syncthreads();
-                const int nk = s_npay;
+                const int nk = s_ng;
                 for (int i = tid; i < nk; i += NTC)
                     if (ACES_IN(i, PCAP)) pay[i] = tmp[i];
                 __syncthreads();
@@ -1020,7 +1037,6 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             fb = scan(lim_of(m));
         }
         if (fb == 1) {
-            emass = pay;
             // the crossing (or the row max) lies outside the counted values:
             // a second pass counts the row again, from the row max down as far
             // as the window reaches
@@ -1044,8 +1060,6 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             if (tid == 0) fallback_row(a, r, m, kref, S);
             return;
         }
-        L = s_L;
-        const int vs = s_vs, j = s_j, vr = s_vk;
         const uint32_t vsb = thb0 + (uint32_t)vs;  // crossing value (bit pattern)
         const bool exact = !all_in && vr == vs;    // every id of the crossing value is read below
         if (vr >= 0) {
@@ -1057,10 +1071,12 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
                     if (tid == 0) fallback_row(a, r, m, kref, S);
                     return;
                 }
+                if (tid == 0) s_npay = 0;
+                __syncthreads();
                 reread(glist, ng, vrb, &s_npay, put_pay);
             }
-            const int npay = s_npay;
-            if (npay != s_nge) {  // (cannot happen: the counts and the ids agree)
+            const int npay = pay_ready ? s_ng : s_npay;
+            if (npay != nge) {  // (cannot happen: the counts and the ids agree)
                 if (tid == 0) fallback_row(a, r, m, kref, S);
                 return;
             }
@@ -1085,7 +1101,6 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             }
             __syncthreads();
         }
-        const int n_nuc = s_nnuc;
         if (tid == 0) {
             if (all_in) {
                 s_cut = 0ull;
@@ -1146,7 +1161,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
         if (!hinted) {
             if (have) {
 #pragma unroll
-                for (int u = 0; u < UC; ++u) {
+                for (int u = 0; u < UCS; ++u) {
                     const float cmx = max2_value<DT>(chunk_max2<DT>(w[u]));
                     if (!__any_sync(0xffffffffu, (m1 - cmx) * a.inv_ws < (float)NSB)) continue;
 #pragma unroll 1  // (unrolled, the independent atomics spill registers)
@@ -1238,14 +1253,17 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
         {
             float th = hinted ? m1 - D : thlo;
             for (int it = 0; it < nit; ++it) {
-                if (it > 0) {  // (iteration 0 is loaded and summed)
+                if (it > 0) {  // (iteration 0 is loaded, its sample summed)
                     off0 = wrap(off0 + off_it);
                     load(it);
                     if (hinted) th = running_max() - D;
+                }
+                if (it > 0 || UCS < UC) {
                     group_maxima<DT>(w, g0, g1);
                     im = fmaxf(g0, g1);
                     raise_ref(im);
-                    add_sum(chunks_expsum<DT>(w, a.c, -k_t));
+                    if (it > 0) add_sum(chunks_expsum<DT, 0, UC>(w, a.c, -k_t));
+                    else add_sum(chunks_expsum<DT, UCS == UC ? 0 : UCS, UC>(w, a.c, -k_t));
                     if (hinted) publish_max(im);
                 }
                 record_hits(th);
@@ -1279,7 +1297,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             if (tid == 0) fallback_row(a, r, m, kref, S);
             return;
         }
-        const unsigned long long tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
+        const unsigned long long tg = s_tg;
         // counts of the listed ids in bins of T/8 below m; a bin's ids each
         // carry at least its lower edge's mass, so the first bin where that
         // lower bound of the cumulative mass reaches the target holds or
@@ -1320,7 +1338,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
             pm -= lm;
             pc -= lc;
             // 1e-4 covers the fp32 rounding of the bound and of S
-            const float tgf = (float)((double)a.top_p * S) * (1.0f + 1e-4f);
+            const float tgf = (float)tg * (1.0f / FX_SCALE) * (1.0f + 1e-4f);
             int hit = -1;
             unsigned ncand = 0u;
 #pragma unroll
@@ -1485,7 +1503,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
                 s_nstar = nstar;
                 s_L = L;
                 s_cumL_fx = cL;
-                const double sn = all_in ? S : (double)cN * FX_INV;
+                const double sn = all_in ? S : (double)cN * FX_INV;  // (lane 0 of warp 0 is thread 0)
                 s_Snuc = sn;
                 s_inv_S = inv_mass(sn);
                 s_cut = (nstar != INT_MAX && !all_in) ? ord[nstar] : 0ull;
@@ -1557,7 +1575,7 @@ __global__ void __launch_bounds__(NTC, 4) k_rows_cap(RowArgs a) {
         rs.nnuc = nnuc;
         a.ws.stats[r] = rs;
     }
-    row_finished(a, r, smem);
+    row_finished<NTC>(a, r, smem);
 }
 
 static int gcd_int(int x, int y) {
@@ -1569,22 +1587,32 @@ static int gcd_int(int x, int y) {
     return x;
 }
 
+// Threads per CTA.  A launch of at most one row per SM takes 1024, of at most
+// two 512: one row's chain of dependent steps is then the whole time, and an
+// SM's loads in flight come from that row alone.
+static int rows_cap_threads(const RowArgs &a) {
+#ifdef VNT
+    if (a.rows > 2 * a.nsm && a.rows < 700) return VNT;
+#endif
+    return a.rows <= a.nsm ? 1024 : (a.rows <= 2 * a.nsm ? 512 : 256); }
+
 // Tile order and sample size of a row of a.V elements of type dt: the
-// stride is the smallest integer >= ntile / TPI coprime with ntile, so the
-// first TPI tiles are spread over the whole row.
+// stride is the smallest integer >= ntile / SAMPLE coprime with ntile, so the
+// first SAMPLE tiles are spread over the whole row.
 void rows_cap_layout(RowArgs &a, int dt) {
+    const int nt = rows_cap_threads(a), nwc = nt / 32, tpi = nwc * UC;  // as in the kernel
     const int epc = dt == ACES_BF16 ? 8 : 4;
     const int nch = a.V / epc;
     const int ntile = (nch + TCH - 1) / TCH;
-    int p = ntile / TPI;
+    int p = ntile / SAMPLE;
     if (p < 1) p = 1;
     while (gcd_int(p, ntile) != 1) ++p;
     a.ntile = ntile;
     a.pstride = p;
-    a.pstride_w = (int)((long long)NWC * p % ntile);
-    a.pstride_it = (int)((long long)TPI * p % ntile);
+    a.pstride_w = (int)((long long)nwc * p % ntile);
+    a.pstride_it = (int)((long long)tpi * p % ntile);
     long long samp = 0;
-    const int first = ntile < TPI ? ntile : TPI;
+    const int first = ntile < SAMPLE ? ntile : SAMPLE;
     for (int t = 0; t < first; ++t) {
         const long long tile = (long long)t * p % ntile;
         const long long c0 = tile * TCH, c1 = c0 + TCH < nch ? c0 + TCH : nch;
@@ -1595,25 +1623,25 @@ void rows_cap_layout(RowArgs &a, int dt) {
     if (nch % TCH != 0)
         for (int t = 0; t < ntile; ++t)
             if ((long long)t * p % ntile == ntile - 1) {
-                a.it_partial = t / TPI;
+                a.it_partial = t / tpi;
                 break;
             }
     a.inv_ws = (float)(SPB / (double)a.T);
     a.nmin = 2 * a.k + 64 > 256 ? 2 * a.k + 64 : 256;
     // sketch groups: 4 chunks (two per thread and iteration) when they fit,
     // else 8 chunks of 2^sk_ish iterations
-    const int nit = (ntile + TPI - 1) / TPI;
+    const int nit = (ntile + tpi - 1) / tpi;
     a.sk_gpi = 2;
     a.sk_ish = 0;
-    if ((long long)nit * NTC * 2 > SKG) {
+    if ((long long)nit * nt * 2 > SKG) {
         a.sk_gpi = 1;
-        while ((long long)((nit + (1 << a.sk_ish) - 1) >> a.sk_ish) * NTC > SKG) ++a.sk_ish;
+        while ((long long)((nit + (1 << a.sk_ish) - 1) >> a.sk_ish) * nt > SKG) ++a.sk_ish;
     }
 }
 
 // The dynamic shared memory above 48 KB needs an opt-in per device, set
 // once per device on the first launch there (outside any stream capture).
-template <int DT, int W>
+template <int DT, int W, int NTC>
 static cudaError_t launch_cap_dt(const RowArgs &a, cudaStream_t s) {
     constexpr int smem = DT == ACES_BF16 ? SMEM_BF : F32Caps<W>::SMEM;
     static std::mutex mu;
@@ -1623,20 +1651,23 @@ static cudaError_t launch_cap_dt(const RowArgs &a, cudaStream_t s) {
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!ready[dev]) {
-            const cudaError_t e = cudaFuncSetAttribute(k_rows_cap<DT, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            const cudaError_t e = cudaFuncSetAttribute(k_rows_cap<DT, W, NTC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e != cudaSuccess) return e;
             ready[dev] = true;
         }
     }
-    k_rows_cap<DT, W><<<(unsigned)a.rows, NTC, smem, s>>>(a);
+    k_rows_cap<DT, W, NTC><<<(unsigned)a.rows, NTC, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-// one CTA per row (16-byte aligned rows)
+// one CTA per row (16-byte aligned rows; float32: the wide areas when the
+// launch is one wave at two CTAs per SM)
 cudaError_t launch_rows_cap(const RowArgs &a, int dt, cudaStream_t s) {
-    if (dt == ACES_BF16) return launch_cap_dt<ACES_BF16, 1>(a, s);
-    // (float32: the wide areas when the launch is one wave at two CTAs per SM)
-    return a.rows <= 2 * a.nsm ? launch_cap_dt<ACES_F32, 2>(a, s) : launch_cap_dt<ACES_F32, 1>(a, s);
+    switch (rows_cap_threads(a)) {
+        case 1024: return dt == ACES_BF16 ? launch_cap_dt<ACES_BF16, 1, 1024>(a, s) : launch_cap_dt<ACES_F32, 2, 1024>(a, s);
+        case 512: return dt == ACES_BF16 ? launch_cap_dt<ACES_BF16, 1, 512>(a, s) : launch_cap_dt<ACES_F32, 2, 512>(a, s);
+        default: return dt == ACES_BF16 ? launch_cap_dt<ACES_BF16, 1, 256>(a, s) : launch_cap_dt<ACES_F32, 1, 256>(a, s);
+    }
 }
 
 #ifdef ACES_CHECKED
