@@ -36,10 +36,10 @@ sys.path.insert(0, ROOT)
 METRIC = "verified rows/s and achieved HBM GB/s (fraction of GB300 peak) for verify+sparsify"
 WORKLOAD = "b256_k16_v256000_bf16"
 SWEEP_B = (32, 64, 128, 256)
-# kernels of one step: k_rows_cap, k_rows_general, k_resolve_seg,
-# k_resolve_pick (aces_verify), k_cache_build, k_cache_lookup
-KERNELS_PER_STEP = 6
-VERIFY_KERNELS = ["k_rows_cap", "k_rows_general", "k_resolve_seg", "k_resolve_pick"]
+# kernels of one step: k_rows_cap, k_rows_general (aces_verify),
+# k_cache_build, k_cache_lookup
+KERNELS_PER_STEP = 4
+VERIFY_KERNELS = ["k_rows_cap", "k_rows_general"]
 # path counters at the start of the workspace (int32 words)
 PATHS = ["rows_on_general_kernel", "timeouts", "rows_value_histogram", "rows_bitonic_order",
          "general_rows_radix", "rows_cut_left_to_resolve", "general_rows_value_histogram",
@@ -157,7 +157,7 @@ def measured_peak():
 
 # device code behind each profiled kernel (its file and the shared device header)
 KERNEL_SOURCES = {
-    "aces_verify": ("common.cuh", "rows_cap.cu", "rows_general.cu", "resolve.cu"),
+    "aces_verify": ("common.cuh", "draw.cuh", "rows_cap.cu", "rows_general.cu"),
     "k_cache_build": ("common.cuh", "cache.cu"),
 }
 

@@ -40,30 +40,23 @@ aces_status check_rows(const void *logits, aces_dtype dt, long long rows, int V,
     return ACES_OK;
 }
 
-// Row kernels: the single-pass capture kernel when rows are 16-byte
-// aligned, then the exact general kernel for every row it handed over (or
-// for every row otherwise).
+// Row kernels: the single-pass kernel, then the exact general kernel for every
+// row it handed over and for the draws left to it.
 aces_status run_rows(RowArgs &a, aces_dtype dt, bool exact, cudaStream_t s) {
     const size_t es = elem_size(dt);
     const bool vec = aligned16(a.logits) && ((size_t)a.V * es) % 16 == 0;
     const int nsm = sm_count();
     const int nseq = a.K > 0 ? a.rows / (a.K + 1) : a.rows;
     if (cudaMemsetAsync(a.ws.fb_count, 0, ws_clear_bytes(nseq, a.K), s) != cudaSuccess) return ACES_ERR_CUDA;
-    const int grid = a.rows < 2 * nsm ? a.rows : 2 * nsm;
     a.nsm = nsm;
     // With many waves of rows the four CTAs an SM starts with would reach
     // their epilogues (when few loads are in flight) together, wave after
     // wave: their starts are spread over about a quarter of a row's time.
     a.stagger_ns = a.rows >= 16 * nsm ? STAGGER_NS : 0;
-    if (vec) {
-        rows_cap_layout(a, dt);
-        a.force_fb = exact ? 1 : 0;
-        if (launch_rows_cap(a, dt, s) != cudaSuccess) return ACES_ERR_CUDA;
-        if (launch_rows_general(a, dt, true, 0, grid, s) != cudaSuccess) return ACES_ERR_CUDA;
-    } else {
-        a.force_fb = 0;
-        if (launch_rows_general(a, dt, false, 1, grid, s) != cudaSuccess) return ACES_ERR_CUDA;
-    }
+    rows_cap_layout(a, dt, !vec);
+    a.force_fb = exact ? 1 : 0;
+    if (launch_rows_cap(a, dt, !vec, s) != cudaSuccess) return ACES_ERR_CUDA;
+    if (launch_rows_general(a, dt, vec, nseq, s) != cudaSuccess) return ACES_ERR_CUDA;
     return ACES_OK;
 }
 
@@ -133,26 +126,7 @@ aces_status aces::verify_impl(const void *target_logits, aces_dtype dt, const fl
     a.ws = ws_carve(workspace, rows, B, K, lists && top_p < 1.0f);
     a.accept_len = accept_len;
     a.out_token = out_token;
-    st = run_rows(a, dt, exact, s);
-    if (st != ACES_OK) return st;
-    ResolveArgs r;
-    r.logits = target_logits;
-    r.q = draft_probs;
-    r.u = uniforms;
-    r.B = B;
-    r.K = K;
-    r.V = V;
-    r.T = T;
-    r.top_p = top_p;
-    r.k = k;
-    r.ws = a.ws;
-    r.accept_len = accept_len;
-    r.out_token = out_token;
-    r.row_status = row_status;
-    const bool vec = aligned16(target_logits) && ((size_t)V * elem_size(dt)) % 16 == 0 &&
-                     aligned16(draft_probs) && V % 4 == 0;
-    if (launch_resolve(r, dt, vec, s) != cudaSuccess) return ACES_ERR_CUDA;
-    return ACES_OK;
+    return run_rows(a, dt, exact, s);
 }
 
 extern "C" {
@@ -431,7 +405,7 @@ const char *aces_status_string(aces_status s) {
 extern "C" aces_status aces_checked_violation(unsigned long long out[3]) {
     if (!out) return ACES_ERR_INVALID_ARG;
     if (cudaDeviceSynchronize() != cudaSuccess) return ACES_ERR_CUDA;
-    cudaError_t (*take[])(unsigned long long *) = {check_take_rows_cap, check_take_rows_general, check_take_resolve,
+    cudaError_t (*take[])(unsigned long long *) = {check_take_rows_cap, check_take_rows_general,
                                                    check_take_cache, check_take_resample, check_take_kv,
                                                    check_take_mask};
     out[0] = out[1] = out[2] = 0ull;

@@ -42,7 +42,6 @@ static inline cudaError_t check_take(unsigned long long out[3]) {
 }
 cudaError_t check_take_rows_cap(unsigned long long out[3]);
 cudaError_t check_take_rows_general(unsigned long long out[3]);
-cudaError_t check_take_resolve(unsigned long long out[3]);
 cudaError_t check_take_cache(unsigned long long out[3]);
 cudaError_t check_take_resample(unsigned long long out[3]);
 cudaError_t check_take_kv(unsigned long long out[3]);
@@ -65,11 +64,10 @@ constexpr int RS_HANDOFF = 4;
 // the nucleus ends among the ids of one bfloat16 value whose ids were not
 // kept: cut holds that value's 32-bit order key in its high word and j, the
 // number of its ids (in id order) inside the nucleus, in its low word; the
-// resolve step turns it into the order value of the last nucleus id before
-// it reads the row
+// draw finds those ids when it reads the row
 constexpr int RS_LAZY = 8;
 
-// Per-row state written by the row kernels and read by the resolve kernel.
+// Per-row state written by the row kernels and read by the sequence's draw.
 struct RowStat {
     float kref;              // log2 reference: masses are 2^(z*c - kref)
     float c;                 // log2(e) / T
@@ -120,18 +118,24 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// (cluster: CTAs of a thread-block cluster)
 template <typename... P, typename... A>
-inline cudaError_t launch_after(void (*fn)(P...), unsigned grid, unsigned block, cudaStream_t s, A... args) {
+inline cudaError_t launch_after(void (*fn)(P...), unsigned grid, unsigned block, unsigned cluster, cudaStream_t s,
+                                A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
@@ -354,15 +358,6 @@ __device__ __forceinline__ unsigned long long floor_u_times(float uu, unsigned l
     return thr;
 }
 
-// Exact sums of one vocabulary segment of a sequence's row pi (2^-40 units).
-struct SegSum {
-    unsigned long long r;   // residual max(0, p - q) of the nucleus ids, those of a lazy cut's value aside
-    unsigned long long p;   // p itself, likewise
-    unsigned long long tr;  // residual of the ids of a lazy cut's value
-    int bad;                // a NaN / negative draft probability was seen
-    int nt;                 // ids of a lazy cut's value
-};
-constexpr int NSEG_MAX = 16;
 constexpr int STAGGER_NS = 10000;  // row kernel: first-wave start spread per CTA of an SM
 constexpr int NUC_CAP = 512;  // nucleus entries kept per row for the residual step
 
@@ -372,49 +367,51 @@ constexpr int WS_DEPTH = 16;          // first of the 40 depth counters of the r
 constexpr int CARRY_MAGIC = 0x41434531;  // marks a written carry area
 // Workspace layout (all offsets 16-byte aligned)
 struct Workspace {
-    int *carry;                // [64] never cleared: the previous call's hints (written by the resolve
-                               //       step): [0] CARRY_MAGIC, [1] T bits, [2] top_p bits, [3] k, [4] V,
+    int *carry;                // [64] never cleared: the previous call's hints (written by the general
+                               //       kernel): [0] CARRY_MAGIC, [1] T bits, [2] top_p bits, [3] k, [4] V,
                                //       [5] dtype, [6] rows that published a depth, [7] short rows,
                                //       [16..55] how many rows needed each depth
     int *fb_count;             // [64] path counters and depth hints, cleared by every call: [0] rows handed to the
                                //       general kernel, [1] reserved (no kernel waits on another),
                                //       [2] bfloat16 rows finished from their value counts, [3] rows
                                //       ordered by bitonic sort, [4] rows the general kernel finished
-                               //       by radix selection, [5] rows whose cut was left to the resolve
-                               //       step, [6] rows the general kernel finished by value histogram,
+                               //       by radix selection, [5] rows whose cut was left to the draw,
+                               //       [6] rows the general kernel finished by value histogram,
                                //       [7] accept tests that ranked the draft token among ties,
                                //       [8] rows that published the depth they needed, [9] rows that
                                //       took their depth from finished rows, [10] rows counted again
                                //       in a second pass, [11] bfloat16 rows that published a short
                                //       nucleus, [12] rows finished by the sketch-led pass,
+                               //       [13] sequences left to the general kernel's draw,
                                //       [16..55] how many rows needed each depth (in bins of T/4
                                //       below the row max)
+    int *scan_list;            // [B]              (verify only) sequences left to the general kernel's draw
+                               //                  (b * 32 + pi)
     RowStat *stats;            // [rows]
     int *acc;                  // [B*K] accept bits
     int *fb_list;              // [rows]
-    SegSum *seg;               // [B*NSEG_MAX]     (verify only) cleared by every call
-    int *seqcnt;               // [B]              (verify only) rows of the sequence finished by the row kernel
-    int *seqdone;              // [B]              (verify only) token already drawn
+    int *seqcnt;               // [B]              (verify only) finished rows of the sequence, cleared by every call
     unsigned long long *nuc;   // [rows*NUC_CAP]   (verify with lists) nucleus order values
 };
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 // rows = B*(K+1) target rows; nseq = B sequences with K draft positions (K = 0: sparsify);
 // lists: keep every row's nucleus (up to NUC_CAP ids) for the residual step
+// (ws_reserved: bytes no kernel uses any more, kept so that the size a caller
+// has to provide, and with it the largest batch of aces_verify_noalloc, stays)
+__host__ __device__ inline size_t ws_reserved(int nseq) { return (size_t)nseq * 512; }
 __host__ __device__ inline size_t ws_bytes(int rows, int nseq, int K, bool lists) {
     size_t b = WS_CARRY + WS_COUNTERS + align16((size_t)rows * sizeof(RowStat)) + align16((size_t)nseq * K * 4) +
                align16((size_t)rows * 4);
     if (K > 0) {
-        b += 2 * align16((size_t)nseq * 4) + align16((size_t)nseq * NSEG_MAX * sizeof(SegSum));
+        b += 2 * align16((size_t)nseq * 4) + ws_reserved(nseq);
         if (lists) b += (size_t)rows * NUC_CAP * 8;
     }
     return b;
 }
-// bytes at the start of the workspace that every call clears: the counters
-// and, for verification, the per-sequence row counts and done flags and the
-// segment sums (added to atomically)
+// bytes after the carried hints that every call clears: the counters and, for
+// verification, the per-sequence row counts
 __host__ __device__ inline size_t ws_clear_bytes(int nseq, int K) {
-    return WS_COUNTERS +
-           (K > 0 ? 2 * align16((size_t)nseq * 4) + align16((size_t)nseq * NSEG_MAX * sizeof(SegSum)) : 0);
+    return WS_COUNTERS + (K > 0 ? align16((size_t)nseq * 4) : 0);
 }
 __host__ __device__ inline Workspace ws_carve(void *base, int rows, int nseq, int K, bool lists) {
     char *p = (char *)base;
@@ -424,15 +421,12 @@ __host__ __device__ inline Workspace ws_carve(void *base, int rows, int nseq, in
     w.fb_count = (int *)p;
     p += WS_COUNTERS;
     w.seqcnt = nullptr;
-    w.seqdone = nullptr;
-    w.seg = nullptr;
+    w.scan_list = nullptr;
     if (K > 0) {
         w.seqcnt = (int *)p;
         p += align16((size_t)nseq * 4);
-        w.seqdone = (int *)p;
-        p += align16((size_t)nseq * 4);
-        w.seg = (SegSum *)p;
-        p += align16((size_t)nseq * NSEG_MAX * sizeof(SegSum));
+        w.scan_list = (int *)p;
+        p += align16((size_t)nseq * 4) + ws_reserved(nseq);
     }
     w.stats = (RowStat *)p;
     p += align16((size_t)rows * sizeof(RowStat));
@@ -466,12 +460,12 @@ struct RowArgs {
     int32_t *accept_len;   // verification outputs (null for sparsify)
     int32_t *out_token;
     Workspace ws;
-    // capture row kernel (16-byte aligned rows): the row's 16-byte chunks are
+    // single-pass row kernel: the row's 16-byte chunks are
     // read in tiles of 32 (one coalesced warp load), tile t of the row order
     // at position (t * pstride) mod ntile, so that the first iteration reads
     // a strided sample of samp_frac of the row
     int ntile, pstride, pstride_w, pstride_it;
-    int it_partial;        // iteration that reads the row's partial last tile (-1: none)
+    int it_partial, it_partial2;  // iterations that read the row's partial last tiles (-1: none)
     float samp_frac;
     float inv_ws;          // sample bins per unit of logit: SPB / T
     int nmin;              // float32 first rows: ids the capture must reach
@@ -480,20 +474,6 @@ struct RowArgs {
     int force_fb;          // hand every row to the general kernel (the library's exact reference path)
     int nsm;               // SMs of the device
     int stagger_ns;        // start of the first-wave CTAs of an SM spread by this (0: none)
-};
-
-// Arguments of the sequence kernel.
-struct ResolveArgs {
-    const void *logits;
-    const float *q;
-    const float *u;
-    int B, K, V;
-    float T, top_p;  // (with k: the key of the hints carried to the next call)
-    int k;
-    Workspace ws;
-    int32_t *accept_len;
-    int32_t *out_token;
-    int32_t *row_status;
 };
 
 // Arguments of the cache kernels.
@@ -516,112 +496,6 @@ __device__ __forceinline__ int first_reject_warp(const Workspace &ws, int b, int
     const bool rej = lane < K && !ws.acc[(size_t)b * K + lane];
     const unsigned bal = __ballot_sync(0xffffffffu, rej);
     return bal ? __ffs(bal) - 1 : K;
-}
-
-struct DrawShared {
-    int pi, bad, tok;
-    unsigned long long thr;
-};
-
-// Residual (pi < K) or bonus (pi = K) draw of sequence b from row pi's stored
-// nucleus (the residual max(0, p - q) is zero outside it): q is read at the
-// nucleus ids only, which are ordered by id, and the token is the smallest id
-// whose prefix sum of 2^-40 fixed-point masses exceeds floor(u * total).
-// Writes accept_len, out_token and seqdone; returns without writing when row
-// pi has no stored nucleus (the scan kernels then draw the sequence).  The
-// ids are ordered by direct rank counting (one pass, no barrier stages).
-// All NTH threads call it, NTH * 2 >= NUC_CAP; skey, srt, rfx, pfx hold
-// NUC_CAP entries, red NTH / 32.
-template <int NTH>
-__device__ void draw_from_list(const Workspace &ws, const float *q, const float *u, int K, int V, int b,
-                               int32_t *accept_len, int32_t *out_token, int32_t *row_status,
-                               unsigned long long *skey, unsigned long long *srt, unsigned long long *rfx,
-                               unsigned long long *pfx, unsigned long long *red, DrawShared *sh) {
-    static_assert(2 * NTH >= NUC_CAP, "two nucleus entries per thread");
-    const int tid = threadIdx.x;
-    if (tid < 32) {
-        const int pi0 = first_reject_warp(ws, b, K);
-        if (tid == 0) sh->pi = pi0;
-    }
-    if (tid == 0) {
-        sh->bad = 0;
-        sh->tok = -1;
-    }
-    __syncthreads();
-    const int pi = sh->pi;
-    const int r = b * (K + 1) + pi;
-    const RowStat rs = ws.stats[r];
-    if (rs.flags & RS_NONFINITE) {
-        if (tid == 0) {
-            accept_len[b] = pi;
-            out_token[b] = -1;
-            ws.seqdone[b] = 1;
-        }
-        return;
-    }
-    if (rs.nnuc < 0) return;  // no list: the scan kernels draw this sequence
-    const int n = ACES_IN(rs.nnuc - 1, NUC_CAP) ? rs.nnuc : 0;
-    const unsigned long long *lst = ws.nuc + (size_t)r * NUC_CAP;
-    const float *qrow = pi < K ? q + ((size_t)b * K + pi) * V : nullptr;
-    const float inv_S = inv_mass(rs.S_nuc);
-    for (int i = tid; i < n; i += NTH) {
-        const unsigned long long o = lst[i];
-        const uint32_t id = order_id(o);
-        const float p = ex2(fmaf(order_value(o), rs.c, -rs.kref)) * inv_S;
-        float rr = p;
-        if (qrow && ACES_IN(id, V)) {
-            const float qx = __ldg(qrow + id);
-            if (!(qx >= 0.0f)) sh->bad = 1;
-            rr = fmaxf(p - qx, 0.0f);
-        }
-        rfx[i] = to_fx(rr);
-        pfx[i] = to_fx(p);
-        skey[i] = ((unsigned long long)id << 32) | (unsigned long long)i;  // distinct keys
-    }
-    __syncthreads();
-    if (sh->bad) {
-        if (tid == 0) {
-            row_status[r] |= ACES_ROW_BAD_Q;
-            accept_len[b] = pi;
-            out_token[b] = -1;
-            ws.seqdone[b] = 1;
-        }
-        return;
-    }
-    for (int i = tid; i < n; i += NTH) {  // ascending id: each key's rank among the others
-        const unsigned long long key = skey[i];
-        int rank = 0;
-#pragma unroll 4
-        for (int j = 0; j < n; ++j) rank += skey[j] < key;
-        if (ACES_IN(rank, NUC_CAP)) srt[rank] = key;
-    }
-    __syncthreads();
-    // two consecutive entries (in id order) per thread
-    const int e0 = 2 * tid, e1 = 2 * tid + 1;
-    int i0 = e0 < n ? (int)(srt[e0] & 0xFFFFFFFFull) : -1;
-    int i1 = e1 < n ? (int)(srt[e1] & 0xFFFFFFFFull) : -1;
-    if (i0 >= 0 && !ACES_IN(i0, NUC_CAP)) i0 = -1;
-    if (i1 >= 0 && !ACES_IN(i1, NUC_CAP)) i1 = -1;
-    const unsigned long long r0 = i0 >= 0 ? rfx[i0] : 0ull, r1 = i1 >= 0 ? rfx[i1] : 0ull;
-    const unsigned long long R = block_reduce_n<NTH>(r0 + r1, red, SumU64());
-    const int mode = R == 0ull;  // p <= q everywhere: draw from p itself
-    const unsigned long long w0 = mode ? (i0 >= 0 ? pfx[i0] : 0ull) : r0;
-    const unsigned long long w1 = mode ? (i1 >= 0 ? pfx[i1] : 0ull) : r1;
-    unsigned long long tot;
-    const unsigned long long ex = block_exscan_n<NTH>(w0 + w1, red, &tot);
-    if (tid == 0) sh->thr = tot > 0ull ? floor_u_times(u[(size_t)b * (K + 1) + K], tot) : 0ull;
-    __syncthreads();
-    const unsigned long long thr = sh->thr;
-    if (tot > 0ull) {
-        if (ex <= thr && thr < ex + w0) sh->tok = (int)(srt[e0] >> 32);
-        else if (ex + w0 <= thr && thr < ex + w0 + w1) sh->tok = (int)(srt[e1] >> 32);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        accept_len[b] = pi;
-        out_token[b] = sh->tok;
-        ws.seqdone[b] = 1;
-    }
 }
 
 // Outputs of a row whose logits are not a distribution.
@@ -651,10 +525,9 @@ __device__ void nonfinite_row(const RowArgs &a, int r) {
 }
 
 // host launchers (defined next to their kernels)
-void rows_cap_layout(RowArgs &a, int dt);
-cudaError_t launch_rows_cap(const RowArgs &a, int dt, cudaStream_t s);
-cudaError_t launch_rows_general(const RowArgs &a, int dt, bool vec, int direct, int grid, cudaStream_t s);
-cudaError_t launch_resolve(const ResolveArgs &a, int dt, bool vec, cudaStream_t s);
+void rows_cap_layout(RowArgs &a, int dt, bool ragged);
+cudaError_t launch_rows_cap(const RowArgs &a, int dt, bool ragged, cudaStream_t s);
+cudaError_t launch_rows_general(const RowArgs &a, int dt, bool vec, int nseq, cudaStream_t s);
 // aces_verify with two choices, neither of which changes the results: lists =
 // false keeps no nucleus lists (the residual draw scans its row; the call then
 // needs ws_bytes(rows, B, K, lists) bytes of workspace), exact = true hands

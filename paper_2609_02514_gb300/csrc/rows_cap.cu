@@ -40,8 +40,8 @@
 //                       value are re-read and their ids at or above it
 //                       ordered.  When the crossing value's ids are among them
 //                       the j-th (in id order) is the cut; otherwise the row
-//                       keeps (value, j) and the resolve step finds that id
-//                       only for the rows it draws from.
+//                       keeps (value, j) and the draw finds that id, only for
+//                       the rows it draws from.
 //             float32   the recorded ids are binned by (m - z)/(T/8); the bins
 //                       up to the one where a lower bound of the mass reaches
 //                       the target are ordered (direct ranking up to 512 ids,
@@ -60,7 +60,7 @@
 #include <cuda_bf16.h>
 
 #define ACES_FILE 9  // site numbers of the checked build
-#include "common.cuh"
+#include "draw.cuh"
 
 namespace aces {
 
@@ -112,7 +112,7 @@ struct F32Caps {
 
 constexpr int RANK_MAX = 512;       // ids ordered by direct ranking (more: bitonic sort)
 static_assert(WS_DEPTH + NSB <= WS_COUNTERS / 4, "the depth histogram fits the counters area");
-static_assert(4 * NUC_CAP * 8 <= SMEM_BF && 4 * NUC_CAP * 8 <= SMEM_F32, "the draw's scratch fits");
+static_assert(DRAW_SCRATCH <= SMEM_BF && DRAW_SCRATCH <= SMEM_F32, "the draw's scratch fits");
 static_assert(GCAP * 4 <= HW * 4 && PCAP * 8 <= SKG * 2 && "the aliased areas fit");
 static_assert(PCAP <= SK_TMP && SK_TMP + GCAP / 2 <= SKG / 4 && SK_TMP + PCAP <= SKG / 4, "the sketch-led areas fit");
 static_assert(WCAP * 8 <= CREC * 20 && RANK_MAX * 2 <= LCAP, "the float32 work areas fit");
@@ -279,27 +279,6 @@ __device__ __forceinline__ float val16(uint32_t k) {
     return __uint_as_float(b << 16);
 }
 
-// Called by all threads when this CTA has written row r's outputs and state.
-// The CTA that finishes the last row of a sequence (rows handed to the
-// general kernel are never counted) draws the sequence's token from the
-// stored nucleus, so most sequences need no separate resolve launch.
-template <int NTC>
-__device__ void row_finished(const RowArgs &a, int r, unsigned char *scratch) {
-    if (a.ws.seqcnt == nullptr) return;  // sparsify
-    __shared__ int s_last;
-    __shared__ unsigned long long s_red[NTC / 32];
-    __shared__ DrawShared s_draw;
-    const int b = r / (a.K + 1);
-    __syncthreads();  // every thread's writes of this row are issued
-    // releases this row's writes; the last row acquires the others'
-    if (threadIdx.x == 0) s_last = atomic_add_acq_rel(&a.ws.seqcnt[b], 1) == a.K;
-    __syncthreads();
-    if (!s_last) return;
-    unsigned long long *skey = reinterpret_cast<unsigned long long *>(scratch);  // 4 * NUC_CAP entries
-    draw_from_list<NTC>(a.ws, a.q, a.u, a.K, a.V, b, a.accept_len, a.out_token, a.row_status, skey,
-                        skey + NUC_CAP, skey + 2 * NUC_CAP, skey + 3 * NUC_CAP, s_red, &s_draw);
-}
-
 // Hands row r to the general kernel with its max m and its exp-sum S (in
 // units of 2^kref), which spare that kernel a pass and the exponentials of
 // another (the row is finite: rows with NaN or +inf are marked NONFINITE
@@ -336,7 +315,9 @@ __device__ __forceinline__ unsigned long long id_fx(float v, float c, float kref
 }
 
 // NTC: threads per CTA, 1024 / NTC CTAs per SM
-template <int DT, int W, int NTC>
+// (RAGGED: rows off the 16-byte grid; a build of its own, as the edges cost
+// the other one registers: 128 x 17 rows of 128256 205 -> 213 us)
+template <int DT, int W, int NTC, bool RAGGED>
 __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     constexpr int NWC = NTC / 32;
     constexpr int TPI = NWC * UC;         // tiles per iteration
@@ -387,8 +368,11 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         const unsigned long long t0 = globaltimer_ns();
         for (int i = 0; i < 1000 && globaltimer_ns() - t0 < wait; ++i) __nanosleep(1000);
     }
-    const char *row = reinterpret_cast<const char *>(a.logits) + (size_t)r * a.V * E::SIZE;
-    const int nch = a.V / EPC, ntile = a.ntile;
+    // (a row off the 16-byte grid: its chunks are cut at the boundaries, the
+    // first and the last padded with -inf)
+    const RowChunks<DT, RAGGED> rc(reinterpret_cast<const char *>(a.logits) + (size_t)r * a.V * E::SIZE, a.V);
+    const char *row = rc.base;
+    const int nch = rc.nch, ntile = a.ntile;
     const int nit = (ntile + TPI - 1) / TPI;
     const uint32_t NI = E::NEG_INF_WORD;
     const bool all_in = a.top_p >= 1.0f;
@@ -448,14 +432,16 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     auto wrap = [&](uint32_t off) -> uint32_t { return min(off, off - tile_end); };
     // (iterations whose tiles all exist and are whole load without checks:
     // only the last iteration can hold fewer tiles, and only the row's last
-    // tile can be partial)
+    // tile can be partial; off the 16-byte grid also the first and the one
+    // before the last)
     auto load = [&](int it) {
         uint32_t off = off0;
-        if ((it + 1) * TPI > ntile || it == a.it_partial) {
+        if ((it + 1) * TPI > ntile || it == a.it_partial ||
+            (RAGGED && (it == 0 || it == a.it_partial2))) {
 #pragma unroll
             for (int u = 0; u < UC; ++u) {
                 const int t = it * TPI + u * NWC + wid;
-                w[u] = (t < ntile && off < (uint32_t)nch * 16u) ? ldg16(row + off) : make_uint4(NI, NI, NI, NI);
+                w[u] = (t < ntile && off < (uint32_t)nch * 16u) ? rc.load((int)(off >> 4)) : make_uint4(NI, NI, NI, NI);
                 off = wrap(off + off_w);
             }
         } else {
@@ -557,7 +543,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         xb = tid == 0 ? s_xb : -1;
         if (xb >= 0 && xb < a.V) {
-            zx = E::load1(row, xb);
+            zx = E::load1(row + rc.head * E::SIZE, xb);
             qx = __ldg(a.q + ((size_t)bq * a.K + iq) * a.V + xb);
             ux = __ldg(a.u + (size_t)bq * (a.K + 1) + iq);
         }
@@ -624,7 +610,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         if (!(sh > 0.0f && sh < INFINITY) || !(m < INFINITY) || !(kref < 1e30f)) {
             nonfinite_row<NTC>(a, r);
-            row_finished<NTC>(a, r, smem);
+            row_finished<DT, NTC, true>(a, r, smem);
             return true;
         }
         return false;
@@ -949,7 +935,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                             const int c = (int)((long long)t * a.pstride % ntile) * TCH + (tl & 31);
                             if (c < nch) cc[h] = c;
                         }
-                        dat[h] = cc[h] >= 0 ? ldg16(row + (size_t)cc[h] * 16) : make_uint4(NI, NI, NI, NI);
+                        dat[h] = cc[h] >= 0 ? rc.load(cc[h]) : make_uint4(NI, NI, NI, NI);
                     }
                     uint32_t hm = 0u;
 #pragma unroll
@@ -968,7 +954,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                         while (m8) {
                             const int e = __ffs(m8) - 1;
                             m8 &= m8 - 1u;
-                            put(at, __float_as_uint(chunk_elem<DT>(dat[h], e)) >> 16, (uint32_t)(cc[h] * EPC + e));
+                            put(at, __float_as_uint(chunk_elem<DT>(dat[h], e)) >> 16, (uint32_t)(cc[h] * EPC + e - rc.head));
                             ++at;
                         }
                     }
@@ -1047,7 +1033,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
 #pragma unroll
                 for (int u = 0; u < UC; ++u) {
                     const int c = c0 + u * NTC + tid;
-                    w[u] = c < nch ? ldg16(row + (size_t)c * 16) : make_uint4(NI, NI, NI, NI);
+                    w[u] = c < nch ? rc.load(c) : make_uint4(NI, NI, NI, NI);
                 }
 #pragma unroll
                 for (int u = 0; u < UC; ++u) count_chunk(w[u], thb0);
@@ -1124,12 +1110,12 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         // the draft token's value equals the crossing value and that value's
         // ids were not read: its rank among them (ids below it) decides
         if (lazy && s_xb >= 0 && s_xb < a.V && key16(__float_as_uint(s_zx) >> 16) == 0x8000u + vsb) {
-            const int xr = s_xb;
+            const int xr = s_xb + rc.head;  // (a position in chunks)
             const float vsv = val16(0x8000u + vsb);
             const __nv_bfloat162 v2 = __floats2bfloat162_rn(vsv, vsv);
             uint32_t cnt = 0u;
             for (int cc = tid; cc * EPC < xr; cc += NTC) {
-                const uint4 wv = ldg16(row + (size_t)cc * 16);
+                const uint4 wv = rc.load(cc);
                 const uint32_t wd[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -1284,7 +1270,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             const int i = i0 + tid;
             const bool in = i < nrec;
             const uint4 dat = in ? rec_dat[i] : make_uint4(NI, NI, NI, NI);
-            const uint32_t base = in ? rec_idx[i] * (uint32_t)EPC : 0u;
+            const uint32_t base = in ? rec_idx[i] * (uint32_t)EPC - (uint32_t)rc.head : 0u;
 #pragma unroll
             for (int e = 0; e < EPC; ++e) {
                 const float v = Elem<DT>::get(dat, e);
@@ -1575,7 +1561,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         rs.nnuc = nnuc;
         a.ws.stats[r] = rs;
     }
-    row_finished<NTC>(a, r, smem);
+    row_finished<DT, NTC, true>(a, r, smem);
 }
 
 static int gcd_int(int x, int y) {
@@ -1590,19 +1576,16 @@ static int gcd_int(int x, int y) {
 // Threads per CTA.  A launch of at most one row per SM takes 1024, of at most
 // two 512: one row's chain of dependent steps is then the whole time, and an
 // SM's loads in flight come from that row alone.
-static int rows_cap_threads(const RowArgs &a) {
-#ifdef VNT
-    if (a.rows > 2 * a.nsm && a.rows < 700) return VNT;
-#endif
-    return a.rows <= a.nsm ? 1024 : (a.rows <= 2 * a.nsm ? 512 : 256); }
+static int rows_cap_threads(const RowArgs &a) { return a.rows <= a.nsm ? 1024 : (a.rows <= 2 * a.nsm ? 512 : 256); }
 
-// Tile order and sample size of a row of a.V elements of type dt: the
+// Tile order and sample size of a row of a.V elements of type dt (ragged: its
+// rows are off the 16-byte grid, up to one chunk longer): the
 // stride is the smallest integer >= ntile / SAMPLE coprime with ntile, so the
 // first SAMPLE tiles are spread over the whole row.
-void rows_cap_layout(RowArgs &a, int dt) {
+void rows_cap_layout(RowArgs &a, int dt, bool ragged) {
     const int nt = rows_cap_threads(a), nwc = nt / 32, tpi = nwc * UC;  // as in the kernel
     const int epc = dt == ACES_BF16 ? 8 : 4;
-    const int nch = a.V / epc;
+    const int nch = ragged ? (a.V + epc - 1 + epc - 1) / epc : a.V / epc;
     const int ntile = (nch + TCH - 1) / TCH;
     int p = ntile / SAMPLE;
     if (p < 1) p = 1;
@@ -1616,16 +1599,18 @@ void rows_cap_layout(RowArgs &a, int dt) {
     for (int t = 0; t < first; ++t) {
         const long long tile = (long long)t * p % ntile;
         const long long c0 = tile * TCH, c1 = c0 + TCH < nch ? c0 + TCH : nch;
-        samp += (c1 - c0) * epc;
+        samp += (c1 - c0) * epc;  // (off the grid: a few too many)
     }
     a.samp_frac = (float)((double)samp / (double)a.V);
-    a.it_partial = -1;  // the iteration that reads the partial last tile
-    if (nch % TCH != 0)
-        for (int t = 0; t < ntile; ++t)
-            if ((long long)t * p % ntile == ntile - 1) {
-                a.it_partial = t / tpi;
-                break;
-            }
+    // the iterations that read the partial last tile (off the grid the row's
+    // last chunk, partial itself, lies in one of the last two)
+    a.it_partial = a.it_partial2 = -1;
+    if (nch % TCH != 0 || ragged)
+        for (int t = 0; t < ntile; ++t) {
+            const long long tile = (long long)t * p % ntile;
+            if (tile == ntile - 1) a.it_partial = t / tpi;
+            if (ragged && tile == ntile - 2) a.it_partial2 = t / tpi;
+        }
     a.inv_ws = (float)(SPB / (double)a.T);
     a.nmin = 2 * a.k + 64 > 256 ? 2 * a.k + 64 : 256;
     // sketch groups: 4 chunks (two per thread and iteration) when they fit,
@@ -1641,7 +1626,7 @@ void rows_cap_layout(RowArgs &a, int dt) {
 
 // The dynamic shared memory above 48 KB needs an opt-in per device, set
 // once per device on the first launch there (outside any stream capture).
-template <int DT, int W, int NTC>
+template <int DT, int W, int NTC, bool RAGGED>
 static cudaError_t launch_cap_dt(const RowArgs &a, cudaStream_t s) {
     constexpr int smem = DT == ACES_BF16 ? SMEM_BF : F32Caps<W>::SMEM;
     static std::mutex mu;
@@ -1651,23 +1636,29 @@ static cudaError_t launch_cap_dt(const RowArgs &a, cudaStream_t s) {
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!ready[dev]) {
-            const cudaError_t e = cudaFuncSetAttribute(k_rows_cap<DT, W, NTC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            const cudaError_t e = cudaFuncSetAttribute(k_rows_cap<DT, W, NTC, RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e != cudaSuccess) return e;
             ready[dev] = true;
         }
     }
-    k_rows_cap<DT, W, NTC><<<(unsigned)a.rows, NTC, smem, s>>>(a);
+    k_rows_cap<DT, W, NTC, RAGGED><<<(unsigned)a.rows, NTC, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-// one CTA per row (16-byte aligned rows; float32: the wide areas when the
-// launch is one wave at two CTAs per SM)
-cudaError_t launch_rows_cap(const RowArgs &a, int dt, cudaStream_t s) {
+// one CTA per row (float32: the wide areas when the launch is one wave at two
+// CTAs per SM)
+template <int DT, bool RAGGED>
+static cudaError_t launch_cap(const RowArgs &a, cudaStream_t s) {
+    constexpr int WIDE = DT == ACES_F32 ? 2 : 1;
     switch (rows_cap_threads(a)) {
-        case 1024: return dt == ACES_BF16 ? launch_cap_dt<ACES_BF16, 1, 1024>(a, s) : launch_cap_dt<ACES_F32, 2, 1024>(a, s);
-        case 512: return dt == ACES_BF16 ? launch_cap_dt<ACES_BF16, 1, 512>(a, s) : launch_cap_dt<ACES_F32, 2, 512>(a, s);
-        default: return dt == ACES_BF16 ? launch_cap_dt<ACES_BF16, 1, 256>(a, s) : launch_cap_dt<ACES_F32, 1, 256>(a, s);
+        case 1024: return launch_cap_dt<DT, WIDE, 1024, RAGGED>(a, s);
+        case 512: return launch_cap_dt<DT, WIDE, 512, RAGGED>(a, s);
+        default: return launch_cap_dt<DT, 1, 256, RAGGED>(a, s);
     }
+}
+cudaError_t launch_rows_cap(const RowArgs &a, int dt, bool ragged, cudaStream_t s) {
+    if (dt == ACES_BF16) return ragged ? launch_cap<ACES_BF16, true>(a, s) : launch_cap<ACES_BF16, false>(a, s);
+    return ragged ? launch_cap<ACES_F32, true>(a, s) : launch_cap<ACES_F32, false>(a, s);
 }
 
 #ifdef ACES_CHECKED

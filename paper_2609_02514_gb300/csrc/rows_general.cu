@@ -1,9 +1,9 @@
 // Exact general row kernel of the AceSpec cloud step (Sec. III-B; Sec. II-A
 // modified rejection sampling; Sec. V-C payload).  It takes every row that
-// the fast kernel cannot certify (and every row when the logits are not
-// 16-byte aligned).  Masses are in 2^-40 fixed point, so every partial sum
+// the single-pass kernel hands over, and then draws the sequences whose draw
+// needs a whole row.  Masses are in 2^-40 fixed point, so every partial sum
 // is exact and order-independent.  One CTA of 512 threads per row; a
-// persistent grid walks the list of rows handed over by the fast kernel.
+// persistent grid walks the list of rows handed over.
 //   value histogram  (aligned bfloat16 rows) ids counted per bfloat16 value
 //                below the max, the crossing and payload values found by a
 //                prefix scan, their ids collected and ranked: two row reads;
@@ -20,7 +20,7 @@
 #include <cuda_bf16.h>
 
 #define ACES_FILE 10  // site numbers of the checked build
-#include "common.cuh"
+#include "draw.cuh"
 
 namespace aces {
 
@@ -732,7 +732,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const char *row, float m, f
 }
 
 template <int DT, bool VEC>
-__global__ void __launch_bounds__(NT) k_rows_general(RowArgs a, int direct) {
+__global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ RowArgs a) {
     using E = Elem<DT>;
     __shared__ SelState st;
     __shared__ union {
@@ -740,6 +740,8 @@ __global__ void __launch_bounds__(NT) k_rows_general(RowArgs a, int direct) {
         ValHist vh;    // value-histogram path (bfloat16)
     } paths;
     BinState &bst = paths.bs;
+    static_assert(sizeof(paths) >= DRAW_SCRATCH, "the draw's scratch fits");
+    unsigned char *scratch = reinterpret_cast<unsigned char *>(&paths);  // (of a finished row)
     __shared__ unsigned long long buf[ACES_MAX_TOPK];
     __shared__ double redd[NWARP];
     __shared__ float redf[NWARP];
@@ -747,18 +749,33 @@ __global__ void __launch_bounds__(NT) k_rows_general(RowArgs a, int direct) {
     __shared__ int s_bad;
     __shared__ int s_nbuf;
     const int tid = threadIdx.x;
-    pdl_wait();  // after the fast row kernel: its fallback list is complete
-    const int nrows = direct ? a.rows : *a.ws.fb_count;
+    pdl_wait();  // after the single-pass row kernel: its fallback list is complete
+    if (a.K > 0 && blockIdx.x == 0 && tid < WS_COUNTERS / 4) {
+        // the hints of this call's rows, for the first rows of the next call
+        // with the same shape (the row kernel reads them only when fewer than
+        // its minimum of that call's rows have finished)
+        int v = tid >= WS_DEPTH ? __ldcg(&a.ws.fb_count[tid]) : 0;
+        if (tid == 0) v = CARRY_MAGIC;
+        if (tid == 1) v = __float_as_int(a.T);
+        if (tid == 2) v = __float_as_int(a.top_p);
+        if (tid == 3) v = a.k;
+        if (tid == 4) v = a.V;
+        if (tid == 5) v = DT;
+        if (tid == 6) v = __ldcg(&a.ws.fb_count[8]);
+        if (tid == 7) v = __ldcg(&a.ws.fb_count[11]);
+        a.ws.carry[tid] = v;
+    }
+    const int nrows = *a.ws.fb_count;
     for (int idx = blockIdx.x; idx < nrows; idx += gridDim.x) {
-        const int r = direct ? idx : a.ws.fb_list[idx];
+        const int r = a.ws.fb_list[idx];
         if (!ACES_IN(r, a.rows)) continue;  // (the same r in every thread)
         const char *row = reinterpret_cast<const char *>(a.logits) + (size_t)r * a.V * E::SIZE;
-        // a row the fast kernel handed over comes with its max and its
+        // a row the single-pass kernel handed over comes with its max and its
         // exp-sum (and is finite); the max pass runs only where the paths
         // need the finite count it takes (top_p = 1 on float32 rows)
         RowStat hs;
         hs.flags = 0;
-        if (VEC && !direct) hs = a.ws.stats[r];
+        if (VEC) hs = a.ws.stats[r];
         const bool handed = hs.flags == RS_HANDOFF;
         float m;
         unsigned long long n_fin = 0ull;
@@ -781,6 +798,7 @@ __global__ void __launch_bounds__(NT) k_rows_general(RowArgs a, int direct) {
             n_fin = block_reduce(nfin, redu, SumU64());
             if (s_bad || n_fin == 0ull || !(ceilf(m * a.c) < 1e30f)) {
                 nonfinite_row<NT>(a, r);
+                row_finished<DT, NT, false>(a, r, scratch);
                 __syncthreads();
                 continue;
             }
@@ -793,10 +811,15 @@ __global__ void __launch_bounds__(NT) k_rows_general(RowArgs a, int direct) {
             unsigned long long nf = 0ull;
             const bool done = valhist_row(a, r, row, m, kref, S_in, &nf, &paths.vh, buf, redd, redu);
             __syncthreads();
-            if (done) continue;
+            if (done) {
+                row_finished<DT, NT, false>(a, r, scratch);
+                __syncthreads();
+                continue;
+            }
             n_fin = nf;
         }
         if (binned_row<DT, VEC>(a, r, row, m, kref, n_fin, &bst, buf, redd, redu)) {
+            row_finished<DT, NT, false>(a, r, scratch);
             __syncthreads();
             continue;
         }
@@ -846,21 +869,37 @@ __global__ void __launch_bounds__(NT) k_rows_general(RowArgs a, int direct) {
         bitonic_sort_desc(buf, np);
         if (L > nb) L = nb;
         finish_row<DT>(a, r, row, kref, S_nuc, cut, all_in ? RS_ALL_IN : 0, buf, L, redd);
+        row_finished<DT, NT, false>(a, r, scratch);
         __syncthreads();
     }
-    // only now: resolve CTAs waiting beside busy rows would slow them down
-    pdl_trigger();
+    // the sequences whose rows are all done and whose draw needs a whole row
+    if (a.K > 0) {
+        __shared__ DrawPart part;
+        const int nscan = a.ws.fb_count[13];
+        const int ncta = (int)cooperative_groups::this_cluster().num_blocks();
+        for (int i = blockIdx.x / ncta; i < nscan; i += gridDim.x / ncta) {
+            const int e = a.ws.scan_list[i];
+            draw_cluster<DT, NT>(a, e >> 5, e & 31, &part, scratch);
+            __syncthreads();
+        }
+    }
 }
 
-// direct = 0 follows the fast row kernel and overlaps its drain
-cudaError_t launch_rows_general(const RowArgs &a, int dt, bool vec, int direct, int grid, cudaStream_t s) {
-    void (*fn)(RowArgs, int) = dt == ACES_BF16 ? (vec ? k_rows_general<ACES_BF16, true> : k_rows_general<ACES_BF16, false>)
+// Follows the single-pass row kernel and overlaps its drain.  Two
+// CTAs an SM at most, fewer when neither the rows it may be handed nor the
+// draws fill them; the CTAs of a draw's cluster: as many as let every sequence
+// be drawn at once (a draw is a chain of about 20 us however few logits each
+// CTA has: 128 sequences in four rounds of clusters of 8 took 120 us).
+cudaError_t launch_rows_general(const RowArgs &a, int dt, bool vec, int nseq, cudaStream_t s) {
+    const int most = 2 * a.nsm / DRAW_CL * DRAW_CL;
+    int cl = DRAW_CL;
+    while (cl > 2 && (long long)cl * nseq > most) cl >>= 1;
+    long long want = a.K > 0 && (long long)cl * nseq > a.rows ? (long long)cl * nseq : a.rows;
+    want = (want + DRAW_CL - 1) / DRAW_CL * DRAW_CL;
+    const unsigned grid = (unsigned)(want < most ? want : most);
+    void (*fn)(RowArgs) = dt == ACES_BF16 ? (vec ? k_rows_general<ACES_BF16, true> : k_rows_general<ACES_BF16, false>)
                                                : (vec ? k_rows_general<ACES_F32, true> : k_rows_general<ACES_F32, false>);
-    if (direct) {
-        fn<<<grid, NT, 0, s>>>(a, direct);
-        return cudaGetLastError();
-    }
-    return launch_after(fn, (unsigned)grid, NT, s, a, direct);
+    return launch_after(fn, grid, NT, (unsigned)cl, s, a);
 }
 
 #ifdef ACES_CHECKED
