@@ -5,10 +5,10 @@
 // its own branch up to itself (the suffix-diagonal block).
 //
 // Packed order: the main chain (K tokens), then the branches in slot order
-// (the slots of the cache lookup), branch_len tokens each.  One thread
-// writes one 32-bit word of one row: a token's allowed keys are at most two
-// intervals, [0, a) of the main chain and [b, c] of its own branch, so each
-// word is two interval masks.
+// (the slots of the cache lookup), branch_len tokens each.  One warp
+// writes one row: a token's allowed keys are at most two intervals, [0, a) of
+// the main chain and [b, c] of its own branch, so each 32-bit word is two
+// interval masks.
 #define ACES_FILE 5  // site numbers of the checked build
 #include "common.cuh"
 
@@ -30,27 +30,33 @@ __device__ __forceinline__ uint32_t interval_bits(int lo, int hi, int w0) {
     return upto_b & ~upto_a;
 }
 
-__global__ void k_tree_mask(MaskArgs a) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)a.n * a.words) return;
-    const int q = (int)(i / a.words), w = (int)(i % a.words);
-    int main_hi, br_lo, br_hi, dep;  // keys [0, main_hi) and [br_lo, br_hi)
-    if (q < a.K) {
-        main_hi = q + 1;
-        br_lo = br_hi = 0;
-        dep = q;
-    } else {
-        const int s = (q - a.K) / a.branch_len, o = (q - a.K) % a.branch_len;
-        int d = 0;
-        while (d + 1 <= a.K && a.off[d + 1] <= s) ++d;  // depth of slot s
-        main_hi = d;
-        br_lo = a.K + s * a.branch_len;
-        br_hi = q + 1;
-        dep = d + o;
+// Eight warps a CTA, one row each: the row's intervals are found once and its
+// lanes write consecutive words (one thread a word recomputed them with four
+// divisions: 9.2 us for 4616 tokens).
+constexpr int NTM = 256;
+
+__global__ void __launch_bounds__(NTM) k_tree_mask(MaskArgs a) {
+    const int lane = threadIdx.x & 31;
+    for (int q = blockIdx.x * (NTM / 32) + (threadIdx.x >> 5); q < a.n; q += gridDim.x * (NTM / 32)) {
+        int main_hi, br_lo, br_hi, dep;  // keys [0, main_hi) and [br_lo, br_hi)
+        if (q < a.K) {
+            main_hi = q + 1;
+            br_lo = br_hi = 0;
+            dep = q;
+        } else {
+            const int s = (q - a.K) / a.branch_len, o = (q - a.K) - s * a.branch_len;
+            int d = 0;  // depth of slot s
+#pragma unroll
+            for (int i = 1; i <= ACES_MAX_K; ++i) d += i <= a.K && a.off[i] <= s;
+            main_hi = d;
+            br_lo = a.K + s * a.branch_len;
+            br_hi = q + 1;
+            dep = d + o;
+        }
+        uint32_t *out = a.mask + (size_t)q * a.words;
+        for (int w = lane; w < a.words; w += 32) out[w] = interval_bits(0, main_hi, w * 32) | interval_bits(br_lo, br_hi, w * 32);
+        if (lane == 0) a.depth[q] = dep;
     }
-    const int w0 = w * 32;
-    a.mask[i] = interval_bits(0, main_hi, w0) | interval_bits(br_lo, br_hi, w0);
-    if (w == 0) a.depth[q] = dep;
 }
 
 cudaError_t launch_tree_mask(const int *off, int K, int branch_len, int n, int words, uint32_t *mask,
@@ -63,8 +69,7 @@ cudaError_t launch_tree_mask(const int *off, int K, int branch_len, int n, int w
     for (int d = 0; d <= K; ++d) a.off[d] = off[d];
     a.mask = mask;
     a.depth = depth;
-    const long long tot = (long long)n * words;
-    k_tree_mask<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(a);
+    k_tree_mask<<<(unsigned)((n + NTM / 32 - 1) / (NTM / 32)), NTM, 0, s>>>(a);
     return cudaGetLastError();
 }
 
