@@ -227,8 +227,7 @@ static aces_status cache_prepare(CacheArgs &c, const float *draft_probs, const i
 
 static aces_status cache_launch(const CacheArgs &c, cudaStream_t s) {
     if (c.total == 0) return ACES_OK;
-    const bool vec = aligned16(c.q) && c.V % 4 == 0;
-    return launch_cache_build(c, vec, s) == cudaSuccess ? ACES_OK : ACES_ERR_CUDA;
+    return launch_cache_build(c, sm_count(), s) == cudaSuccess ? ACES_OK : ACES_ERR_CUDA;
 }
 
 // The library's side stream of the current device, with a fork and a join
