@@ -337,9 +337,8 @@ aces_status aces_resample_sparse(const int32_t *accept_len, const int32_t *topk_
     if (!accept_len || !topk_ids || !topk_probs || !tail_mass || !row_status || !draft_probs || !uniforms ||
         !token || !status)
         return ACES_ERR_INVALID_ARG;
-    const bool vec = aligned16(draft_probs) && V % 4 == 0;
     if (launch_resample_sparse(accept_len, topk_ids, topk_probs, tail_mass, row_status, draft_probs, uniforms, B,
-                               K, V, k, token, status, vec, reinterpret_cast<cudaStream_t>(stream)) !=
+                               K, V, k, token, status, reinterpret_cast<cudaStream_t>(stream)) !=
         cudaSuccess)
         return ACES_ERR_CUDA;
     return ACES_OK;

@@ -17,7 +17,7 @@
 #include <cooperative_groups.h>
 
 #define ACES_FILE 3  // site numbers of the checked build
-#include "common.cuh"
+#include "qrow.cuh"
 
 namespace aces {
 
@@ -28,28 +28,6 @@ constexpr int CCAP = 4096; // candidates kept per row
 constexpr int CCL = 8;     // CTAs of a row's cluster, at most
 constexpr int TOPL = 8;    // per-thread list of the repeated passes
 constexpr int RANK_MAX = 512;  // candidates ordered by direct ranking (more: bitonic sort)
-
-// A draft row in 16-byte chunks: element e of chunk c is id c * 4 + e - head
-// (rows off the 16-byte grid start inside chunk 0); 0 outside the row.
-struct QChunks {
-    const float *base;
-    int head, V, nch;
-    __device__ __forceinline__ QChunks(const float *row, int V_) : V(V_) {
-        head = (int)((uintptr_t)row & 15u) >> 2;
-        base = row - head;
-        nch = (V + head + 3) >> 2;
-    }
-    static __device__ __noinline__ uint4 edge(const float *row, int V, int x0) {
-        uint32_t v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = x0 + e >= 0 && x0 + e < V ? __float_as_uint(__ldg(row + x0 + e)) : 0u;
-        return make_uint4(v[0], v[1], v[2], v[3]);
-    }
-    __device__ __forceinline__ uint4 load(int c) const {
-        if (c * 4 >= head && c * 4 + 4 <= V + head) return ldg16(base + (size_t)c * 4);
-        return edge(base + head, V, c * 4 - head);
-    }
-};
 
 __device__ __forceinline__ void list_insert(unsigned long long (&Lst)[TOPL], unsigned long long o) {
     Lst[TOPL - 1] = o;

@@ -547,7 +547,7 @@ cudaError_t launch_compact_kv(void *kv, int planes, int B, int H, int S, size_t 
 cudaError_t launch_resample_sparse(const int32_t *accept_len, const int32_t *ids, const float *probs,
                                    const float *tail, const int32_t *row_status, const float *q,
                                    const float *u, int B, int K, int V, int k, int32_t *token,
-                                   int32_t *status, bool vec, cudaStream_t s);
+                                   int32_t *status, cudaStream_t s);
 cudaError_t launch_cache_lookup(const int32_t *bt, const CacheArgs &a, const int32_t *accept_len,
                                 const int32_t *token, int32_t *slot, cudaStream_t s);
 

@@ -11,31 +11,34 @@
 // uses p^_I alone.  When the nucleus of row pi fits in the payload, tau = 0
 // and the draw is the exact residual draw of aces_verify.
 //
-// One thread-block cluster of 8 CTAs (256 threads each) per sequence:
+// One thread-block cluster of 8 CTAs (512 threads each) per sequence:
 //   1. the payload of row pi is ordered by id in shared memory (direct rank
 //      counting), and its weights (p^ - q on I) are gathered;
-//   2. only when tau > 0, the 8 CTAs split q_pi's 2048-id tiles: one pass
+//   2. only when tau > 0, the 8 CTAs split q_pi's 16-byte chunks: one pass
 //      gives each CTA's share of q_rest (compensated fp32), combined through
 //      distributed shared memory; once the spread factor is known a second
-//      pass gives the weight of every tile (four tiles' loads in flight per
-//      thread), and the CTA holding the draw rescans its tile.  Otherwise
-//      the first CTA draws alone and the others exit at once;
+//      pass (from L2) gives the weight of every task of whole warp steps, and
+//      the CTA holding the draw scans its task with one warp.  A bit per
+//      chunk says whether it holds payload ids: nearly none does, and the
+//      others need no look at the payload (a merge of every id with the
+//      sorted payload took 45 us on 32 rows of 152064 with k = 32).
+//      Otherwise the first CTA draws alone and the others exit at once;
 //   3. the draw: smallest id j whose prefix sum exceeds floor(u * R), with
 //      every weight an integer in units of 2^-52 (exact, order independent).
 #include <cooperative_groups.h>
 
 #define ACES_FILE 7  // site numbers of the checked build
-#include "common.cuh"
+#include "qrow.cuh"
 
 namespace aces {
 
-constexpr int NTS = 256;
-constexpr int SEPT = 8;                // consecutive ids per thread
-constexpr int STILE = NTS * SEPT;      // ids per tile
+constexpr int NTS = 512;
+constexpr int NWS = NTS / 32;
 constexpr int SPAY = ACES_MAX_TOPK;    // payload entries
-constexpr int STILES = (ACES_MAX_V + STILE - 1) / STILE;
-constexpr int TPI = 4;                 // tiles per round of the q passes
 constexpr int SCL = 8;                 // CTAs per sequence: one thread-block cluster
+constexpr int SU = 4;                  // warp steps (32 chunks) in flight
+constexpr int SSTEPS = (ACES_MAX_V / 4 + 1 + 32 * SCL - 1) / (32 * SCL);  // warp steps of a CTA, at most
+constexpr int STASKS = NTS;            // tasks of a CTA, at most
 
 // floor(x * 2^52) of a float x in [0, 2^11) from its bits (0 for x <= 0 or NaN)
 __device__ __forceinline__ unsigned long long to_fx52(float x) {
@@ -66,37 +69,27 @@ __device__ __forceinline__ int lower_bound_id(const int *sid, int n, int x) {
     return lo;
 }
 
-// q at ids [x0, x0 + SEPT) (0 past V)
-template <bool VEC>
-__device__ __forceinline__ void load_q(const float *qr, int V, int x0, float (&qv)[SEPT]) {
-    if (VEC && x0 + SEPT <= V) {
-        const uint4 w0 = ldg16(qr + x0), w1 = ldg16(qr + x0 + 4);
-        qv[0] = __uint_as_float(w0.x); qv[1] = __uint_as_float(w0.y);
-        qv[2] = __uint_as_float(w0.z); qv[3] = __uint_as_float(w0.w);
-        qv[4] = __uint_as_float(w1.x); qv[5] = __uint_as_float(w1.y);
-        qv[6] = __uint_as_float(w1.z); qv[7] = __uint_as_float(w1.w);
-    } else {
-#pragma unroll
-        for (int e = 0; e < SEPT; ++e) qv[e] = x0 + e < V ? __ldg(qr + x0 + e) : 0.0f;
-    }
-}
+// What a CTA shares with its cluster.
+struct SparsePart {
+    unsigned long long w;  // weight of its slice
+    float ph, pl;          // its share of q_rest
+    int bad;
+};
 
-template <bool VEC>
 __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sparse(SparseArgs a) {
     namespace cg = cooperative_groups;
     __shared__ unsigned long long skey[SPAY];  // id << 32 | entry (all ones: invalid id)
     __shared__ int sid[SPAY];                  // valid payload ids, ascending
     __shared__ int sidx[SPAY];                 // their payload entries
     __shared__ unsigned long long sw[SPAY];    // their weights (2^-52 units)
-    __shared__ unsigned long long tsum[(STILES + SCL - 1) / SCL];  // this CTA's tiles
-    __shared__ unsigned long long red[NTS / 32];
-    __shared__ unsigned long long red4[TPI][NTS / 32];
-    __shared__ float redh[NTS / 32], redl[NTS / 32];
-    __shared__ float s_ph, s_pl;               // this CTA's share of q_rest (read by the cluster)
-    __shared__ int s_pbad;
-    __shared__ int s_n, s_bad, s_tok, s_tile;
+    __shared__ uint32_t held[SSTEPS];          // bit l of word k: chunk l of warp step k holds a payload id
+    __shared__ unsigned long long tsum[STASKS];  // this CTA's tasks
+    __shared__ unsigned long long red[NWS];
+    __shared__ float redh[NWS], redl[NWS];
+    __shared__ SparsePart part, parts[SCL];
+    __shared__ int s_n, s_bad, s_tok, s_task;
     __shared__ float s_gam;
-    __shared__ unsigned long long s_thr, s_base, s_R;
+    __shared__ unsigned long long s_base;
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int b = blockIdx.x / SCL, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -121,6 +114,11 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
     const int32_t *I = a.ids + row * a.k;
     const float *P = a.probs + row * a.k;
     const int V = a.V;
+    // this CTA's chunks of q_pi: nstep warp steps of 32 from chunk c_lo
+    const QChunks qc(qr != nullptr ? qr : a.q, V);
+    const int nws = (qc.nch + 31) / 32, pw = (nws + SCL - 1) / SCL;
+    const int w_lo = min(nws, rank * pw), nstep = min(nws, w_lo + pw) - w_lo;
+    const int c_lo = w_lo * 32;
 
     // ---- 1. payload sorted by id, weights on it ----
     // The valid entries (0 <= id < V) are ordered by (id, entry) by direct
@@ -129,7 +127,7 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
         s_n = 0;
         s_bad = 0;
         s_tok = -1;
-        s_tile = -1;
+        s_task = -1;
         s_gam = 0.0f;
     }
     for (int j = tid; j < a.k; j += NTS) {
@@ -138,31 +136,34 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
         if (x >= 0 && x < V) key = ((unsigned long long)x << 32) | (unsigned long long)j;
         skey[j] = key;
     }
+    if (cluster_work)
+        for (int i = tid; i < nstep; i += NTS)
+            if (ACES_IN(i, SSTEPS)) held[i] = 0u;
     __syncthreads();
     for (int j = tid; j < a.k; j += NTS) {
         const unsigned long long key = skey[j];
         if (key == ~0ull) continue;
-        int rank = 0;
-        for (int i = 0; i < a.k; ++i) rank += skey[i] < key;
-        if (ACES_IN(rank, SPAY)) {
-            sid[rank] = (int)(key >> 32);
-            sidx[rank] = (int)(key & 0xFFFFFFFFull);
-        }
-        atomicAdd(&s_n, 1);
-    }
-    __syncthreads();
-    const int n = s_n;
-    for (int i = tid; i < n; i += NTS) {
-        const int x = sid[i], j = sidx[i];
-        float w = fmaxf(P[j], 0.0f);
+        int rk = 0;
+#pragma unroll 8
+        for (int i = 0; i < a.k; ++i) rk += skey[i] < key;
+        const int x = (int)(key >> 32), e = (int)(key & 0xFFFFFFFFull);
+        float w = fmaxf(P[e], 0.0f);
         if (qr && ACES_IN(x, V)) {
             const float qx = __ldg(qr + x);
             if (!(qx >= 0.0f)) s_bad = 1;
-            w = fmaxf(P[j] - qx, 0.0f);
+            w = fmaxf(P[e] - qx, 0.0f);
         }
-        sw[i] = to_fx52(w);
+        if (ACES_IN(rk, SPAY)) {
+            sid[rk] = x;
+            sidx[rk] = e;
+            sw[rk] = to_fx52(w);
+        }
+        atomicAdd(&s_n, 1);
+        const int c = ((x + qc.head) >> 2) - c_lo;
+        if (cluster_work && c >= 0 && c < nstep * 32 && ACES_IN(c >> 5, SSTEPS)) atomicOr(&held[c >> 5], 1u << (c & 31));
     }
     __syncthreads();
+    const int n = s_n;
     if (s_bad || n == 0) {  // the same in every CTA of the cluster
         if (rank == 0 && tid == 0) {
             a.token[b] = -1;
@@ -170,39 +171,50 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
         }
         return;
     }
+    // the chunk of this lane in warp step k (0 outside the row)
+    auto load = [&](int k) {
+        const int c = c_lo + k * 32 + lane;
+        return k < nstep && c < qc.nch ? qc.load(c) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    auto first_id = [&](int k) { return (c_lo + k * 32 + lane) * 4 - qc.head; };
+    // the payload entry of id x, -1 when there is none
+    auto entry_of = [&](int x) {
+        const int j = lower_bound_id(sid, n, x);
+        return j < n && sid[j] == x ? j : -1;
+    };
 
     // ---- 2. the tail, spread like the draft (pi < K, tau > 0): the cluster ----
-    const int ntile = (V + STILE - 1) / STILE;  // 2048-id tiles
-    const int per = (ntile + SCL - 1) / SCL;     // tiles of each CTA
-    const int t_lo = rank * per < ntile ? rank * per : ntile;
-    const int t_hi = t_lo + per < ntile ? t_lo + per : ntile;
+    const int spt = (pw + STASKS - 1) / STASKS;  // warp steps per task
+    const int ntask = (nstep + spt - 1) / spt;
     bool spread = false;
+    float gam = 0.0f;
+    unsigned long long thr = 0ull;
     if (cluster_work) {
         float hi = 0.0f, lo = 0.0f;  // compensated sum of q outside the payload
         int bad = 0;
-        for (int t0 = t_lo; t0 < t_hi; t0 += TPI) {  // TPI tiles' loads in flight
-            float qv[TPI][SEPT];
+        for (int k0 = wid; k0 < nstep; k0 += NWS * SU) {
+            uint4 v[SU];
 #pragma unroll
-            for (int h = 0; h < TPI; ++h) {
-                const int x0 = (t0 + h) * STILE + tid * SEPT;
-                if (t0 + h < t_hi && x0 < V) load_q<VEC>(qr, V, x0, qv[h]);
-            }
+            for (int i = 0; i < SU; ++i) v[i] = load(k0 + i * NWS);
 #pragma unroll
-            for (int h = 0; h < TPI; ++h) {
-                const int x0 = (t0 + h) * STILE + tid * SEPT;
-                if (t0 + h >= t_hi || x0 >= V) break;
-                int j = lower_bound_id(sid, n, x0);
+            for (int i = 0; i < SU; ++i) {
+                const int k = k0 + i * NWS;
+                if (k >= nstep) break;
+                float q[4];
 #pragma unroll
-                for (int e = 0; e < SEPT; ++e) {
-                    const int x = x0 + e;
-                    if (x >= V) break;
-                    const float qx = qv[h][e];
-                    if (!(qx >= 0.0f)) bad = 1;
-                    while (j < n && sid[j] < x) ++j;
-                    if (j < n && sid[j] == x) continue;
-                    const float t = hi + qx;
-                    if (fabsf(hi) >= fabsf(qx)) lo += (hi - t) + qx;
-                    else lo += (qx - t) + hi;
+                for (int e = 0; e < 4; ++e) {
+                    q[e] = Elem<ACES_F32>::get(v[i], e);
+                    if (!(q[e] >= 0.0f)) bad = 1;
+                }
+                if ((held[k] >> lane) & 1u) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (entry_of(first_id(k) + e) >= 0) q[e] = 0.0f;
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {  // two-sum
+                    const float t = hi + q[e], bb = t - hi;
+                    lo += (hi - (t - bb)) + (q[e] - bb);
                     hi = t;
                 }
             }
@@ -220,26 +232,29 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
             redh[wid] = hi;
             redl[wid] = lo;
         }
+        for (int i = tid; i < ntask; i += NTS) tsum[i] = 0ull;
         __syncthreads();
         if (tid == 0) {
             float h = 0.0f, l = 0.0f;
-            for (int i = 0; i < NTS / 32; ++i) {
+            for (int i = 0; i < NWS; ++i) {
                 const float sm = h + redh[i];
                 const float bb = sm - h;
                 l = l + redl[i] + ((h - (sm - bb)) + (redh[i] - bb));
                 h = sm;
             }
-            s_ph = h;
-            s_pl = l;
-            s_pbad = s_bad;
+            part.ph = h;
+            part.pl = l;
+            part.bad = s_bad;
         }
         cl.sync();  // every CTA's share is written
+        if (tid < SCL) parts[tid] = *cl.map_shared_rank(&part, tid);
+        __syncthreads();
         if (tid == 0) {  // every CTA sums the shares in rank order: the same value everywhere
             double qrest = 0.0;
             int anybad = 0;
             for (int j = 0; j < SCL; ++j) {
-                qrest += (double)*cl.map_shared_rank(&s_ph, j) + (double)*cl.map_shared_rank(&s_pl, j);
-                anybad |= *cl.map_shared_rank(&s_pbad, j);
+                qrest += (double)parts[j].ph + (double)parts[j].pl;
+                anybad |= parts[j].bad;
             }
             const double g = qrest > 0.0 ? (double)tau / qrest - 1.0 : 0.0;
             s_gam = g > 0.0 ? (float)g : 0.0f;
@@ -253,122 +268,93 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
             }
             return;
         }
-        spread = s_gam > 0.0f;
+        gam = s_gam;
+        spread = gam > 0.0f;
         if (!spread && rank != 0) return;
     }
+    // the weights of a chunk's ids: q * gam outside the payload, sw on it
+    auto weights = [&](int k, const uint4 &v, unsigned long long (&w)[4]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[e] = to_fx52(Elem<ACES_F32>::get(v, e) * gam);
+        if ((held[k] >> lane) & 1u) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = entry_of(first_id(k) + e);
+                if (j >= 0) w[e] = sw[j];
+            }
+        }
+    };
 
     // ---- 3. the draw ----
     if (spread) {
-        const float gam = s_gam;
-        // weight of each of this CTA's tiles: q * gam outside the payload, sw on it
-        for (int t0 = t_lo; t0 < t_hi; t0 += TPI) {
-            float qv[TPI][SEPT];
+        for (int k0 = wid; k0 < nstep; k0 += NWS * SU) {
+            uint4 v[SU];
 #pragma unroll
-            for (int h = 0; h < TPI; ++h) {
-                const int x0 = (t0 + h) * STILE + tid * SEPT;
-                if (t0 + h < t_hi && x0 < V) load_q<VEC>(qr, V, x0, qv[h]);
-            }
-            unsigned long long loc[TPI];
+            for (int i = 0; i < SU; ++i) v[i] = load(k0 + i * NWS);
 #pragma unroll
-            for (int h = 0; h < TPI; ++h) {
-                const int x0 = (t0 + h) * STILE + tid * SEPT;
-                loc[h] = 0ull;
-                if (t0 + h >= t_hi || x0 >= V) continue;
-                int j = lower_bound_id(sid, n, x0);
-#pragma unroll
-                for (int e = 0; e < SEPT; ++e) {
-                    const int x = x0 + e;
-                    if (x >= V) break;
-                    while (j < n && sid[j] < x) ++j;
-                    loc[h] += (j < n && sid[j] == x) ? sw[j] : to_fx52(qv[h][e] * gam);
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < TPI; ++h) loc[h] = warp_sum(loc[h]);
-            if (lane == 0)
-#pragma unroll
-                for (int h = 0; h < TPI; ++h) red4[h][wid] = loc[h];
-            __syncthreads();
-            if (tid < TPI && t0 + tid < t_hi) {
-                unsigned long long ts = 0ull;
-                for (int i = 0; i < NTS / 32; ++i) ts += red4[tid][i];
-                tsum[t0 + tid - t_lo] = ts;
-            }
-            __syncthreads();
-        }
-        cl.sync();  // every CTA's tile weights are written
-        if (tid == 0) {  // the same walk over all tiles in every CTA
-            unsigned long long tot = 0ull;
-            for (int j = 0; j < SCL; ++j) {
-                const int lo_j = j * per < ntile ? j * per : ntile;
-                const int hi_j = lo_j + per < ntile ? lo_j + per : ntile;
-                const unsigned long long *rt = cl.map_shared_rank(tsum, j);
-                for (int t = lo_j; t < hi_j; ++t) tot += rt[t - lo_j];
-            }
-            s_R = tot;
-            s_tile = -1;
-            if (tot > 0ull) {
-                const unsigned long long thr = floor_u_times(a.u[(size_t)b * R1 + a.K], tot);
-                unsigned long long base = 0ull;
-                int tt = ntile - 1;
-                bool found = false;
-                for (int j = 0; j < SCL && !found; ++j) {
-                    const int lo_j = j * per < ntile ? j * per : ntile;
-                    const int hi_j = lo_j + per < ntile ? lo_j + per : ntile;
-                    const unsigned long long *rt = cl.map_shared_rank(tsum, j);
-                    for (int t = lo_j; t < hi_j; ++t) {
-                        if (base + rt[t - lo_j] > thr) {
-                            tt = t;
-                            found = true;
-                            break;
-                        }
-                        base += rt[t - lo_j];
-                    }
-                }
-                if (tt >= t_lo && tt < t_hi) s_tile = tt;
-                s_base = base;
-                s_thr = thr;
+            for (int i = 0; i < SU; ++i) {
+                const int k = k0 + i * NWS;
+                if (k >= nstep) break;  // (warp-uniform)
+                unsigned long long w[4];
+                weights(k, v[i], w);
+                const unsigned long long ws = warp_sum((w[0] + w[1]) + (w[2] + w[3]));
+                if (lane == 0 && ACES_IN(k / spt, STASKS)) atomicAdd(&tsum[k / spt], ws);
             }
         }
-        cl.sync();  // the tile weights are read before any CTA exits
-        if (s_R == 0ull) {  // nothing above 2^-52: rank 0 draws on the payload
+        __syncthreads();
+        const unsigned long long own = tid < ntask ? tsum[tid] : 0ull;
+        unsigned long long tot;
+        const unsigned long long ex = block_exscan_n<NTS>(own, red, &tot);
+        if (tid == 0) part.w = tot;
+        cl.sync();  // every CTA's weight is written
+        if (tid < SCL) parts[tid].w = cl.map_shared_rank(&part, tid)->w;
+        __syncthreads();
+        unsigned long long R = 0ull, before = 0ull;
+        for (int j = 0; j < SCL; ++j) {
+            if (j == rank) before = R;
+            R += parts[j].w;
+        }
+        cl.sync();  // the weights are read before any CTA exits
+        if (R == 0ull) {  // nothing above 2^-52: rank 0 draws on the payload
             spread = false;
             if (rank != 0) return;
-        } else if (s_tile < 0) {
-            return;  // another CTA holds the draw
+        } else {
+            thr = floor_u_times(a.u[(size_t)b * R1 + a.K], R);
+            if (!(before <= thr && thr < before + tot)) return;  // another CTA holds the draw
+            if (before + ex <= thr && thr < before + ex + own) {  // (one thread)
+                s_task = tid;
+                s_base = before + ex;
+            }
+            __syncthreads();
         }
     }
     if (spread) {
-        const float gam = s_gam;
-        // rescan the tile holding the draw
-        const int x0 = s_tile * STILE + tid * SEPT;
-        unsigned long long wv[SEPT];
-        unsigned long long loc = 0ull;
-        float qv[SEPT];
-        if (x0 < V) load_q<VEC>(qr, V, x0, qv);
-        int j = x0 < V ? lower_bound_id(sid, n, x0) : n;
-#pragma unroll
-        for (int e = 0; e < SEPT; ++e) {
-            const int x = x0 + e;
-            wv[e] = 0ull;
-            if (x < V) {
-                while (j < n && sid[j] < x) ++j;
-                wv[e] = (j < n && sid[j] == x) ? sw[j] : to_fx52(qv[e] * gam);
-            }
-            loc += wv[e];
-        }
-        unsigned long long tot;
-        const unsigned long long ex = block_exscan_n<NTS>(loc, red, &tot);
-        const unsigned long long thr = s_thr;
-        unsigned long long c = s_base + ex;
-        if (c <= thr && thr < c + loc) {
-#pragma unroll
-            for (int e = 0; e < SEPT; ++e) {
-                c += wv[e];
-                if (c > thr) {
-                    s_tok = x0 + e;
-                    break;
+        // one warp scans the task holding the draw
+        if (wid == 0) {
+            unsigned long long base = s_base;
+            for (int k = s_task * spt; k < min(nstep, (s_task + 1) * spt); ++k) {
+                unsigned long long w[4];
+                weights(k, load(k), w);
+                const unsigned long long loc = (w[0] + w[1]) + (w[2] + w[3]);
+                unsigned long long inc = loc;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += t;
                 }
+                unsigned long long c = base + inc - loc;
+                const bool mine = c <= thr && thr < c + loc;
+                if (mine) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        c += w[e];
+                        if (c > thr) {
+                            s_tok = first_id(k) + e;
+                            break;
+                        }
+                    }
+                }
+                if (__any_sync(0xffffffffu, mine)) break;
+                base += __shfl_sync(0xffffffffu, inc, 31);
             }
         }
         __syncthreads();
@@ -385,8 +371,8 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
             ex = block_exscan_n<NTS>(w, red, &tot);
         }
         if (tot > 0ull) {
-            const unsigned long long thr = floor_u_times(a.u[(size_t)b * R1 + a.K], tot);
-            if (ex <= thr && thr < ex + w) s_tok = sid[tid];
+            const unsigned long long t2 = floor_u_times(a.u[(size_t)b * R1 + a.K], tot);
+            if (ex <= t2 && t2 < ex + w) s_tok = sid[tid];
         }
         __syncthreads();
     }
@@ -399,7 +385,7 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
 cudaError_t launch_resample_sparse(const int32_t *accept_len, const int32_t *ids, const float *probs,
                                    const float *tail, const int32_t *row_status, const float *q,
                                    const float *u, int B, int K, int V, int k, int32_t *token,
-                                   int32_t *status, bool vec, cudaStream_t s) {
+                                   int32_t *status, cudaStream_t s) {
     SparseArgs a;
     a.accept_len = accept_len;
     a.ids = ids;
@@ -414,8 +400,7 @@ cudaError_t launch_resample_sparse(const int32_t *accept_len, const int32_t *ids
     a.k = k;
     a.token = token;
     a.status = status;
-    if (vec) k_resample_sparse<true><<<B * SCL, NTS, 0, s>>>(a);
-    else k_resample_sparse<false><<<B * SCL, NTS, 0, s>>>(a);
+    k_resample_sparse<<<B * SCL, NTS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
