@@ -56,7 +56,7 @@ aces_status run_rows(RowArgs &a, aces_dtype dt, bool exact, cudaStream_t s) {
     rows_cap_layout(a, dt, !vec);
     a.force_fb = exact ? 1 : 0;
     if (launch_rows_cap(a, dt, !vec, s) != cudaSuccess) return ACES_ERR_CUDA;
-    if (launch_rows_general(a, dt, vec, nseq, s) != cudaSuccess) return ACES_ERR_CUDA;
+    if (launch_rows_general(a, dt, nseq, s) != cudaSuccess) return ACES_ERR_CUDA;
     return ACES_OK;
 }
 

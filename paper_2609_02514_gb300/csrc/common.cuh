@@ -527,7 +527,7 @@ __device__ void nonfinite_row(const RowArgs &a, int r) {
 // host launchers (defined next to their kernels)
 void rows_cap_layout(RowArgs &a, int dt, bool ragged);
 cudaError_t launch_rows_cap(const RowArgs &a, int dt, bool ragged, cudaStream_t s);
-cudaError_t launch_rows_general(const RowArgs &a, int dt, bool vec, int nseq, cudaStream_t s);
+cudaError_t launch_rows_general(const RowArgs &a, int dt, int nseq, cudaStream_t s);
 // aces_verify with two choices, neither of which changes the results: lists =
 // false keeps no nucleus lists (the residual draw scans its row; the call then
 // needs ws_bytes(rows, B, K, lists) bytes of workspace), exact = true hands

@@ -13,14 +13,13 @@
 //                 at those ids only, they are ordered by id, and the draw is
 //                 taken from their prefix sums.  Run by the CTA that finishes
 //                 the sequence's last row.
-//   draw_cluster  the other sequences the single-pass kernel finished (it
-//                 lists them): a cluster of CTAs sums the residual of 32-chunk
+//   draw_cluster  the other sequences: a cluster of CTAs sums the residual of 32-chunk
 //                 tasks of row pi (q is read where a chunk holds a nucleus
 //                 id), then one warp scans the task holding the draw.  Run by
-//                 the general kernel once its rows are done.
-//   draw_scan     sequences whose last row the general kernel finished, and
-//                 those whose residual is zero everywhere: one CTA, the same
-//                 with more sums (p as well) and a loop over the members.
+//                 the general kernel once its rows are done, and for the
+//                 sequences that they complete.
+//   draw_scan     sequences whose residual is zero everywhere: one CTA, the
+//                 same with more sums (p as well) and a loop over the members.
 // When row pi kept its cut as (value v, count j) (RS_LAZY: the nucleus ends
 // among the ids of one bfloat16 value, which the row kernel did not list), the
 // ids of value v are summed and counted apart, and the task holding the j-th
@@ -53,6 +52,7 @@ struct RowChunks {
         base = row - head * Elem<DT>::SIZE;
         nch = (V + head + EPC - 1) / EPC;
     }
+    __device__ __forceinline__ const char *row() const { return base + head * Elem<DT>::SIZE; }
     __device__ __forceinline__ bool whole(int c) const { return !RAGGED || (c * EPC >= head && (c + 1) * EPC <= V + head); }
     // the elements from id x0 on, one by one (V: the row's length)
     static __device__ __noinline__ uint4 edge(const char *row, int V, int x0) {
@@ -85,6 +85,18 @@ struct ScanRow {
     float c, kref, inv_S, u;
     unsigned long long cut;
 };
+
+// a row's state, perhaps written by another CTA of this kernel
+__device__ __forceinline__ RowStat row_stat(const Workspace &ws, int r) {
+    union {
+        uint4 w[2];
+        RowStat rs;
+    } v;
+    const uint4 *p = reinterpret_cast<const uint4 *>(ws.stats + r);
+    v.w[0] = __ldcg(p);
+    v.w[1] = __ldcg(p + 1);
+    return v.rs;
+}
 
 template <int DT>
 __device__ __forceinline__ ScanRow scan_row(const RowArgs &a, int b, int pi, const RowStat &rs) {
@@ -489,6 +501,7 @@ struct DrawPart {
     unsigned long long tcut;  // of that value's ids inside the nucleus (the CTA holding the cut)
     uint32_t nt;              // ids of that value
     int bad;                  // an invalid q was seen
+    int pend;                 // (general kernel) a sequence this CTA completed, left to the cluster
 };
 
 // The draw of sequence b from row pi by a cluster of up to DRAW_CL CTAs (all
@@ -518,7 +531,7 @@ __device__ __noinline__ void draw_cluster(const RowArgs &a, int b, int pi, DrawP
     if (tid == 0) sh->bad = 0;
     __syncthreads();
     const int rp = b * (a.K + 1) + pi;
-    const RowStat rs = a.ws.stats[rp];  // (finite: rows that are not are drawn where they finish)
+    const RowStat rs = row_stat(a.ws, rp);  // (finite: rows that are not are drawn where they finish)
     const ScanRow s = scan_row<DT>(a, b, pi, rs);
     const RowChunks<DT> rc(s.z, s.V);
     const bool qvec = s.q != nullptr && ((uintptr_t)(s.q - rc.head) & 15u) == 0;
@@ -886,39 +899,34 @@ __device__ int draw_list(const ScanRow &s, const unsigned long long *lst, int n,
 }
 
 // Called by all threads when this CTA has written row r's outputs and state.
-// The CTA that finishes the last row of a sequence draws its token; with
-// `defer` it lists the sequence for draw_cluster instead when row pi kept no
-// nucleus.
-template <int DT, int NTH, bool DEFER>
-__device__ void row_finished(const RowArgs &a, int r, unsigned char *scratch) {
-    if (a.ws.seqcnt == nullptr) return;  // sparsify
+// The CTA that finishes the last row of a sequence draws its token when row
+// pi kept its nucleus; otherwise it gets b * 32 + pi, for draw_cluster (the
+// others, and those that have drawn, get -1).
+template <int DT, int NTH>
+__device__ int row_finished(const RowArgs &a, int r, unsigned char *scratch) {
+    if (a.ws.seqcnt == nullptr) return -1;  // sparsify
     __shared__ int s_last, s_pi;
     const int b = r / (a.K + 1);
     __syncthreads();  // every thread's writes of this row are issued
     // releases this row's writes; the last row acquires the others'
     if (threadIdx.x == 0) s_last = atomic_add_acq_rel(&a.ws.seqcnt[b], 1) == a.K;
     __syncthreads();
-    if (!s_last) return;
+    if (!s_last) return -1;
     if (threadIdx.x < 32) {
         const int pi0 = first_reject_warp(a.ws, b, a.K);
         if (threadIdx.x == 0) s_pi = pi0;
     }
     __syncthreads();
     const int pi = s_pi, rp = b * (a.K + 1) + pi;
-    const RowStat rs = a.ws.stats[rp];
+    const RowStat rs = row_stat(a.ws, rp);
     int tok = -1;
     if (!(rs.flags & RS_NONFINITE)) {
-        if (DEFER && rs.nnuc < 0) {
-            if (threadIdx.x == 0) a.ws.scan_list[atomicAdd(&a.ws.fb_count[13], 1)] = b * 32 + pi;
-            return;
-        }
+        if (rs.nnuc < 0) return b * 32 + pi;
         const ScanRow s = scan_row<DT>(a, b, pi, rs);
-        if (rs.nnuc >= 0)
-            tok = draw_list<NTH>(s, a.ws.nuc + (size_t)rp * NUC_CAP, ACES_IN(rs.nnuc - 1, NUC_CAP) ? rs.nnuc : 0, scratch);
-        else if constexpr (!DEFER)
-            tok = draw_scan<DT, NTH>(s, scratch);
+        tok = draw_list<NTH>(s, a.ws.nuc + (size_t)rp * NUC_CAP, ACES_IN(rs.nnuc - 1, NUC_CAP) ? rs.nnuc : 0, scratch);
     }
     if (threadIdx.x == 0) write_draw(a, b, pi, tok);
+    return -1;
 }
 
 }  // namespace aces

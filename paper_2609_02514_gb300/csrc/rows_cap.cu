@@ -296,6 +296,11 @@ __device__ __forceinline__ void fallback_row(const RowArgs &a, int r, float m, f
     a.ws.fb_list[pos] = r;
 }
 
+// lists a sequence for the general kernel's draw (e: row_finished's)
+__device__ __forceinline__ void defer_draw(const RowArgs &a, int e) {
+    if (e >= 0 && threadIdx.x == 0) a.ws.scan_list[atomicAdd(&a.ws.fb_count[13], 1)] = e;
+}
+
 // appends o to arr[*n] for every lane with take (one atomic per warp); *n
 // may pass cap, entries beyond it are dropped (all lanes of the warp call it)
 __device__ __forceinline__ void append_cap(unsigned long long *arr, int *n, bool take, unsigned long long o, int cap) {
@@ -610,7 +615,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         if (!(sh > 0.0f && sh < INFINITY) || !(m < INFINITY) || !(kref < 1e30f)) {
             nonfinite_row<NTC>(a, r);
-            row_finished<DT, NTC, true>(a, r, smem);
+            defer_draw(a, row_finished<DT, NTC>(a, r, smem));
             return true;
         }
         return false;
@@ -1215,6 +1220,8 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         // chunk position that has any; the ids are extracted after the stream
         auto record_hits = [&](float th) {
             if (!__any_sync(0xffffffffu, im >= th)) return;
+            // (past the capacity the row goes to the general kernel)
+            if (*reinterpret_cast<volatile int *>(&s_nrec) > CREC) return;
             uint32_t off = off0;
 #pragma unroll
             for (int u = 0; u < UC; ++u) {
@@ -1561,7 +1568,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         rs.nnuc = nnuc;
         a.ws.stats[r] = rs;
     }
-    row_finished<DT, NTC, true>(a, r, smem);
+    defer_draw(a, row_finished<DT, NTC>(a, r, smem));
 }
 
 static int gcd_int(int x, int y) {

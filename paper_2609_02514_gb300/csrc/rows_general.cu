@@ -4,9 +4,12 @@
 // needs a whole row.  Masses are in 2^-40 fixed point, so every partial sum
 // is exact and order-independent.  One CTA of 512 threads per row; a
 // persistent grid walks the list of rows handed over.
-//   value histogram  (aligned bfloat16 rows) ids counted per bfloat16 value
+//   value histogram  (bfloat16 rows) ids counted per bfloat16 value
 //                below the max, the crossing and payload values found by a
 //                prefix scan, their ids collected and ranked: two row reads;
+//   depth histogram  (handed float32 rows, then bfloat16) ids counted in fine
+//                bins of depth, exact masses only above the crossing's range:
+//                two row reads;
 //   binned path  exact per-bin masses over bins of distance below the max
 //                (warp-aggregated shared-memory atomics, farther elements
 //                summed in registers), then the crossing bin and the payload
@@ -91,41 +94,30 @@ __device__ void finish_row(const RowArgs &a, int r, const char *row, float kref,
 // General path: exact radix selection over the 64-bit order value
 // O = key(z) << 32 | (2^32 - 1 - id), 8 bits per pass, masses in 2^-40
 // fixed point so that every partial sum is exact and order-independent.
-template <int DT, bool VEC, class F>
-__device__ __forceinline__ void for_each_elem(const char *row, int V, F f) {
-    using E = Elem<DT>;
-    if (VEC) {
-        const int nch = V / E::EPC;
+template <int DT, class F>
+__device__ __forceinline__ void for_each_elem(const RowChunks<DT> &rc, F f) {
+    constexpr int EPC = Elem<DT>::EPC;
 #pragma unroll 2
-        for (int cc = threadIdx.x; cc < nch; cc += NT) {
-            uint4 w = ldg16(row + (size_t)cc * 16);
+    for (int c = threadIdx.x; c < rc.nch; c += NT) {
+        const uint4 w = rc.load(c);
 #pragma unroll
-            for (int e = 0; e < E::EPC; ++e) f(cc * E::EPC + e, E::get(w, e));
-        }
-    } else {
-        for (int x = threadIdx.x; x < V; x += NT) f(x, E::load1(row, x));
+        for (int e = 0; e < EPC; ++e) f(c * EPC + e - rc.head, Elem<DT>::get(w, e));  // (-inf outside the row)
     }
 }
 
 // Warp-uniform walk over the row: every lane of a warp takes part in every
-// round (f gets valid = false past the end), so f may use warp collectives.
-template <int DT, bool VEC, class F>
-__device__ __forceinline__ void for_each_elem_warp(const char *row, int V, F f) {
-    using E = Elem<DT>;
-    if (VEC) {
-        const int nch = V / E::EPC;
-        for (int c0 = threadIdx.x & ~31; c0 < nch; c0 += NT) {
-            const int cc = c0 + (threadIdx.x & 31);
-            const bool in = cc < nch;
-            const uint4 w = in ? ldg16(row + (size_t)cc * 16) : make_uint4(0u, 0u, 0u, 0u);
+// round (f gets valid = false outside the row), so f may use warp collectives.
+template <int DT, class F>
+__device__ __forceinline__ void for_each_elem_warp(const RowChunks<DT> &rc, F f) {
+    constexpr int EPC = Elem<DT>::EPC;
+    for (int c0 = threadIdx.x & ~31; c0 < rc.nch; c0 += NT) {
+        const int c = c0 + (threadIdx.x & 31);
+        const bool in = c < rc.nch;
+        const uint4 w = in ? rc.load(c) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int e = 0; e < E::EPC; ++e) f(in, cc * E::EPC + e, E::get(w, e));
-        }
-    } else {
-        for (int x0 = threadIdx.x & ~31; x0 < V; x0 += NT) {
-            const int x = x0 + (threadIdx.x & 31);
-            const bool in = x < V;
-            f(in, x, in ? E::load1(row, x) : 0.0f);
+        for (int e = 0; e < EPC; ++e) {
+            const int x = c * EPC + e - rc.head;
+            f(in && x >= 0 && x < rc.V, x, Elem<DT>::get(w, e));
         }
     }
 }
@@ -167,8 +159,8 @@ struct SelState {
 // target_fx (as a double); mode 1: the kk-th id (1-based) by count.
 // Returns the order value of the selected id; st->above / above_cnt hold the
 // mass / count strictly before it; when want_S, st->S_fx gets the total mass.
-template <int DT, bool VEC>
-__device__ unsigned long long radix_select(const char *row, int V, float kref, float c, int mode,
+template <int DT>
+__device__ unsigned long long radix_select(const RowChunks<DT> &rc, float kref, float c, int mode,
                                            double target, unsigned kk, bool want_S, SelState *st) {
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -199,7 +191,7 @@ __device__ unsigned long long radix_select(const char *row, int V, float kref, f
         const unsigned long long prefix = st->prefix;
         const int sh = 64 - nbits;
         const bool with_mass = mode == 0 || want_S;
-        for_each_elem_warp<DT, VEC>(row, V, [&](bool in, int x, float v) {
+        for_each_elem_warp<DT>(rc, [&](bool in, int x, float v) {
             const unsigned long long o = order_val(fkey(v), (uint32_t)x);
             const bool ok = in && v > -INFINITY && (nbits == 0 || (o >> sh) == prefix);
             const int d = (int)((o >> s) & 255ull);
@@ -244,7 +236,7 @@ __device__ unsigned long long radix_select(const char *row, int V, float kref, f
             // a single id carries this prefix: fetch its full order value
             const unsigned long long pf = st->prefix;
             const int sh2 = 64 - nbits;
-            for_each_elem<DT, VEC>(row, V, [&](int x, float v) {
+            for_each_elem<DT>(rc, [&](int x, float v) {
                 if (!(v > -INFINITY)) return;
                 unsigned long long o = order_val(fkey(v), (uint32_t)x);
                 if ((o >> sh2) == pf) st->prefix = o;
@@ -293,11 +285,12 @@ __device__ __forceinline__ void warp_append(unsigned long long *arr, int *n, boo
     if (take && pos < GB_CAP) arr[pos] = o;
 }
 
-template <int DT, bool VEC>
-__device__ bool binned_row(const RowArgs &a, int r, const char *row, float m, float kref,
+template <int DT>
+__device__ bool binned_row(const RowArgs &a, int r, const RowChunks<DT> &rc, float m, float kref,
                            unsigned long long n_fin, BinState *bs, unsigned long long *buf, double *redd,
                            unsigned long long *redu) {
     const int tid = threadIdx.x;
+    const char *row = rc.row();
     const bool all_in = a.top_p >= 1.0f;
     // Two windows: the first pass histograms the GB_WIN bins nearest the max
     // with shared-memory atomics and only sums the farther elements in
@@ -319,7 +312,7 @@ __device__ bool binned_row(const RowArgs &a, int r, const char *row, float m, fl
         for (int i = tid; i < WN; i += NT) bs->mass[i] = 0ull;
         __syncthreads();
         unsigned long long far_cnt = 0ull, far_mass = 0ull;
-        for_each_elem_warp<DT, VEC>(row, a.V, [&](bool in, int, float v) {
+        for_each_elem_warp<DT>(rc, [&](bool in, int, float v) {
             const bool fin = in && v > -INFINITY;
             const float dd = (m - v) * a.inv_w;
             const int d = dd < (float)(NBIN - 1) ? (int)dd : NBIN - 1;
@@ -384,7 +377,7 @@ __device__ bool binned_row(const RowArgs &a, int r, const char *row, float m, fl
     __syncthreads();
     const int bx = bs->bx, bk = bs->bk;
     // collect the crossing bin and the payload bins
-    for_each_elem_warp<DT, VEC>(row, a.V, [&](bool in, int x, float v) {
+    for_each_elem_warp<DT>(rc, [&](bool in, int x, float v) {
         const bool fin = in && v > -INFINITY;
         const float dd = (m - v) * a.inv_w;
         const int d = dd < (float)(NBIN - 1) ? (int)dd : NBIN - 1;
@@ -513,17 +506,18 @@ __device__ __forceinline__ void warp_append_cap(unsigned long long *arr, int *n,
     if (take && pos < cap) arr[pos] = o;
 }
 
-// (aligned bfloat16 rows; all threads of the CTA)
+// (bfloat16 rows; all threads of the CTA)
 // S_in: the row's exp-sum in units of 2^kref for a row handed over by the
 // fast kernel, 0 otherwise.  *n_fin_out gets the row's count of finite ids
 // when top_p = 1 or S_in = 0 (its only uses), even when the row is declined.
-__device__ bool valhist_row(const RowArgs &a, int r, const char *row, float m, float kref, double S_in,
+__device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &rc, float m, float kref, double S_in,
                             unsigned long long *n_fin_out, ValHist *vh, unsigned long long *buf, double *redd,
                             unsigned long long *redu) {
     using E = Elem<ACES_BF16>;
     const int tid = threadIdx.x, lane = tid & 31;
     const bool all_in = a.top_p >= 1.0f;
     const bool have_S = S_in > 0.0;
+    const char *row = rc.row();
     const uint32_t km = bkey16(__float_as_uint(m) >> 16);  // m is a bfloat16 value
     for (int i = tid; i < VH_W; i += NT) vh->cnt[i] = 0u;
     if (tid == 0) {
@@ -555,8 +549,8 @@ __device__ bool valhist_row(const RowArgs &a, int r, const char *row, float m, f
     // compensated exp-sum where they are needed) ----
     float hi = 0.f, lo = 0.f;
     unsigned long long nfin = 0ull;
-    const int nch = a.V / E::EPC;
-    // (-inf words past the end count nowhere)
+    const int nch = rc.nch;
+    // (-inf words outside the row count nowhere)
     auto count_pass = [&](auto with_sum, auto with_nfin) {
         constexpr bool WS = decltype(with_sum)::value, WN = decltype(with_nfin)::value;
         for (int c0 = tid; c0 < nch; c0 += VH_U * NT) {
@@ -564,7 +558,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const char *row, float m, f
 #pragma unroll
             for (int u = 0; u < VH_U; ++u) {
                 const int cc = c0 + u * NT;
-                wu[u] = cc < nch ? ldg16(row + (size_t)cc * 16) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+                wu[u] = cc < nch ? rc.load(cc) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
             }
             float cs = 0.f;
             uint32_t nf = 0u;
@@ -666,12 +660,12 @@ __device__ bool valhist_row(const RowArgs &a, int r, const char *row, float m, f
     const float vs = dstar >= 0 ? bval16(km - (uint32_t)dstar) : NAN;
     const __nv_bfloat162 vk2 = __floats2bfloat162_rn(vk, vk), vs2 = __floats2bfloat162_rn(vs, vs);
     // (the next round's chunk is loaded before this round's ids are examined)
-    uint4 pw = tid < nch ? ldg16(row + (size_t)tid * 16) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+    uint4 pw = tid < nch ? rc.load(tid) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
     for (int c0 = tid & ~31; c0 < nch; c0 += NT) {  // warp-uniform rounds
         const int c = c0 + lane;
         const bool in = c < nch;
         const uint4 w = pw;
-        pw = c + NT < nch ? ldg16(row + (size_t)(c + NT) * 16) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+        pw = c + NT < nch ? rc.load(c + NT) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
         const uint32_t wd[4] = {w.x, w.y, w.z, w.w};
         uint32_t hm = 0u;
 #pragma unroll
@@ -691,7 +685,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const char *row, float m, f
                 const bool tt = fin && dstar >= 0 && d == (uint32_t)dstar;
                 if (!__any_sync(0xffffffffu, tp || tt)) continue;
                 const unsigned long long o =
-                    order_val(fkey(__uint_as_float(b << 16)), (uint32_t)(c * E::EPC + 2 * q + h));
+                    order_val(fkey(__uint_as_float(b << 16)), (uint32_t)(c * E::EPC + 2 * q + h - rc.head));
                 warp_append_cap(vh->pay, &vh->npay, tp, o, VH_CAP);
                 warp_append_cap(vh->tie, &vh->ntie, tt, o, VH_CAP);
             }
@@ -731,15 +725,249 @@ __device__ bool valhist_row(const RowArgs &a, int r, const char *row, float m, f
     return true;
 }
 
-template <int DT, bool VEC>
+// ---------------------------------------------------------------------------
+// Depth-histogram path for handed rows (their max m and exp-sum S are known):
+// the float32 counterpart of the value histogram, and the second try for
+// bfloat16.  One read counts the ids in DH_W equal bins of depth below the
+// max, down to a value the crossing cannot lie below (top_p = 1: to where an
+// id's mass is below 2^-41); a bin's ids each carry at least its lower and at
+// most its upper edge's mass, so bounds of the cumulative mass give a first
+// and a last bin between which the crossing lies (about 0.5% of the mass apart
+// with bins of T / 200).  A second read sums the exact 2^-40 masses of the ids
+// above that range and lists those inside it and the payload's; the ordered
+// list gives the crossing id.  Returns false, having written nothing, when a
+// list is too long or the payload ends below the bins; the binned path then
+// takes the row (it sums a 64-bit mass per id with shared-memory atomics: 297
+// us a call against 158 with this path, 256 rows of 128256 float32 logits of
+// which 213 are handed over).
+constexpr int DH_W = 4096;    // bins
+constexpr int DH_PAD = 32;    // counters of the ids below them, one per lane
+constexpr int DH_XCAP = 1536; // listed ids around the crossing
+constexpr int DH_PCAP = 768;  // listed ids of the payload's bins
+constexpr int DH_U = 4;       // 16-byte loads in flight per thread
+
+struct DepthHist {
+    union {
+        uint32_t cnt[DH_W + DH_PAD];
+        struct {  // (once the counts are read)
+            unsigned long long xs[2048];  // (a power of two for the sort)
+        };
+    };
+    unsigned long long ps[DH_PCAP];
+    unsigned long long fx[DH_XCAP];  // masses of the ordered crossing list
+    float wu[NWARP], wl[NWARP];
+    uint32_t wc[NWARP];
+    int b_hi, b_lo, b_k, nx, np;
+    uint32_t above_cnt;
+    unsigned long long above;
+    int ix;
+    unsigned long long cum;
+};
+
+template <int DT>
+__device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, float m, float kref, double S, DepthHist *h,
+                          unsigned long long *buf, double *redd, unsigned long long *redu) {
+    constexpr int EPC = Elem<DT>::EPC;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const bool all_in = a.top_p >= 1.0f;
+    const unsigned long long tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
+    // no id below vt holds the crossing (as in the value histogram)
+    const float g = all_in ? -41.0f : fmaxf(log2f((1.0f - a.top_p) * (float)S / (16.0f * (float)a.V)), -41.0f);
+    const float depth = fmaxf(m - (kref + g) / a.c, a.T * 1e-3f);
+    const float inv = (float)(DH_W - 4) / depth, wid_b = depth / (float)(DH_W - 4);
+    // the bin of v is round(C + 1 - v * inv) with the integer C = round(m * inv):
+    // one multiply-add onto 2^23 leaves it in the low bits
+    if (!(fabsf(m * inv) < 4.0e6f)) return false;  // (uniform) the index needs 23 bits
+    const float C = rintf(m * inv), c0 = 8388608.0f + C + 1.0f, cmax = 8388608.0f + (float)(DH_W + lane);
+    auto bin_of = [&](float v) -> int {
+        return (int)(__float_as_uint(fminf(fmaf(v, -inv, c0), cmax)) - 0x4B000000u);
+    };
+    for (int i = tid; i < DH_W + DH_PAD; i += NT) h->cnt[i] = 0u;
+    if (tid == 0) {
+        h->b_hi = all_in ? -1 : INT_MAX;
+        h->b_lo = all_in ? -1 : INT_MAX;
+        h->b_k = INT_MAX;
+        h->nx = 0;
+        h->np = 0;
+        h->ix = -1;
+    }
+    __syncthreads();
+    const uint32_t NI = Elem<DT>::NEG_INF_WORD;
+    for (int c0i = tid; c0i < rc.nch; c0i += NT * DH_U) {
+        uint4 w[DH_U];
+#pragma unroll
+        for (int u = 0; u < DH_U; ++u) {
+            const int c = c0i + u * NT;
+            w[u] = c < rc.nch ? rc.load(c) : make_uint4(NI, NI, NI, NI);
+        }
+#pragma unroll
+        for (int u = 0; u < DH_U; ++u)
+#pragma unroll
+            for (int e = 0; e < EPC; ++e) {
+                const int bn = bin_of(Elem<DT>::get(w[u], e));
+                if (ACES_IN(bn, DH_W + DH_PAD)) atomicAdd(&h->cnt[bn], 1u);
+            }
+    }
+    __syncthreads();
+    // ---- the bins around the crossing and the payload's last ----
+    {
+        constexpr int PER = DH_W / NT;
+        uint32_t cn[PER], lc = 0u;
+        float lu = 0.0f, ll = 0.0f, mu[PER], ml[PER];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int bn = tid * PER + i;
+            cn[i] = h->cnt[bn];
+            // v * inv lies within [C + 0.5 - bn, C + 1.5 - bn]
+            const float vu = fminf((C + 1.5f - (float)bn) * wid_b, m), vl = (C + 0.5f - (float)bn) * wid_b;
+            mu[i] = (float)cn[i] * ex2(fmaf(vu, a.c, -kref)) * (1.0f + 1e-4f);
+            ml[i] = (float)cn[i] * ex2(fmaf(vl, a.c, -kref)) * (1.0f - 1e-4f);
+            lu += mu[i];
+            ll += ml[i];
+            lc += cn[i];
+        }
+        float iu = lu, il = ll;
+        uint32_t ic = lc;
+        for (int o = 1; o < 32; o <<= 1) {
+            const float tu = __shfl_up_sync(0xffffffffu, iu, o), tl = __shfl_up_sync(0xffffffffu, il, o);
+            const uint32_t tc = __shfl_up_sync(0xffffffffu, ic, o);
+            if (lane >= o) {
+                iu += tu;
+                il += tl;
+                ic += tc;
+            }
+        }
+        if (lane == 31) {
+            h->wu[wid] = iu;
+            h->wl[wid] = il;
+            h->wc[wid] = ic;
+        }
+        __syncthreads();
+        for (int i = 0; i < wid; ++i) {
+            iu += h->wu[i];
+            il += h->wl[i];
+            ic += h->wc[i];
+        }
+        float cu = iu - lu, cl = il - ll;
+        uint32_t cc = ic - lc;
+        const float tgf = (float)tg * (1.0f / FX_SCALE);
+        const uint32_t ku = (uint32_t)a.k;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int bn = tid * PER + i;
+            cu += mu[i];
+            cl += ml[i];
+            cc += cn[i];
+            if (!all_in) {  // (1e-4: the rounding of the sums and of the target)
+                if (cu >= tgf * (1.0f - 1e-4f)) atomicMin(&h->b_hi, bn);
+                if (cl >= tgf * (1.0f + 1e-4f)) atomicMin(&h->b_lo, bn);
+            }
+            if (cc >= ku) atomicMin(&h->b_k, bn);
+        }
+        __syncthreads();
+    }
+    const int b_hi = h->b_hi, b_lo = h->b_lo;
+    if (b_lo == INT_MAX || (all_in && h->b_k == INT_MAX)) return false;
+    const int b_k = a.k == 0 ? -1 : (all_in ? h->b_k : min(h->b_k, b_lo));
+    __syncthreads();  // (every bin is read: the lists may take the counters' place)
+    // ---- exact masses above the range, the ids inside it and the payload's ----
+    const int b_top = max(b_lo, b_k);
+    uint32_t hs = 0u, ls = 0u, na = 0u;
+    for (int c0i = tid & ~31; c0i < rc.nch; c0i += NT * 2) {  // warp-uniform rounds
+        uint4 w[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = c0i + lane + u * NT;
+            w[u] = c < rc.nch ? rc.load(c) : make_uint4(NI, NI, NI, NI);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int c = c0i + lane + u * NT;
+            float mx = Elem<DT>::get(w[u], 0);
+#pragma unroll
+            for (int e = 1; e < EPC; ++e) mx = fmaxf(mx, Elem<DT>::get(w[u], e));
+            if (!__any_sync(0xffffffffu, bin_of(mx) <= b_top)) continue;
+#pragma unroll
+            for (int e = 0; e < EPC; ++e) {
+                const float v = Elem<DT>::get(w[u], e);
+                const int bn = bin_of(v);
+                if (bn < b_hi) {
+                    uint32_t fh, fl;
+                    to_fx_parts(ex2(fmaf(v, a.c, -kref)), fh, fl);
+                    hs += fh;
+                    ls += fl;
+                    ++na;
+                }
+                const bool tx = bn >= b_hi && bn <= b_lo, tp = bn <= b_k;
+                if (__any_sync(0xffffffffu, tx || tp)) {
+                    const unsigned long long o = order_val(fkey(v), (uint32_t)(c * EPC + e - rc.head));
+                    warp_append_cap(h->xs, &h->nx, tx, o, DH_XCAP);
+                    warp_append_cap(h->ps, &h->np, tp, o, DH_PCAP);
+                }
+            }
+        }
+    }
+    const unsigned long long above = block_reduce(((unsigned long long)hs << 20) + ls, redu, SumU64());
+    const unsigned long long n_above = block_reduce((unsigned long long)na, redu, SumU64());
+    __syncthreads();
+    const int nx = h->nx, np = h->np;
+    if (nx > DH_XCAP || np > DH_PCAP || (!all_in && above >= tg)) return false;
+    // the payload's ids by rank
+    const int lp = np < a.k ? np : a.k;
+    for (int i = tid; i < np; i += NT) {
+        const unsigned long long key = h->ps[i];
+        int rank = 0;
+#pragma unroll 4
+        for (int t = 0; t < np; ++t) rank += h->ps[t] > key;
+        if (rank < lp && ACES_IN(rank, ACES_MAX_TOPK)) buf[rank] = key;
+    }
+    double S_nuc = S;
+    unsigned long long cut = 0ull;
+    int L = lp;
+    if (!all_in) {
+        const int p2 = next_pow2(nx < 2 ? 2 : nx);
+        for (int i = nx + tid; i < p2; i += NT) h->xs[i] = 0ull;
+        __syncthreads();
+        bitonic_sort_desc(h->xs, p2);
+        for (int i = tid; i < nx; i += NT) h->fx[i] = to_fx(ex2(fmaf(order_value(h->xs[i]), a.c, -kref)));
+        __syncthreads();
+        const int per = (nx + NT - 1) / NT;
+        const int lo = min(nx, tid * per), hi = min(nx, lo + per);
+        unsigned long long loc = 0ull;
+        for (int i = lo; i < hi; ++i) loc += h->fx[i];
+        unsigned long long tot;
+        unsigned long long cum = above + block_exscan_n<NT>(loc, redu, &tot);
+        for (int i = lo; i < hi; ++i) {
+            const unsigned long long prev = cum;
+            cum += h->fx[i];
+            if (prev < tg && cum >= tg) {  // one id crosses
+                h->ix = i;
+                h->cum = cum;
+            }
+        }
+        __syncthreads();
+        const int ix = h->ix;
+        if (ix < 0) return false;
+        S_nuc = (double)h->cum * FX_INV;
+        cut = ACES_IN(ix, DH_XCAP) ? h->xs[ix] : 0ull;
+        const unsigned long long n_nuc = n_above + (unsigned long long)ix + 1ull;
+        if (n_nuc < (unsigned long long)L) L = (int)n_nuc;
+    }
+    __syncthreads();
+    finish_row<DT>(a, r, rc.row(), kref, S_nuc, cut, all_in ? RS_ALL_IN : 0, buf, L, redd);
+    return true;
+}
+
+template <int DT>
 __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ RowArgs a) {
+    namespace cg = cooperative_groups;
     using E = Elem<DT>;
     __shared__ SelState st;
     __shared__ union {
         BinState bs;   // binned path
         ValHist vh;    // value-histogram path (bfloat16)
+        DepthHist dh;  // depth-histogram path
     } paths;
-    BinState &bst = paths.bs;
     static_assert(sizeof(paths) >= DRAW_SCRATCH, "the draw's scratch fits");
     unsigned char *scratch = reinterpret_cast<unsigned char *>(&paths);  // (of a finished row)
     __shared__ unsigned long long buf[ACES_MAX_TOPK];
@@ -748,7 +976,11 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
     __shared__ unsigned long long redu[NWARP];
     __shared__ int s_bad;
     __shared__ int s_nbuf;
+    __shared__ DrawPart part;
+    __shared__ int pend[DRAW_CL];
     const int tid = threadIdx.x;
+    cg::cluster_group cl = cg::this_cluster();
+    const int CL = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     pdl_wait();  // after the single-pass row kernel: its fallback list is complete
     if (a.K > 0 && blockIdx.x == 0 && tid < WS_COUNTERS / 4) {
         // the hints of this call's rows, for the first rows of the next call
@@ -765,30 +997,33 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
         if (tid == 7) v = __ldcg(&a.ws.fb_count[11]);
         a.ws.carry[tid] = v;
     }
-    const int nrows = *a.ws.fb_count;
-    for (int idx = blockIdx.x; idx < nrows; idx += gridDim.x) {
-        const int r = a.ws.fb_list[idx];
-        if (!ACES_IN(r, a.rows)) continue;  // (the same r in every thread)
-        const char *row = reinterpret_cast<const char *>(a.logits) + (size_t)r * a.V * E::SIZE;
-        // a row the single-pass kernel handed over comes with its max and its
-        // exp-sum (and is finite); the max pass runs only where the paths
-        // need the finite count it takes (top_p = 1 on float32 rows)
-        RowStat hs;
-        hs.flags = 0;
-        if (VEC) hs = a.ws.stats[r];
+    // one handed row (all threads)
+    auto do_row = [&](int r) {
+        const RowChunks<DT> rc(reinterpret_cast<const char *>(a.logits) + (size_t)r * a.V * E::SIZE, a.V);
+        // it comes with its max and its exp-sum (and is finite); the max pass
+        // runs only where the paths need the finite count it takes (top_p = 1
+        // on float32 rows)
+        const RowStat hs = a.ws.stats[r];
         const bool handed = hs.flags == RS_HANDOFF;
-        float m;
+        float m = hs.kref;
         unsigned long long n_fin = 0ull;
-        if (handed && (DT == ACES_BF16 || a.top_p < 1.0f)) {
-            m = hs.kref;
-        } else {
+        float kref = ceilf(m * a.c);  // masses are 2^(z*c - kref) <= 1
+        // the handed exp-sum in units of 2^kref (its reference is the same
+        // ceil(m c); the power-of-two rescale is exact)
+        const double S_in = handed ? ldexp(hs.S_nuc, (int)(hs.c - kref)) : 0.0;
+        if (DT == ACES_F32 && handed) {
+            const bool done = depth_row<DT>(a, r, rc, m, kref, S_in, &paths.dh, buf, redd, redu);
+            __syncthreads();
+            if (done) return;
+        }
+        if (!(handed && (DT == ACES_BF16 || a.top_p < 1.0f))) {
             // pass 0: max, finite count, invalid values
             if (tid == 0) s_bad = 0;
             __syncthreads();
             float mx = -INFINITY;
             unsigned long long nfin = 0;
             int bad = 0;
-            for_each_elem<DT, VEC>(row, a.V, [&](int, float v) {
+            for_each_elem<DT>(rc, [&](int, float v) {
                 if (v != v || v == INFINITY) bad = 1;
                 if (v > -INFINITY) ++nfin;
                 mx = fmaxf(mx, v);
@@ -796,45 +1031,36 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
             if (bad) s_bad = 1;
             m = block_reduce(mx, redf, MaxF());
             n_fin = block_reduce(nfin, redu, SumU64());
-            if (s_bad || n_fin == 0ull || !(ceilf(m * a.c) < 1e30f)) {
+            kref = ceilf(m * a.c);
+            if (s_bad || n_fin == 0ull || !(kref < 1e30f)) {
                 nonfinite_row<NT>(a, r);
-                row_finished<DT, NT, false>(a, r, scratch);
-                __syncthreads();
-                continue;
+                return;
             }
         }
-        const float kref = ceilf(m * a.c);  // masses are 2^(z*c - kref) <= 1
-        if (DT == ACES_BF16 && VEC) {
-            // the handed exp-sum in units of 2^kref (its reference is the same
-            // ceil(m c); the power-of-two rescale is exact)
-            const double S_in = handed ? ldexp(hs.S_nuc, (int)(hs.c - kref)) : 0.0;
+        if constexpr (DT == ACES_BF16) {
             unsigned long long nf = 0ull;
-            const bool done = valhist_row(a, r, row, m, kref, S_in, &nf, &paths.vh, buf, redd, redu);
+            bool done = valhist_row(a, r, rc, m, kref, S_in, &nf, &paths.vh, buf, redd, redu);
             __syncthreads();
-            if (done) {
-                row_finished<DT, NT, false>(a, r, scratch);
+            if (!done && handed) {
+                done = depth_row<DT>(a, r, rc, m, kref, S_in, &paths.dh, buf, redd, redu);
                 __syncthreads();
-                continue;
             }
+            if (done) return;
             n_fin = nf;
         }
-        if (binned_row<DT, VEC>(a, r, row, m, kref, n_fin, &bst, buf, redd, redu)) {
-            row_finished<DT, NT, false>(a, r, scratch);
-            __syncthreads();
-            continue;
-        }
+        if (binned_row<DT>(a, r, rc, m, kref, n_fin, &paths.bs, buf, redd, redu)) return;
         if (tid == 0) atomicAdd(&a.ws.fb_count[4], 1);
         const bool all_in = a.top_p >= 1.0f;
         unsigned long long cut = 0ull;
         double S_nuc;
         unsigned long long n_nuc;
         if (!all_in) {
-            cut = radix_select<DT, VEC>(row, a.V, kref, a.c, 0, (double)a.top_p, 0u, true, &st);
+            cut = radix_select<DT>(rc, kref, a.c, 0, (double)a.top_p, 0u, true, &st);
             S_nuc = (double)(st.above + st.found) * FX_INV;
             n_nuc = (unsigned long long)st.above_cnt + 1ull;
         } else {
             unsigned long long sfx = 0ull;
-            for_each_elem<DT, VEC>(row, a.V, [&](int, float v) {
+            for_each_elem<DT>(rc, [&](int, float v) {
                 if (v > -INFINITY) sfx += to_fx(ex2(fmaf(v, a.c, -kref)));
             });
             S_nuc = (double)block_reduce(sfx, redu, SumU64()) * FX_INV;
@@ -846,13 +1072,13 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
         unsigned long long lim = all_in ? 0ull : cut;
         int L = (int)(n_nuc < (unsigned long long)a.k ? n_nuc : (unsigned long long)a.k);
         if (a.k > 0 && n_nuc > (unsigned long long)a.k)
-            lim = radix_select<DT, VEC>(row, a.V, kref, a.c, 1, 0.0, (unsigned)a.k, false, &st);
+            lim = radix_select<DT>(rc, kref, a.c, 1, 0.0, (unsigned)a.k, false, &st);
         __syncthreads();
         // collect the payload ids (order value >= lim)
         if (tid == 0) s_nbuf = 0;
         __syncthreads();
         if (a.k > 0) {
-            for_each_elem<DT, VEC>(row, a.V, [&](int x, float v) {
+            for_each_elem<DT>(rc, [&](int x, float v) {
                 if (!(v > -INFINITY)) return;
                 unsigned long long o = order_val(fkey(v), (uint32_t)x);
                 if (o >= lim) {
@@ -868,16 +1094,37 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
         __syncthreads();
         bitonic_sort_desc(buf, np);
         if (L > nb) L = nb;
-        finish_row<DT>(a, r, row, kref, S_nuc, cut, all_in ? RS_ALL_IN : 0, buf, L, redd);
-        row_finished<DT, NT, false>(a, r, scratch);
+        finish_row<DT>(a, r, rc.row(), kref, S_nuc, cut, all_in ? RS_ALL_IN : 0, buf, L, redd);
+    };
+    // the handed rows, one a CTA and cluster round; the sequences a round
+    // completes are then drawn by the cluster
+    const int nrows = *a.ws.fb_count;
+    for (int i0 = (int)(blockIdx.x / CL) * CL; i0 < nrows; i0 += (int)gridDim.x) {
+        int e = -1;
+        if (i0 + rank < nrows) {
+            const int r = a.ws.fb_list[i0 + rank];
+            if (ACES_IN(r, a.rows)) {  // (the same r in every thread)
+                do_row(r);
+                e = row_finished<DT, NT>(a, r, scratch);
+            }
+        }
+        if (a.K > 0) {
+            if (tid == 0) part.pend = e;
+            cl.sync();
+            if (tid < CL) pend[tid] = cl.map_shared_rank(&part, tid)->pend;
+            cl.sync();
+            for (int c = 0; c < CL; ++c)
+                if (pend[c] >= 0) {
+                    draw_cluster<DT, NT>(a, pend[c] >> 5, pend[c] & 31, &part, scratch);
+                    __syncthreads();
+                }
+        }
         __syncthreads();
     }
-    // the sequences whose rows are all done and whose draw needs a whole row
+    // the sequences the single-pass kernel completed whose draw needs a whole row
     if (a.K > 0) {
-        __shared__ DrawPart part;
         const int nscan = a.ws.fb_count[13];
-        const int ncta = (int)cooperative_groups::this_cluster().num_blocks();
-        for (int i = blockIdx.x / ncta; i < nscan; i += gridDim.x / ncta) {
+        for (int i = blockIdx.x / CL; i < nscan; i += gridDim.x / CL) {
             const int e = a.ws.scan_list[i];
             draw_cluster<DT, NT>(a, e >> 5, e & 31, &part, scratch);
             __syncthreads();
@@ -890,16 +1137,14 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
 // draws fill them; the CTAs of a draw's cluster: as many as let every sequence
 // be drawn at once (a draw is a chain of about 20 us however few logits each
 // CTA has: 128 sequences in four rounds of clusters of 8 took 120 us).
-cudaError_t launch_rows_general(const RowArgs &a, int dt, bool vec, int nseq, cudaStream_t s) {
+cudaError_t launch_rows_general(const RowArgs &a, int dt, int nseq, cudaStream_t s) {
     const int most = 2 * a.nsm / DRAW_CL * DRAW_CL;
     int cl = DRAW_CL;
     while (cl > 2 && (long long)cl * nseq > most) cl >>= 1;
     long long want = a.K > 0 && (long long)cl * nseq > a.rows ? (long long)cl * nseq : a.rows;
     want = (want + DRAW_CL - 1) / DRAW_CL * DRAW_CL;
     const unsigned grid = (unsigned)(want < most ? want : most);
-    void (*fn)(RowArgs) = dt == ACES_BF16 ? (vec ? k_rows_general<ACES_BF16, true> : k_rows_general<ACES_BF16, false>)
-                                               : (vec ? k_rows_general<ACES_F32, true> : k_rows_general<ACES_F32, false>);
-    return launch_after(fn, grid, NT, (unsigned)cl, s, a);
+    return launch_after(dt == ACES_BF16 ? k_rows_general<ACES_BF16> : k_rows_general<ACES_F32>, grid, NT, (unsigned)cl, s, a);
 }
 
 #ifdef ACES_CHECKED
