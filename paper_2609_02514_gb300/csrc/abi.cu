@@ -1,5 +1,6 @@
 // C ABI of the AceSpec path: argument validation, launch configuration and
 // workspace carving.  Nothing here allocates memory.
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <mutex>
@@ -13,10 +14,14 @@ namespace {
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
+// SMs of the current device (asked once per device)
 int sm_count() {
+    static std::atomic<int> of[64];
     int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 132;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 132;
+    if (dev < 64 && (n = of[dev].load(std::memory_order_relaxed)) > 0) return n;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 132;
+    if (dev < 64) of[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
