@@ -513,8 +513,9 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         const int hq = bal ? __shfl_sync(0xffffffffu, hb, __ffs(bal) - 1) : NSB - 1;
         if (lane == 0) {
             s_dbins = hr >= HINT_MIN ? min(hq + HINT_MARGIN, NSB - 1) + 1 : -1;
-            // the sketch-led pass when nearly every finished row was short
-            s_skm = BF && hr >= HINT_MIN && (long long)hs * SHORT_DEN >= (long long)hr * SHORT_NUM;
+            // the sketch-led pass when nearly every finished row was short, and
+            // for top_p = 1 (its payload is all that is needed of the row)
+            s_skm = BF && (all_in || (hr >= HINT_MIN && (long long)hs * SHORT_DEN >= (long long)hr * SHORT_NUM));
         }
     }
     publish_max(im);
@@ -983,6 +984,32 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                 const uint32_t lb = t > 0.0f ? (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rd(t)) : 1u;
                 const uint32_t kfull = km > (uint32_t)(HW - 1) ? km - (uint32_t)(HW - 1) : 1u;
                 thb0 = lb > kfull ? lb : kfull;
+                if (all_in) {
+                    // top_p = 1: the k-th largest group max, from counts of the
+                    // sketch's values, is at or below the k-th id, and only the
+                    // groups that reach it are read back.  (The hinted depth D
+                    // spans too many groups on flat rows: 133 of 160 rows of
+                    // 102400 were counted in a second pass, 10 us a row.)
+                    thb0 = kfull;
+                    auto add = [&](int v) {
+                        const int i = v - (int)kfull;
+                        if (i >= 0 && ACES_IN(i, HW)) atomicAdd(&hist[i], 1u);
+                    };
+                    for (int i = tid; i < (gpi == 2 ? ng_all / 2 : ng_all); i += NTC) {
+                        if (gpi == 2) {
+                            const uint32_t g = reinterpret_cast<const uint32_t *>(sk)[i];
+                            add((int)(int16_t)(g & 0xFFFFu));
+                            add((int)g >> 16);
+                        } else {
+                            add((int)(int16_t)sk[i]);
+                        }
+                    }
+                    __syncthreads();
+                    if (scan(kfull) != 0) return 1;  // (fewer than k groups reach the window, or far too many tie)
+                    thb0 = vr >= 0 ? kfull + (uint32_t)vr : km;  // (k = 0: nothing but the max)
+                    for (int i = tid; i < HW; i += NTC) hist[i] = 0u;
+                    __syncthreads();
+                }
             }
             uint32_t *gls = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(sk) + SK_TMP);
             const int nc = compact(thb0, gls);  // (ends with a barrier)
