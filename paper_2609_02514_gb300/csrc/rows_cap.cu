@@ -1483,50 +1483,42 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                 if (ACES_IN(i, WCAP)) efx[i] = id_fx(order_value(ord[i]), a.c, kref);
         }
         __syncthreads();
-        // nucleus crossing with exact fixed-point prefix sums (warp 0)
-        if (wid == 0) {
-            const int per = (n + 31) / 32;
-            const int lo = lane * per, hi = min(n, lo + per);
-            unsigned long long loc = 0ull;
+        // nucleus crossing with exact fixed-point prefix sums (consecutive
+        // entries per thread; by one warp it took 3 us, up to 8 on long lists)
+        {
+            const int per = (n + NTC - 1) / NTC;
+            const int lo = min(n, tid * per), hi = min(n, lo + per);
+            unsigned long long loc = 0ull, tot;
             for (int i = lo; i < hi; ++i) loc += efx[i];
-            unsigned long long inc = loc;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long tt = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += tt;
-            }
-            const unsigned long long ex = inc - loc;
-            int nstar = n - 1;
-            if (!all_in) {
-                int found = INT_MAX;
-                unsigned long long c = ex;
+            const unsigned long long ex = block_exscan_n<NTC>(loc, s_redu, &tot);
+            unsigned long long c = ex;
+            if (!all_in)
                 for (int i = lo; i < hi; ++i) {
+                    const unsigned long long prev = c;
                     c += efx[i];
-                    if (c >= tg) {
-                        found = i;
-                        break;
+                    if (prev < tg && c >= tg) {  // (one entry)
+                        s_nstar = i;
+                        s_above = c;
                     }
                 }
-                const unsigned bal = __ballot_sync(0xffffffffu, found != INT_MAX);
-                nstar = bal ? __shfl_sync(0xffffffffu, found, __ffs(bal) - 1) : INT_MAX;
-            }
-            int L = 0;
-            if (nstar != INT_MAX) L = all_in ? min(n, a.k) : min(nstar + 1, a.k);
-            unsigned long long cN = 0ull, cL = 0ull, c = ex;
-            for (int i = lo; i < hi; ++i) {
-                c += efx[i];
-                if (i == nstar) cN = c;
-                if (i == L - 1) cL = c;
-            }
-            cN = warp_sum(cN);
-            cL = warp_sum(cL);
-            if (lane == 0) {
-                s_nstar = nstar;
-                s_L = L;
-                s_cumL_fx = cL;
-                const double sn = all_in ? S : (double)cN * FX_INV;  // (lane 0 of warp 0 is thread 0)
-                s_Snuc = sn;
-                s_inv_S = inv_mass(sn);
-                s_cut = (nstar != INT_MAX && !all_in) ? ord[nstar] : 0ull;
+            __syncthreads();
+            const int nstar = all_in ? n - 1 : s_nstar;  // (INT_MAX: below the list)
+            if (nstar != INT_MAX) {
+                const int Lw = min(nstar + 1, a.k);
+                c = ex;
+                for (int i = lo; i < hi && i < Lw; ++i) {
+                    c += efx[i];
+                    if (i == Lw - 1) s_cumL_fx = c;
+                }
+                if (tid == 0) {
+                    s_nstar = nstar;
+                    s_L = Lw;
+                    if (Lw == 0) s_cumL_fx = 0ull;
+                    const double sn = all_in ? S : (double)s_above * FX_INV;
+                    s_Snuc = sn;
+                    s_inv_S = inv_mass(sn);
+                    s_cut = all_in ? 0ull : ord[nstar];
+                }
             }
         }
         __syncthreads();
