@@ -303,6 +303,44 @@ __device__ __forceinline__ void bitonic_sort_desc(unsigned long long *a, int n_p
     }
 }
 
+// How many of the n 32-bit keys at k (shared memory, 16-byte aligned, zeros up
+// to a multiple of four) are above key; EQ: and how many equal it (itself
+// included) in *eq.  Four keys a load: the loads are what ranking by direct
+// counting is bound by (n * n / 32 of them for 64-bit keys: 4 us at n = 512).
+template <bool EQ>
+__device__ __forceinline__ int count_above(const uint32_t *k, int n, uint32_t key, int *eq) {
+    const uint4 *k4 = reinterpret_cast<const uint4 *>(k);
+    int r = 0, q = 0;
+#pragma unroll 4
+    for (int t = 0; t < (n + 3) >> 2; ++t) {
+        const uint4 v = k4[t];
+        r += (int)(v.x > key) + (int)(v.y > key) + (int)(v.z > key) + (int)(v.w > key);
+        if (EQ) q += (int)(v.x == key) + (int)(v.y == key) + (int)(v.z == key) + (int)(v.w == key);
+    }
+    if (EQ) *eq = q;
+    return r;
+}
+
+// The ranks of n distinct 64-bit order values (descending) handed to put(rank,
+// value), by all NTH threads: counted on their upper halves (written to k32,
+// room for n rounded up to four), on all 64 bits only where those tie.  (o is
+// complete, by a barrier, before the call.)
+template <int NTH, class Put>
+__device__ __forceinline__ void rank_order_values(const unsigned long long *o, int n, uint32_t *k32, Put put) {
+    for (int i = threadIdx.x; i < ((n + 3) & ~3); i += NTH) k32[i] = i < n ? (uint32_t)(o[i] >> 32) : 0u;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += NTH) {
+        const unsigned long long v = o[i];
+        int eq;
+        int rank = count_above<true>(k32, n, (uint32_t)(v >> 32), &eq);
+        if (eq > 1) {
+            rank = 0;
+            for (int t = 0; t < n; ++t) rank += o[t] > v;
+        }
+        put(rank, v);
+    }
+}
+
 __host__ __device__ __forceinline__ int next_pow2(int n) {
     int p = 1;
     while (p < n) p <<= 1;

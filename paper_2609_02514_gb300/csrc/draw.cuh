@@ -35,7 +35,7 @@ namespace aces {
 constexpr int DRAW_TASKS = 512;
 constexpr int DRAW_CL = 8;  // CTAs of a draw's cluster, at most
 constexpr int DRAW_CH = 4;  // 16-byte chunks per lane and step of a task
-constexpr int DRAW_SCRATCH = 4 * NUC_CAP * 8;  // bytes of shared memory either draw uses
+constexpr int DRAW_SCRATCH = 4 * NUC_CAP * 8;  // bytes of shared memory the draws use, on a 16-byte boundary
 static_assert(DRAW_TASKS * (3 * 8 + 4) <= DRAW_SCRATCH, "the tasks' sums fit");
 
 // A row of V logits in 16-byte chunks.  A row that does not start on a
@@ -849,37 +849,39 @@ __device__ int draw_list(const ScanRow &s, const unsigned long long *lst, int n,
     static_assert(2 * NTH >= NUC_CAP, "two nucleus entries per thread");
     __shared__ unsigned long long red[NTH / 32];
     __shared__ int s_tok, s_bad;
-    unsigned long long *skey = reinterpret_cast<unsigned long long *>(scratch), *srt = skey + NUC_CAP;
-    unsigned long long *rfx = srt + NUC_CAP, *pfx = rfx + NUC_CAP;
+    unsigned long long *rfx = reinterpret_cast<unsigned long long *>(scratch), *pfx = rfx + NUC_CAP;
+    uint32_t *inv = reinterpret_cast<uint32_t *>(pfx + NUC_CAP);  // 2^32 - 1 - id (0: none), to be counted from above
+    uint32_t *srt = inv + NUC_CAP;                               // entries in ascending id order
     const int tid = threadIdx.x;
     if (tid == 0) {
         s_bad = 0;
         s_tok = -1;
     }
     __syncthreads();
-    for (int i = tid; i < n; i += NTH) {
+    for (int i = tid; i < ((n + 3) & ~3); i += NTH) {
+        if (i >= n) {
+            inv[i] = 0u;
+            continue;
+        }
         const unsigned long long o = lst[i];
         const uint32_t id = order_id(o);
         int bad = 0;
         const bool has_q = s.q != nullptr && ACES_IN(id, s.V);
         rfx[i] = member_mass(order_value(o), has_q ? __ldg(s.q + id) : 0.0f, has_q, s, &pfx[i], &bad);
         if (bad) s_bad = 1;
-        skey[i] = ((unsigned long long)id << 32) | (unsigned long long)i;  // distinct keys
+        inv[i] = 0xFFFFFFFFu - id;
     }
     __syncthreads();
     if (s_bad) return -2;
-    for (int i = tid; i < n; i += NTH) {  // ascending id: each key's rank among the others
-        const unsigned long long key = skey[i];
-        int rank = 0;
-#pragma unroll 4
-        for (int j = 0; j < n; ++j) rank += skey[j] < key;
-        if (ACES_IN(rank, NUC_CAP)) srt[rank] = key;
+    for (int i = tid; i < n; i += NTH) {  // ascending id (ids are distinct)
+        const int rank = count_above<false>(inv, n, inv[i], nullptr);
+        if (ACES_IN(rank, NUC_CAP)) srt[rank] = (uint32_t)i;
     }
     __syncthreads();
     // two consecutive entries (in id order) per thread
     const int e0 = 2 * tid, e1 = 2 * tid + 1;
-    int i0 = e0 < n ? (int)(srt[e0] & 0xFFFFFFFFull) : -1;
-    int i1 = e1 < n ? (int)(srt[e1] & 0xFFFFFFFFull) : -1;
+    int i0 = e0 < n ? (int)srt[e0] : -1;
+    int i1 = e1 < n ? (int)srt[e1] : -1;
     if (i0 >= 0 && !ACES_IN(i0, NUC_CAP)) i0 = -1;
     if (i1 >= 0 && !ACES_IN(i1, NUC_CAP)) i1 = -1;
     unsigned long long w0 = i0 >= 0 ? rfx[i0] : 0ull, w1 = i1 >= 0 ? rfx[i1] : 0ull, tot;
@@ -891,8 +893,8 @@ __device__ int draw_list(const ScanRow &s, const unsigned long long *lst, int n,
     }
     if (tot > 0ull) {
         const unsigned long long thr = floor_u_times(s.u, tot);
-        if (ex <= thr && thr < ex + w0) s_tok = (int)(srt[e0] >> 32);
-        else if (ex + w0 <= thr && thr < ex + w0 + w1) s_tok = (int)(srt[e1] >> 32);
+        if (ex <= thr && thr < ex + w0) s_tok = (int)(0xFFFFFFFFu - inv[i0]);
+        else if (ex + w0 <= thr && thr < ex + w0 + w1) s_tok = (int)(0xFFFFFFFFu - inv[i1]);
     }
     __syncthreads();
     return s_tok;

@@ -113,9 +113,10 @@ struct F32Caps {
 constexpr int RANK_MAX = 512;       // ids ordered by direct ranking (more: bitonic sort)
 static_assert(WS_DEPTH + NSB <= WS_COUNTERS / 4, "the depth histogram fits the counters area");
 static_assert(DRAW_SCRATCH <= SMEM_BF && DRAW_SCRATCH <= SMEM_F32, "the draw's scratch fits");
+static_assert(ACES_MAX_V <= 1 << 20 && HW <= 1 << 10 && RANK_MAX <= HW, "a value and an id in 30 bits");
 static_assert(GCAP * 4 <= HW * 4 && PCAP * 8 <= SKG * 2 && "the aliased areas fit");
 static_assert(PCAP <= SK_TMP && SK_TMP + GCAP / 2 <= SKG / 4 && SK_TMP + PCAP <= SKG / 4, "the sketch-led areas fit");
-static_assert(WCAP * 8 <= CREC * 20 && RANK_MAX * 2 <= LCAP, "the float32 work areas fit");
+static_assert(WCAP * 8 <= CREC * 20 && RANK_MAX * 5 / 2 <= LCAP, "the float32 work areas fit");
 static_assert(F32Caps<2>::WC * 8 <= F32Caps<2>::CR * 20 && RANK_MAX * 2 <= F32Caps<2>::LC &&
                   2 * (F32Caps<2>::SMEM + 1024) <= 228 * 1024,
               "the wide float32 areas fit, two CTAs per SM");
@@ -1101,12 +1102,16 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             // order them (descending order value)
             if (npay <= RANK_MAX) {
                 ord = sorted;
+                // (the value in the window, then the lower id: 30 bits)
+                for (int i = tid; i < ((npay + 3) & ~3); i += NTC) {
+                    const unsigned long long o = i < npay ? pay[i] : 0ull;
+                    const uint32_t idx = (__float_as_uint(order_value(o)) >> 16) - thb0;
+                    hist[i] = i < npay ? (idx << 20 | (0xFFFFFu - order_id(o))) + 1u : 0u;
+                }
+                __syncthreads();
                 for (int i = tid; i < npay; i += NTC) {
-                    const unsigned long long key = pay[i];
-                    int rank = 0;
-#pragma unroll 4
-                    for (int t = 0; t < npay; ++t) rank += pay[t] > key;
-                    if (ACES_IN(rank, PCAP)) ord[rank] = key;
+                    const int rank = count_above<false>(hist, npay, hist[i], nullptr);
+                    if (ACES_IN(rank, PCAP)) ord[rank] = pay[i];
                 }
             } else {
                 if (tid == 0) atomicAdd(&a.ws.fb_count[3], 1);
@@ -1419,16 +1424,12 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         if (n <= RANK_MAX) {
             ord = list;
             efx = list + RANK_MAX;
-            for (int i = tid; i < n; i += NTC) {
-                const unsigned long long v = cv[i];
-                int rank = 0;
-#pragma unroll 4
-                for (int j = 0; j < n; ++j) rank += cv[j] > v;
+            rank_order_values<NTC>(cv, n, reinterpret_cast<uint32_t *>(list + 2 * RANK_MAX), [&](int rank, unsigned long long v) {
                 if (ACES_IN(rank, RANK_MAX)) {
                     ord[rank] = v;
                     efx[rank] = id_fx(order_value(v), a.c, kref);
                 }
-            }
+            });
         } else {
             // more: bin by bin (the bins of T/8 below m order the values), and
             // inside a bin by direct ranking among its own ids

@@ -754,7 +754,7 @@ struct DepthHist {
         };
     };
     unsigned long long ps[DH_PCAP];
-    unsigned long long fx[DH_XCAP];  // masses of the ordered crossing list
+    alignas(16) unsigned long long fx[DH_XCAP];  // masses of the ordered crossing list
     float wu[NWARP], wl[NWARP];
     uint32_t wc[NWARP];
     int b_hi, b_lo, b_k, nx, np;
@@ -914,13 +914,9 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
     if (nx > DH_XCAP || np > DH_PCAP || (!all_in && above >= tg)) return false;
     // the payload's ids by rank
     const int lp = np < a.k ? np : a.k;
-    for (int i = tid; i < np; i += NT) {
-        const unsigned long long key = h->ps[i];
-        int rank = 0;
-#pragma unroll 4
-        for (int t = 0; t < np; ++t) rank += h->ps[t] > key;
+    rank_order_values<NT>(h->ps, np, reinterpret_cast<uint32_t *>(h->fx), [&](int rank, unsigned long long key) {
         if (rank < lp && ACES_IN(rank, ACES_MAX_TOPK)) buf[rank] = key;
-    }
+    });
     double S_nuc = S;
     unsigned long long cut = 0ull;
     int L = lp;
@@ -963,7 +959,7 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
     namespace cg = cooperative_groups;
     using E = Elem<DT>;
     __shared__ SelState st;
-    __shared__ union {
+    __shared__ __align__(16) union {
         BinState bs;   // binned path
         ValHist vh;    // value-histogram path (bfloat16)
         DepthHist dh;  // depth-histogram path
