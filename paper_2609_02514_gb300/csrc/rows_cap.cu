@@ -70,6 +70,7 @@ constexpr int SAMPLE = 64;          // tiles of the sample: the first of the row
 constexpr int NSB = 40;             // depth bins (of T/SPB) of the hints; D before any hint
 constexpr int SPB = 4;              // depth bins per temperature
 constexpr int MARGIN_BINS = 2;      // float32 first rows: theta below the sample's crossing
+constexpr float LIST_FILL = 0.75f;  // of the list's room, at most, where the sample can tell
 constexpr int HINT_MIN = 32;        // finished rows before their depths set D
 constexpr int HINT_MARGIN = 2;      // depth bins of margin above that quantile
 constexpr float HINT_Q = 0.99f;     // the quantile of the finished rows' depths D covers
@@ -356,7 +357,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     __shared__ int s_nrec, s_nl, s_fb, s_n, s_bsel, s_nstar, s_L, s_npay, s_ng, s_nge, s_j, s_vs, s_vk;
     __shared__ float s_thlo, s_zx;
     __shared__ int s_dbins, s_xb;  // s_dbins: D in depth bins (-1: no hints yet)
-    __shared__ int s_skm;          // bfloat16: the sketch-led pass (no counting while streaming)
+    __shared__ int s_skm;          // bfloat16: the sketch-led pass (no counting while streaming); float32: see there
     __shared__ uint32_t s_mr;  // order key of the running max
     __shared__ double s_Snuc;
     __shared__ float s_inv_S;
@@ -402,10 +403,11 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     }
     // the depths published by the call's finished rows (read by warp 0 only,
     // once: they change while this row streams)
-    int hr = 0, hc0 = 0, hc1 = 0, hs = 0;
+    int hr = 0, hc0 = 0, hc1 = 0, hs = 0, hf = 0;
     if (wid == 0) {
         hr = __ldcg(&a.ws.fb_count[8]);
         hs = __ldcg(&a.ws.fb_count[11]);
+        if (!BF) hf = __ldcg(&a.ws.fb_count[0]);
         hc0 = 2 * lane < NSB ? __ldcg(&a.ws.fb_count[WS_DEPTH + 2 * lane]) : 0;
         hc1 = 2 * lane + 1 < NSB ? __ldcg(&a.ws.fb_count[WS_DEPTH + 2 * lane + 1]) : 0;
         if (BF && hr < HINT_MIN) {
@@ -514,9 +516,11 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         const int hq = bal ? __shfl_sync(0xffffffffu, hb, __ffs(bal) - 1) : NSB - 1;
         if (lane == 0) {
             s_dbins = hr >= HINT_MIN ? min(hq + HINT_MARGIN, NSB - 1) + 1 : -1;
-            // the sketch-led pass when nearly every finished row was short, and
-            // for top_p = 1 (its payload is all that is needed of the row)
-            s_skm = BF && (all_in || (hr >= HINT_MIN && (long long)hs * SHORT_DEN >= (long long)hr * SHORT_NUM));
+            // bfloat16: the sketch-led pass when nearly every finished row was
+            // short, and for top_p = 1 (its payload is all that is needed of
+            // the row); float32: hinted rows look at their sample too once
+            // one row in 16 was handed to the general kernel
+            s_skm = BF ? all_in || (hr >= HINT_MIN && (long long)hs * SHORT_DEN >= (long long)hr * SHORT_NUM) : hf > hr / 16;
         }
     }
     publish_max(im);
@@ -1176,12 +1180,14 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         // Chunks holding an id >= the capture threshold are recorded (16-byte
         // chunk and index).  Hinted rows: the threshold is the running max
         // minus D, so at the end every id >= (row max - D) was recorded.
-        // The first rows: the sample's ids within NSB bins of its max are
+        // The first rows, and those whose sample says that D would list more
+        // than the areas hold: the sample's ids within NSB bins of its max are
         // binned; the bins where the sample's mass (from the exact exp-sums)
         // reaches top_p and where its count reaches nmin set a fixed
-        // threshold.
+        // threshold, MARGIN_BINS lower where the areas hold that many.
         float thlo = INFINITY;
-        if (!hinted) {
+        bool by_depth = hinted;
+        if (!hinted || s_skm) {
             if (have) {
 #pragma unroll
                 for (int u = 0; u < UCS; ++u) {
@@ -1233,19 +1239,27 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                     return bal ? __shfl_sync(0xffffffffu, hb, __ffs(bal) - 1) : NSB;
                 };
                 auto bin_of_count = [&](float n) { return first_bin(pc0f >= n * f, (float)pc >= n * f); };
+                // the first bin where the areas would be LIST_FILL full
+                const int bfull = bin_of_count(LIST_FILL * (float)LCAP);
                 int blo;
                 if (all_in) {
                     blo = bin_of_count((float)a.nmin);
                 } else {
                     const float tm = a.top_p * M;
                     const int bx = first_bin(pm0 >= tm, pm >= tm);
-                    blo = max(bx + MARGIN_BINS, bin_of_count((float)a.nmin));
+                    blo = max(max(min(bx + MARGIN_BINS, bfull - 1), bx + 1), bin_of_count((float)a.nmin));
                 }
                 blo = min(blo, NSB - 1);
-                if (lane == 0) s_thlo = m1 - (float)(blo + 1) * (a.T / SPB);
+                if (lane == 0) {
+                    s_thlo = m1 - (float)(blo + 1) * (a.T / SPB);
+                    s_fb = hinted && hbins - 1 < bfull;
+                }
             }
             __syncthreads();
-            if (have) thlo = s_thlo;
+            if (have) {
+                thlo = s_thlo;
+                by_depth = s_fb != 0;
+            }
         }
         // records the chunks in hb (those holding an id >= the capture
         // threshold): one vote per iteration, one warp-aggregated atomic per
@@ -1276,12 +1290,12 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             }
         };
         {
-            float th = hinted ? m1 - D : thlo;
+            float th = by_depth ? m1 - D : thlo;
             for (int it = 0; it < nit; ++it) {
                 if (it > 0) {  // (iteration 0 is loaded, its sample summed)
                     off0 = wrap(off0 + off_it);
                     load(it);
-                    if (hinted) th = running_max() - D;
+                    if (by_depth) th = running_max() - D;
                 }
                 if (it > 0 || UCS < UC) {
                     group_maxima<DT>(w, g0, g1);
@@ -1289,7 +1303,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                     raise_ref(im);
                     if (it > 0) add_sum(chunks_expsum<DT, 0, UC>(w, a.c, -k_t));
                     else add_sum(chunks_expsum<DT, UCS == UC ? 0 : UCS, UC>(w, a.c, -k_t));
-                    if (hinted) publish_max(im);
+                    if (by_depth) publish_max(im);
                 }
                 record_hits(th);
             }
@@ -1300,7 +1314,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             if (tid == 0) fallback_row(a, r, m, kref, S);
             return;
         }
-        const float thc = hinted ? m - D : thlo;  // every id >= thc was recorded
+        const float thc = by_depth ? m - D : thlo;  // every id >= thc was recorded
         // expand the records: the ids >= thc of every recorded chunk (all such
         // ids lie in recorded chunks), as 64-bit order values
         if (tid == 0) s_nl = 0;

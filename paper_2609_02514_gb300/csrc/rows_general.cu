@@ -871,26 +871,29 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
     const int b_k = a.k == 0 ? -1 : (all_in ? h->b_k : min(h->b_k, b_lo));
     __syncthreads();  // (every bin is read: the lists may take the counters' place)
     // ---- exact masses above the range, the ids inside it and the payload's ----
+    // (ids are looked at one by one only from a value just below the lowest
+    // needed bin: their number per lane, not the row's length, is what costs)
     const int b_top = max(b_lo, b_k);
+    const float v_min = fminf((C + 0.5f - (float)b_top) * wid_b, m) - 2.0f * wid_b;
     uint32_t hs = 0u, ls = 0u, na = 0u;
-    for (int c0i = tid & ~31; c0i < rc.nch; c0i += NT * 2) {  // warp-uniform rounds
-        uint4 w[2];
+    for (int c0i = tid & ~31; c0i < rc.nch; c0i += NT * DH_U) {  // warp-uniform rounds
+        uint4 w[DH_U];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
+        for (int u = 0; u < DH_U; ++u) {
             const int c = c0i + lane + u * NT;
             w[u] = c < rc.nch ? rc.load(c) : make_uint4(NI, NI, NI, NI);
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int c = c0i + lane + u * NT;
-            float mx = Elem<DT>::get(w[u], 0);
+        for (int u = 0; u < DH_U; ++u) {
+            uint32_t mk = 0u;
 #pragma unroll
-            for (int e = 1; e < EPC; ++e) mx = fmaxf(mx, Elem<DT>::get(w[u], e));
-            if (!__any_sync(0xffffffffu, bin_of(mx) <= b_top)) continue;
-#pragma unroll
-            for (int e = 0; e < EPC; ++e) {
-                const float v = Elem<DT>::get(w[u], e);
-                const int bn = bin_of(v);
+            for (int e = 0; e < EPC; ++e) mk |= (uint32_t)(Elem<DT>::get(w[u], e) >= v_min) << e;
+            while (__any_sync(0xffffffffu, mk != 0u)) {
+                const bool on = mk != 0u;
+                const int e = on ? __ffs(mk) - 1 : 0;
+                mk &= mk - 1u;
+                const float v = chunk_at<DT>(w[u], e);
+                const int bn = on ? bin_of(v) : INT_MAX;
                 if (bn < b_hi) {
                     uint32_t fh, fl;
                     to_fx_parts(ex2(fmaf(v, a.c, -kref)), fh, fl);
@@ -900,7 +903,7 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
                 }
                 const bool tx = bn >= b_hi && bn <= b_lo, tp = bn <= b_k;
                 if (__any_sync(0xffffffffu, tx || tp)) {
-                    const unsigned long long o = order_val(fkey(v), (uint32_t)(c * EPC + e - rc.head));
+                    const unsigned long long o = order_val(fkey(v), (uint32_t)((c0i + lane + u * NT) * EPC + e - rc.head));
                     warp_append_cap(h->xs, &h->nx, tx, o, DH_XCAP);
                     warp_append_cap(h->ps, &h->np, tp, o, DH_PCAP);
                 }
