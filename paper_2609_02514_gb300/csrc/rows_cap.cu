@@ -861,13 +861,13 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                 vr = vs;
                 nge = (int)(s_cab + s_cnvs);
             } else if (L > 0) {
-                const bool at_k = nn > ku;  // else the payload ends with the nucleus
+                const bool at_k = all_in || nn > ku;  // else the payload ends with the nucleus, at vs
                 vr = at_k ? s_vk : vs;
                 nge = at_k ? s_nge : (int)(s_cab + s_cnvs);
                 if (nge > PCAP) return 2;
             }
             if (tid == 0) {  // (read after later barriers)
-                if (nn <= ku) s_cumL_fx = nuc;
+                if (!all_in && nn <= ku) s_cumL_fx = nuc;
                 if (ku == 0u) s_cumL_fx = 0ull;
                 s_Snuc = all_in ? S : (double)nuc * FX_INV;
                 s_inv_S = inv_mass(s_Snuc);
