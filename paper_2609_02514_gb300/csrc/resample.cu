@@ -164,10 +164,12 @@ __global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(NTS) k_resample_sp
     }
     __syncthreads();
     const int n = s_n;
-    if (s_bad || n == 0) {  // the same in every CTA of the cluster
+    const int bad_pay = s_bad;
+    __syncthreads();  // (the pass below sets s_bad: every thread has read it)
+    if (bad_pay || n == 0) {  // the same in every CTA of the cluster
         if (rank == 0 && tid == 0) {
             a.token[b] = -1;
-            a.status[b] = s_bad ? ACES_ROW_BAD_Q : 0;
+            a.status[b] = bad_pay ? ACES_ROW_BAD_Q : 0;
         }
         return;
     }

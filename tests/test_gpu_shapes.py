@@ -247,3 +247,27 @@ def test_resample_on_ragged_rows(A, orc, V, offset):
     near = np.array([any(np.isfinite(c) and abs(o["res_target"][b] - c) < 1e-6 * o["res_sum"][b]
                          for c in (o["res_cj"][b], o["res_cjm1"][b])) for b in range(B)])
     assert (tok == o["token"])[~near].all() and near.sum() <= 2
+
+
+@pytest.mark.parametrize("V", [1001, 152064])
+def test_resample_with_a_bad_draft_value_outside_the_payload(A, orc, V):
+    # a NaN or a negative value that one thread of one CTA meets, at the start,
+    # in the middle and at the end of the row: the whole cluster gives the row up
+    bad = [0, 5, 31, 32, V // 3, V // 2, V - 2, V - 1]
+    B, K, k = 2 * len(bad) + 1, 1, 4
+    rng = np.random.default_rng(V + 1)
+    q = rng.random((B, K, V)).astype(np.float32)
+    q /= q.sum(-1, keepdims=True)
+    for i, x in enumerate(bad):
+        q[2 * i, 0, x] = np.nan
+        q[2 * i + 1, 0, x] = -1e-3
+    ids = np.tile(np.array([100, 200, 300, 400], np.int32), (B, K + 1, 1))
+    probs = np.full((B, K + 1, k), 0.15, np.float32)
+    tail = np.full((B, K + 1), 0.4, np.float32)
+    al, st = np.zeros(B, np.int32), np.zeros((B, K + 1), np.int32)
+    u = np.full((B, K + 1), 0.25, np.float32)
+    o = orc.resample_sparse(al, ids, probs, tail, st, q, u)
+    g = A.resample_sparse(_dev(al), _dev(ids), _dev(probs), _dev(tail), _dev(st), _dev(q), _dev(u))
+    np.testing.assert_array_equal(g["status"].cpu().numpy(), o["status"])
+    assert (g["status"].cpu().numpy()[:-1] != 0).all() and g["status"][-1] == 0
+    assert (g["token"].cpu().numpy()[:-1] == -1).all()
