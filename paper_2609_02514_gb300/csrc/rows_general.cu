@@ -457,8 +457,8 @@ __device__ bool binned_row(const RowArgs &a, int r, const RowChunks<DT> &rc, flo
 // of each value is enough: the values of a window below the row max (at most
 // VH_W of them) get a count, one shared-memory atomic per element and no
 // per-element mass.  The exp-sum S of the whole row comes with a row handed
-// over by the fast kernel; otherwise the counting pass sums it in compensated
-// fp32, as the fast kernel does.  A prefix scan over the values then gives,
+// over by the row kernel; otherwise the counting pass sums it in compensated
+// fp32, as the row kernel does.  A prefix scan over the values then gives,
 // exactly in 2^-40 fixed point (count x the value's mass), the value holding
 // the nucleus crossing (first prefix reaching ceil(top_p * S * 2^40)) and the
 // value holding the k-th payload id; the elements of those values (ties are
@@ -508,7 +508,7 @@ __device__ __forceinline__ void warp_append_cap(unsigned long long *arr, int *n,
 
 // (bfloat16 rows; all threads of the CTA)
 // S_in: the row's exp-sum in units of 2^kref for a row handed over by the
-// fast kernel, 0 otherwise.  *n_fin_out gets the row's count of finite ids
+// row kernel, 0 otherwise.  *n_fin_out gets the row's count of finite ids
 // when top_p = 1 or S_in = 0 (its only uses), even when the row is declined.
 __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &rc, float m, float kref, double S_in,
                             unsigned long long *n_fin_out, ValHist *vh, unsigned long long *buf, double *redd,
@@ -737,9 +737,11 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
 // above that range and lists those inside it and the payload's; the ordered
 // list gives the crossing id.  Returns false, having written nothing, when a
 // list is too long or the payload ends below the bins; the binned path then
-// takes the row (it sums a 64-bit mass per id with shared-memory atomics: 297
-// us a call against 158 with this path, 256 rows of 128256 float32 logits of
-// which 213 are handed over).
+// takes the row (it sums a 64-bit mass per id with shared-memory atomics).  256
+// rows of 128256 float32 logits, about 200 of them handed over: 297 us a call
+// with the binned path, 158 with this one, 147 with the second read's work
+// done per hit and fewer rows handed over.  What is left is two more reads of
+// those rows by one CTA each.
 constexpr int DH_W = 4096;    // bins
 constexpr int DH_PAD = 32;    // counters of the ids below them, one per lane
 constexpr int DH_XCAP = 1536; // listed ids around the crossing
