@@ -767,14 +767,13 @@ struct DepthHist {
 };
 
 template <int DT>
-__device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, float m, float kref, double S, DepthHist *h,
+__device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, float m, float kref, double S_in, DepthHist *h,
                           unsigned long long *buf, double *redd, unsigned long long *redu) {
     constexpr int EPC = Elem<DT>::EPC;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const bool all_in = a.top_p >= 1.0f;
-    const unsigned long long tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
     // no id below vt holds the crossing (as in the value histogram)
-    const float g = all_in ? -41.0f : fmaxf(log2f((1.0f - a.top_p) * (float)S / (16.0f * (float)a.V)), -41.0f);
+    const float g = all_in ? -41.0f : fmaxf(log2f((1.0f - a.top_p) * (float)S_in / (16.0f * (float)a.V)), -41.0f);
     const float depth = fmaxf(m - (kref + g) / a.c, a.T * 1e-3f);
     const float inv = (float)(DH_W - 4) / depth, wid_b = depth / (float)(DH_W - 4);
     // the bin of v is round(C + 1 - v * inv) with the integer C = round(m * inv):
@@ -795,6 +794,8 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
     }
     __syncthreads();
     const uint32_t NI = Elem<DT>::NEG_INF_WORD;
+    uint32_t ah = 0u, al = 0u;  // the row's exact mass (20-bit parts: at most 2^11 + 4 ids a thread)
+    static_assert(ACES_MAX_V / NT + 2 * EPC < 1 << 12, "the parts' sums fit");
     for (int c0i = tid; c0i < rc.nch; c0i += NT * DH_U) {
         uint4 w[DH_U];
 #pragma unroll
@@ -806,10 +807,18 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
         for (int u = 0; u < DH_U; ++u)
 #pragma unroll
             for (int e = 0; e < EPC; ++e) {
-                const int bn = bin_of(Elem<DT>::get(w[u], e));
+                const float v = Elem<DT>::get(w[u], e);
+                const int bn = bin_of(v);
                 if (ACES_IN(bn, DH_W + DH_PAD)) atomicAdd(&h->cnt[bn], 1u);
+                uint32_t fh, fl;
+                to_fx_parts(ex2(fmaf(v, a.c, -kref)), fh, fl);
+                ah += fh;
+                al += fl;
             }
     }
+    const unsigned long long all_fx = block_reduce(((unsigned long long)ah << 20) + al, redu, SumU64());
+    const double S = (double)all_fx * FX_INV;
+    const unsigned long long tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * (double)all_fx);
     __syncthreads();
     // ---- the bins around the crossing and the payload's last ----
     {
