@@ -236,34 +236,15 @@ __device__ __forceinline__ float acc_total(unsigned long long acc0, unsigned lon
     return a + b;
 }
 
-// Sum over the chunks U0 <= j < U1 of 2^(z*c - k), two logits per instruction,
-// float32 rows: the same with the rounding error of every add in err (the
-// two-sum of two logits at a time), as close to the sum of exact masses as the
-// general kernel's.  Of 358400 rows of 50000 to 128256 logits 15 are cut one id
-// away from float64, 32 with 32 plain adds a step; 256 rows of 128256 take 157
-// us (153), one wave of rows the same.
-template <int U0, int U1>
-__device__ __forceinline__ float chunks_expsum_err(const uint4 (&w)[UC], float c, float nk, float &err) {
-    err = 0.0f;
-    if constexpr (U0 >= U1) return 0.0f;
-    const unsigned long long c2 = pack2(c, c), nk2 = pack2(nk, nk), m1 = pack2(-1.0f, -1.0f);
-    unsigned long long s = 0ull, e = 0ull;
-    auto add = [&](unsigned long long x) {
-        const unsigned long long t = fadd2(s, x), b = ffma2(s, m1, t);  // b = t - s
-        e = fadd2(e, fadd2(ffma2(ffma2(b, m1, t), m1, s), ffma2(b, m1, x)));
-        s = t;
-    };
+// sum over the chunks of 2^(z*c - k), two logits per instruction
+// (chunks U0 <= j < U1)
+template <int DT, int U0, int U1>
+__device__ __forceinline__ float chunks_expsum(const uint4 (&w)[UC], float c, float nk) {
+    const unsigned long long c2 = pack2(c, c), nk2 = pack2(nk, nk);
+    unsigned long long acc0 = 0ull, acc1 = 0ull;
 #pragma unroll
-    for (int j = U0; j < U1; ++j) {
-        add(ex2_pair(pack2(__uint_as_float(w[j].x), __uint_as_float(w[j].y)), c2, nk2));
-        add(ex2_pair(pack2(__uint_as_float(w[j].z), __uint_as_float(w[j].w)), c2, nk2));
-    }
-    float a, b, ea, eb, sm;
-    unpack2(s, a, b);
-    unpack2(e, ea, eb);
-    two_sum(a, b, sm, err);
-    err += ea + eb;
-    return sm;
+    for (int j = U0; j < U1; ++j) acc_pair(j - U0, chunk_expsum2<DT>(w[j], c2, nk2), acc0, acc1);
+    return acc_total(acc0, acc1);
 }
 
 // maxima of chunks 0..3 and 4..7 (bfloat16: packed over all their pairs,
@@ -508,11 +489,6 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         else e_t += (gs - t) + s_t;
         s_t = t;
     };
-    auto add_sum_err = [&](auto u0, auto u1) {  // (float32)
-        float err;
-        add_sum(chunks_expsum_err<decltype(u0)::value, decltype(u1)::value>(w, a.c, -k_t, err));
-        e_t += err;
-    };
     // the running max of the CTA (a lower bound of the row max at any time)
     auto publish_max = [&](float im) {
         const uint32_t wm = __reduce_max_sync(0xffffffffu, fkey(im));
@@ -532,7 +508,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     }
     if (!BF) {  // (bfloat16: with the other iterations, below)
         raise_ref(im);
-        add_sum_err(std::integral_constant<int, 0>(), std::integral_constant<int, UCS>());
+        add_sum(chunks_expsum<DT, 0, UCS>(w, a.c, -k_t));
     }
     // D: how far below the row max the nucleus crossing (top_p = 1: the
     // payload's end) can lie.  Rows of this call that have finished published
@@ -1336,8 +1312,8 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                     group_maxima<DT>(w, g0, g1);
                     im = fmaxf(g0, g1);
                     raise_ref(im);
-                    if (it > 0) add_sum_err(std::integral_constant<int, 0>(), std::integral_constant<int, UC>());
-                    else add_sum_err(std::integral_constant<int, UCS == UC ? 0 : UCS>(), std::integral_constant<int, UC>());
+                    if (it > 0) add_sum(chunks_expsum<DT, 0, UC>(w, a.c, -k_t));
+                    else add_sum(chunks_expsum<DT, UCS == UC ? 0 : UCS, UC>(w, a.c, -k_t));
                     if (by_depth) publish_max(im);
                 }
                 record_hits(th);

@@ -740,9 +740,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
 // takes the row (it sums a 64-bit mass per id with shared-memory atomics).  256
 // rows of 128256 float32 logits, about 200 of them handed over: 297 us a call
 // with the binned path, 158 with this one, 147 with the second read's work
-// done per hit and fewer rows handed over, 153 with the row's mass summed in
-// the first read (with the row kernel's sum 10 of 3072 rows at T = 1.2 were cut
-// one id away from float64, 3 with the exact one).  What is left is two more reads of
+// done per hit and fewer rows handed over.  What is left is two more reads of
 // those rows by one CTA each.
 constexpr int DH_W = 4096;    // bins
 constexpr int DH_PAD = 32;    // counters of the ids below them, one per lane
