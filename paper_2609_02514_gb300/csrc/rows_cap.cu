@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     __shared__ float s_thlo, s_zx;
     __shared__ int s_dbins, s_xb;  // s_dbins: D in depth bins (-1: no hints yet)
     __shared__ int s_skm;          // bfloat16: the sketch-led pass (no counting while streaming); float32: see there
-    __shared__ uint32_t s_mr;  // order key of the running max
+    __shared__ uint32_t s_m1, s_mr;  // order keys of the sample's max and of the running max after it
     __shared__ double s_Snuc;
     __shared__ float s_inv_S;
     __shared__ unsigned long long s_cut, s_cumL_fx, s_tg;
@@ -410,8 +410,9 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         s_nl = 0;
         s_fb = 0;
         s_nstar = INT_MAX;
-        s_mr = fkey(-INFINITY);
+        s_m1 = s_mr = fkey(-INFINITY);
     }
+    __syncthreads();  // (other warps add to these before the next barrier)
     // the depths published by the call's finished rows (read by warp 0 only,
     // once: they change while this row streams)
     int hr = 0, hc0 = 0, hc1 = 0, hs = 0, hf = 0;
@@ -490,11 +491,10 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         s_t = t;
     };
     // the running max of the CTA (a lower bound of the row max at any time)
-    auto publish_max = [&](float im) {
+    auto publish_max = [&](float im, uint32_t *to) {
         const uint32_t wm = __reduce_max_sync(0xffffffffu, fkey(im));
-        if (lane == 0 && wm > fkey(-INFINITY)) atomicMax(&s_mr, wm);
+        if (lane == 0 && wm > fkey(-INFINITY)) atomicMax(to, wm);
     };
-    auto running_max = [&]() -> float { return fkey_inv(*reinterpret_cast<volatile uint32_t *>(&s_mr)); };
 
     // iteration 0 begins with a strided sample (1/8 to 1/16 of a large row,
     // spread over it): chunks u < UCS
@@ -534,10 +534,13 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             s_skm = BF ? all_in || (hr >= HINT_MIN && (long long)hs * SHORT_DEN >= (long long)hr * SHORT_NUM) : hf > hr / 16;
         }
     }
-    publish_max(im);
+    publish_max(im, &s_m1);
     if (tid == 0) s_xb = xb0;
     __syncthreads();
-    const float m1 = running_max();  // the sample's max
+    // the sample's max: the same for every warp (later maxima go to another
+    // word, as the first warps publish them while the last ones read this)
+    const float m1 = fkey_inv(s_m1);
+    auto running_max = [&]() -> float { return fmaxf(m1, fkey_inv(*reinterpret_cast<volatile uint32_t *>(&s_mr))); };
     const bool have = m1 > -INFINITY && m1 < INFINITY;
     const int hbins = s_dbins;
     const bool hinted = have && hbins > 0;
@@ -726,7 +729,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                 const uint32_t im2 = group_maxima<DT>(w, g0, g1);
                 im = fmaxf(g0, g1);
                 raise_ref(im);
-                if (COUNT) publish_max(im);
+                if (COUNT) publish_max(im, &s_mr);
                 uint32_t any = 0u;  // chunk positions where some lane of the warp reaches thb
                 if (COUNT) {
                     uint32_t hb = 0u;
@@ -1314,7 +1317,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                     raise_ref(im);
                     if (it > 0) add_sum(chunks_expsum<DT, 0, UC>(w, a.c, -k_t));
                     else add_sum(chunks_expsum<DT, UCS == UC ? 0 : UCS, UC>(w, a.c, -k_t));
-                    if (by_depth) publish_max(im);
+                    if (by_depth) publish_max(im, &s_mr);
                 }
                 record_hits(th);
             }

@@ -149,6 +149,32 @@ def test_float32_rows_by_depth_histogram(A, orc, V, offset, shift, top_p):
     assert res["checked_seqs"] >= 2, res
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("B", [20, 50, 250])           # CTAs of 1024, 512 and 256 threads
+@pytest.mark.parametrize("top_p", [0.9, 1.0])
+def test_rows_whose_sample_is_masked(A, orc, dtype, B, top_p):
+    # the row kernel's sample is tiles 3 t mod 128, t < 64, of 32 chunks: all of
+    # it -inf, a few ids left outside it; every third row keeps all its ids, so
+    # that the depths of finished rows are known
+    V = 128 * 32 * (8 if dtype == "bf16" else 4)
+    w = gen.make_workload(B, 4, V, dtype, T=0.9, top_p=top_p, k=16, seed=89)
+    inp = gen.generate(w)
+    rng = np.random.default_rng(89)
+    z = (rng.standard_normal((B, 5, V)) * 3.0).astype(np.float32)
+    tile = np.arange(V) // (V // 128)
+    out = np.flatnonzero(~np.isin(tile, 3 * np.arange(64) % 128))
+    for r in range(B * 5):
+        if r % 3:
+            row = z[r // 5, r % 5]
+            keep = rng.choice(out, 40, replace=False)
+            left = row[keep].copy()
+            row[:] = -np.inf
+            row[keep] = left
+    inp["z"] = _logits(z, dtype)
+    res, _, _ = _verify(A, orc, w, inp)
+    assert res["checked_seqs"] >= 0.9 * B
+
+
 # ---------------------------------------------------------------------------
 # payloads and nuclei around the ranking limits
 
