@@ -247,6 +247,36 @@ __device__ __forceinline__ float chunks_expsum(const uint4 (&w)[UC], float c, fl
     return acc_total(acc0, acc1);
 }
 
+// The same for float32 rows, with the rounding error of every add in err (the
+// two-sum of two logits at a time): rows off the 16-byte grid, which without
+// the single-pass kernel are summed exactly by the general one.  Cut one id away from
+// float64, of 128000 rows each of 50003 and 20001 logits: 5 and 2, with plain
+// adds 7 and 5, by the general kernel 9 and 0.  Rows on the grid keep the
+// plain adds (11 of 128000 rows of 50000, 12 before; 3% faster).
+template <int U0, int U1>
+__device__ __forceinline__ float chunks_expsum_err(const uint4 (&w)[UC], float c, float nk, float &err) {
+    err = 0.0f;
+    if constexpr (U0 >= U1) return 0.0f;
+    const unsigned long long c2 = pack2(c, c), nk2 = pack2(nk, nk), m1 = pack2(-1.0f, -1.0f);
+    unsigned long long s = 0ull, e = 0ull;
+    auto add = [&](unsigned long long x) {
+        const unsigned long long t = fadd2(s, x), b = ffma2(s, m1, t);  // b = t - s
+        e = fadd2(e, fadd2(ffma2(ffma2(b, m1, t), m1, s), ffma2(b, m1, x)));
+        s = t;
+    };
+#pragma unroll
+    for (int j = U0; j < U1; ++j) {
+        add(ex2_pair(pack2(__uint_as_float(w[j].x), __uint_as_float(w[j].y)), c2, nk2));
+        add(ex2_pair(pack2(__uint_as_float(w[j].z), __uint_as_float(w[j].w)), c2, nk2));
+    }
+    float a, b, ea, eb, sm;
+    unpack2(s, a, b);
+    unpack2(e, ea, eb);
+    two_sum(a, b, sm, err);
+    err += ea + eb;
+    return sm;
+}
+
 // maxima of chunks 0..3 and 4..7 (bfloat16: packed over all their pairs,
 // unpacked once); returns the packed max of both
 template <int DT>
@@ -490,6 +520,16 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         else e_t += (gs - t) + s_t;
         s_t = t;
     };
+    auto add_chunks = [&](auto u0, auto u1) {  // (float32)
+        constexpr int U0 = decltype(u0)::value, U1 = decltype(u1)::value;
+        if constexpr (RAGGED) {
+            float err;
+            add_sum(chunks_expsum_err<U0, U1>(w, a.c, -k_t, err));
+            e_t += err;
+        } else {
+            add_sum(chunks_expsum<DT, U0, U1>(w, a.c, -k_t));
+        }
+    };
     // the running max of the CTA (a lower bound of the row max at any time)
     auto publish_max = [&](float im, uint32_t *to) {
         const uint32_t wm = __reduce_max_sync(0xffffffffu, fkey(im));
@@ -505,10 +545,6 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
 #pragma unroll
         for (int u = 1; u < UCS; ++u) sm2 = max2<DT>(sm2, chunk_max2<DT>(w[u]));
         im = max2_value<DT>(sm2);
-    }
-    if (!BF) {  // (bfloat16: with the other iterations, below)
-        raise_ref(im);
-        add_sum(chunks_expsum<DT, 0, UCS>(w, a.c, -k_t));
     }
     // D: how far below the row max the nucleus crossing (top_p = 1: the
     // payload's end) can lie.  Rows of this call that have finished published
@@ -545,6 +581,15 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     const int hbins = s_dbins;
     const bool hinted = have && hbins > 0;
     const float D = (float)(hinted ? hbins : NSB) * (a.T / SPB);
+    if (!BF) {  // (bfloat16: with the other iterations, below)
+        // one reference for all threads (the final one, unless the row max lies
+        // outside the sample and across an integer of log2): an id's mass then
+        // has the same rounding in S as in the sums that find the crossing (a
+        // reference per thread: 15 of 128000 rows of 50000 logits cut one id
+        // away from float64, 11 with one)
+        raise_ref(have ? fmaxf(m1, im) : im);
+        add_chunks(std::integral_constant<int, 0>(), std::integral_constant<int, UCS>());
+    }
 
     // dependent loads of the accept test, consumed at the end
     float zx = 0.f, qx = 0.f, ux = 0.f;
@@ -1315,8 +1360,8 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                     group_maxima<DT>(w, g0, g1);
                     im = fmaxf(g0, g1);
                     raise_ref(im);
-                    if (it > 0) add_sum(chunks_expsum<DT, 0, UC>(w, a.c, -k_t));
-                    else add_sum(chunks_expsum<DT, UCS == UC ? 0 : UCS, UC>(w, a.c, -k_t));
+                    if (it > 0) add_chunks(std::integral_constant<int, 0>(), std::integral_constant<int, UC>());
+                    else add_chunks(std::integral_constant<int, UCS == UC ? 0 : UCS>(), std::integral_constant<int, UC>());
                     if (by_depth) publish_max(im, &s_mr);
                 }
                 record_hits(th);
