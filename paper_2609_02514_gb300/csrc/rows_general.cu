@@ -730,8 +730,8 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
 // the float32 counterpart of the value histogram, and the second try for
 // bfloat16.  One read counts the ids in DH_W equal bins of depth below the
 // max, down to a value the crossing cannot lie below (top_p = 1: to where an
-// id's mass is below 2^-41), and sums the row's 2^-40 masses; a bin's ids each carry at least its lower and at
-// most its upper edge's mass, so bounds of the cumulative mass give a first
+// id's mass is below 2^-41), and sums the row's 2^-40 masses; a bin's ids each
+// carry at least its lower and at most its upper edge's mass, so bounds of the cumulative mass give a first
 // and a last bin between which the crossing lies (about 0.5% of the mass apart
 // with bins of T / 200).  A second read sums the exact 2^-40 masses of the ids
 // above that range and lists those inside it and the payload's; the ordered
@@ -743,8 +743,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
 // done per hit and fewer rows handed over, 153 with the row's exact mass summed
 // in the first read (as the binned path does; with the row kernel's float32 sum
 // 117 of 46080 rows were cut one id away from float64, 34 with the exact one).
-// What is left is two more reads of
-// those rows by one CTA each.
+// What is left is two more reads of those rows by one CTA each.
 constexpr int DH_W = 4096;    // bins
 constexpr int DH_PAD = 32;    // counters of the ids below them, one per lane
 constexpr int DH_XCAP = 1536; // listed ids around the crossing
