@@ -1325,8 +1325,9 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         // chunk position that has any; the ids are extracted after the stream
         auto record_hits = [&](float th) {
             if (!__any_sync(0xffffffffu, im >= th)) return;
-            // (past the capacity the row goes to the general kernel)
-            if (*reinterpret_cast<volatile int *>(&s_nrec) > CREC) return;
+            // (past the capacity the row goes to the general kernel; the counter
+            // changes meanwhile, so one lane's reading decides for its warp)
+            if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile int *>(&s_nrec), 0) > CREC) return;
             uint32_t off = off0;
 #pragma unroll
             for (int u = 0; u < UC; ++u) {

@@ -149,6 +149,20 @@ def test_float32_rows_by_depth_histogram(A, orc, V, offset, shift, top_p):
     assert res["checked_seqs"] >= 2, res
 
 
+@pytest.mark.parametrize("B", [20, 100, 250])          # CTAs of 1024, 512 and 256 threads
+@pytest.mark.parametrize("V", [40000, 40003])
+def test_float32_rows_whose_records_overflow(A, orc, B, V):
+    # equal logits everywhere: every chunk is recorded until the records are
+    # full, and the warps stop recording while others still add to them.  (An
+    # id carries 2.5e-5 of the mass and the crossing lies inside one, so only
+    # draws within 1e-6 of an id's end, one in 12, are flagged.)
+    w = gen.make_workload(B, 1, V, "f32", T=1.0, top_p=0.9001125, k=8, seed=90)
+    inp = gen.generate(w)
+    inp["z"] = np.full_like(inp["z"], 1.5)
+    res, counters, _ = _verify(A, orc, w, inp)
+    assert counters[FALLBACK] == 2 * B and res["checked_seqs"] >= 0.6 * B, (res, counters)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("B", [20, 50, 250])           # CTAs of 1024, 512 and 256 threads
 @pytest.mark.parametrize("top_p", [0.9, 1.0])
