@@ -96,9 +96,9 @@ static aces_status verify_check(const void *target_logits, aces_dtype dt, const 
     return ACES_OK;
 }
 
-// Results depend on neither `lists` (without them the residual draw scans its
-// whole row instead of the stored nucleus) nor `exact` (every row on the
-// general kernel).
+// Results do not depend on `lists` (without them the residual draw scans its
+// whole row instead of the stored nucleus), nor, but for the last bits that
+// aces_verify_exact names, on `exact` (every row on the general kernel).
 aces_status aces::verify_impl(const void *target_logits, aces_dtype dt, const float *draft_probs,
                         const int32_t *draft_tokens, const float *uniforms, int B, int K, int V,
                         float T, float top_p, int32_t *accept_len, int32_t *out_token, int k,

@@ -348,8 +348,8 @@ __host__ __device__ __forceinline__ int next_pow2(int n) {
 }
 
 // 1/S as a float, the same in every kernel: a probability is always
-// e * inv_mass(S) for a mass e, so a row's outputs do not depend on which
-// kernel finished it (and no fp64 divide sits on the row's critical path)
+// e * inv_mass(S) for a mass e, so rows of one nucleus mass S get the same
+// outputs from every kernel (and no fp64 divide sits on the row's critical path)
 __device__ __forceinline__ float inv_mass(double S) { return __frcp_rn((float)S); }
 
 // atomicAdd that releases this CTA's earlier writes (ordered before it by a
@@ -506,6 +506,7 @@ struct RowArgs {
     int it_partial, it_partial2;  // iterations that read the row's partial last tiles (-1: none)
     float samp_frac;
     float inv_ws;          // sample bins per unit of logit: SPB / T
+    float sum_err;         // bound of the float32 exp-sum's relative distance from the exact one
     int nmin;              // float32 first rows: ids the capture must reach
     int sk_gpi, sk_ish;    // bfloat16 sketch: groups per thread and iteration (2: 4 chunks each; 1: 8
                            // chunks of 2^sk_ish iterations)
@@ -566,7 +567,8 @@ __device__ void nonfinite_row(const RowArgs &a, int r) {
 void rows_cap_layout(RowArgs &a, int dt, bool ragged);
 cudaError_t launch_rows_cap(const RowArgs &a, int dt, bool ragged, cudaStream_t s);
 cudaError_t launch_rows_general(const RowArgs &a, int dt, int nseq, cudaStream_t s);
-// aces_verify with two choices, neither of which changes the results: lists =
+// aces_verify with two choices, neither of which changes the results (exact: but
+// for the last bits that aces_verify_exact names): lists =
 // false keeps no nucleus lists (the residual draw scans its row; the call then
 // needs ws_bytes(rows, B, K, lists) bytes of workspace), exact = true hands
 // every row to the general kernel.

@@ -19,8 +19,7 @@
 //             call's finished rows published, plus a margin (before 32 have
 //             finished: those the previous call on the same workspace left,
 //             for bfloat16 rows of the same shape; else NSB bins of T/4).  D
-//             only decides what is kept; every result below is proved from
-//             exact sums.
+//             only decides what is kept, never a result.
 //   keep      bfloat16, counting pass: every id >= (running max - D)
 //             increments a shared-memory counter of its bfloat16 value (a
 //             window of HW values); sketch-led pass (when nearly all finished
@@ -30,10 +29,12 @@
 //             recorded (chunk and index).  The running max only rises, so at
 //             the end every id >= (row max - D) was kept (or, sketch-led,
 //             lies in a group whose max reaches it).
-//   finish    from the exact row max and exp-sum, exact 2^-40 fixed-point
+//   finish    from the exact row max and the exp-sum, exact 2^-40 fixed-point
 //             masses give the nucleus crossing (a crossing below the kept
 //             values: a second counting pass over the row; a capacity
-//             exceeded: the exact general kernel):
+//             exceeded: the exact general kernel; float32 rows and rows off
+//             the 16-byte grid whose crossing depends on the exp-sum's rounding:
+//             a second read for the exact mass):
 //             bfloat16  (sketch-led: the groups reaching row max - D are read
 //                       back and their ids counted first) the CTA scans the
 //                       value counts for the crossing value, the number j of
@@ -65,6 +66,7 @@
 // On launches of four waves or more, the j-th CTA each SM starts with waits
 // j x 10 us first, so that the first wave's epilogues do not coincide.
 #include <climits>
+#include <cmath>
 #include <mutex>
 #include <type_traits>
 
@@ -247,36 +249,6 @@ __device__ __forceinline__ float chunks_expsum(const uint4 (&w)[UC], float c, fl
     return acc_total(acc0, acc1);
 }
 
-// The same for float32 rows, with the rounding error of every add in err (the
-// two-sum of two logits at a time): rows off the 16-byte grid, which without
-// the single-pass kernel are summed exactly by the general one.  Cut one id away from
-// float64, of 128000 rows each of 50003 and 20001 logits: 5 and 2, with plain
-// adds 7 and 5, by the general kernel 9 and 0.  Rows on the grid keep the
-// plain adds (11 of 128000 rows of 50000, 12 before; 3% faster).
-template <int U0, int U1>
-__device__ __forceinline__ float chunks_expsum_err(const uint4 (&w)[UC], float c, float nk, float &err) {
-    err = 0.0f;
-    if constexpr (U0 >= U1) return 0.0f;
-    const unsigned long long c2 = pack2(c, c), nk2 = pack2(nk, nk), m1 = pack2(-1.0f, -1.0f);
-    unsigned long long s = 0ull, e = 0ull;
-    auto add = [&](unsigned long long x) {
-        const unsigned long long t = fadd2(s, x), b = ffma2(s, m1, t);  // b = t - s
-        e = fadd2(e, fadd2(ffma2(ffma2(b, m1, t), m1, s), ffma2(b, m1, x)));
-        s = t;
-    };
-#pragma unroll
-    for (int j = U0; j < U1; ++j) {
-        add(ex2_pair(pack2(__uint_as_float(w[j].x), __uint_as_float(w[j].y)), c2, nk2));
-        add(ex2_pair(pack2(__uint_as_float(w[j].z), __uint_as_float(w[j].w)), c2, nk2));
-    }
-    float a, b, ea, eb, sm;
-    unpack2(s, a, b);
-    unpack2(e, ea, eb);
-    two_sum(a, b, sm, err);
-    err += ea + eb;
-    return sm;
-}
-
 // maxima of chunks 0..3 and 4..7 (bfloat16: packed over all their pairs,
 // unpacked once); returns the packed max of both
 template <int DT>
@@ -362,6 +334,36 @@ __device__ __forceinline__ unsigned long long id_fx(float v, float c, float kref
     return to_fx(ex2(fmaf(v, c, -kref)));
 }
 
+// The row's mass against its reference kref as the general kernel sums it: in
+// 2^-40 units, exactly (a second read of the row; all NTC threads).
+template <int DT, int NTC, bool RAGGED>
+__device__ __noinline__ unsigned long long exact_mass(const char *row, int V, float c, float kref, unsigned long long *red) {
+    constexpr int EPC = Elem<DT>::EPC, U = 4;  // loads in flight
+    const RowChunks<DT, RAGGED> rc(row, V);
+    const uint32_t ni = Elem<DT>::NEG_INF_WORD;
+    unsigned long long sum = 0ull;
+    for (int c0 = threadIdx.x; c0 < rc.nch; c0 += NTC * U) {
+        uint4 w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ch = c0 + u * NTC;
+            w[u] = ch < rc.nch ? rc.load(ch) : make_uint4(ni, ni, ni, ni);
+        }
+        uint32_t hi = 0u, lo = 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int e = 0; e < EPC; ++e) {
+                uint32_t h, l;
+                to_fx_parts(ex2(fmaf(Elem<DT>::get(w[u], e), c, -kref)), h, l);
+                hi += h;
+                lo += l;
+            }
+        sum += ((unsigned long long)hi << 20) + lo;
+    }
+    return block_reduce_n<NTC>(sum, red, SumU64());
+}
+
 // NTC: threads per CTA, 1024 / NTC CTAs per SM
 // (RAGGED: rows off the 16-byte grid; a build of its own, as the edges cost
 // the other one registers: 128 x 17 rows of 128256 205 -> 213 us)
@@ -376,6 +378,14 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     using E = Elem<DT>;
     constexpr int EPC = E::EPC;
     constexpr bool BF = DT == ACES_BF16;
+    // The cut of float32 rows, and of bfloat16 rows off the 16-byte grid, is the
+    // one of the row's exact mass, whichever kernel finishes the row: the
+    // float32 sum places the target within a bound (sum_err), and where the cut
+    // is not the same over that whole range the row is read again for its exact
+    // mass.  (Of 128000 float32 rows 2 to 12 were cut one id away from float64 by
+    // the float32 sum alone.)  Off the grid the mass of top_p = 1 rows is the
+    // exact one too.
+    constexpr bool EXACT_CUT = !BF || RAGGED;
     extern __shared__ __align__(16) unsigned char smem[];
     // bfloat16: [HPAD dummies, value counts: HW u32 | sketch: SKG u16 | ids >=
     //           the payload's last value: PCAP u64]; the list of re-read groups
@@ -402,9 +412,11 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     __shared__ uint32_t s_m1, s_mr;  // order keys of the sample's max and of the running max after it
     __shared__ double s_Snuc;
     __shared__ float s_inv_S;
-    __shared__ unsigned long long s_cut, s_cumL_fx, s_tg;
+    __shared__ unsigned long long s_cut, s_cumL_fx;
+    __shared__ unsigned long long s_tg, s_th;  // the target lies in [s_tg, s_th] (one value when it is exact)
     __shared__ unsigned long long s_redu[NWC], s_above, s_evs;
     __shared__ uint32_t s_redc[NWC], s_cab, s_cnvs;
+    __shared__ int s_settled;
 
     const int r = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -521,14 +533,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         s_t = t;
     };
     auto add_chunks = [&](auto u0, auto u1) {  // (float32)
-        constexpr int U0 = decltype(u0)::value, U1 = decltype(u1)::value;
-        if constexpr (RAGGED) {
-            float err;
-            add_sum(chunks_expsum_err<U0, U1>(w, a.c, -k_t, err));
-            e_t += err;
-        } else {
-            add_sum(chunks_expsum<DT, U0, U1>(w, a.c, -k_t));
-        }
+        add_sum(chunks_expsum<DT, decltype(u0)::value, decltype(u1)::value>(w, a.c, -k_t));
     };
     // the running max of the CTA (a lower bound of the row max at any time)
     auto publish_max = [&](float im, uint32_t *to) {
@@ -583,10 +588,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     const float D = (float)(hinted ? hbins : NSB) * (a.T / SPB);
     if (!BF) {  // (bfloat16: with the other iterations, below)
         // one reference for all threads (the final one, unless the row max lies
-        // outside the sample and across an integer of log2): an id's mass then
-        // has the same rounding in S as in the sums that find the crossing (a
-        // reference per thread: 15 of 128000 rows of 50000 logits cut one id
-        // away from float64, 11 with one)
+        // outside the sample and across an integer of log2)
         raise_ref(have ? fmaxf(m1, im) : im);
         add_chunks(std::integral_constant<int, 0>(), std::integral_constant<int, UCS>());
     }
@@ -603,9 +605,9 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     bool short_row = false;  // (bfloat16) few ids reach the crossing: published for later rows' pass
 
     // reduces the row max, the reference and the exp-sum S (fp32 two-sum tree,
-    // fp64 in thread 0 only, which also leaves the nucleus target in s_tg:
-    // valid after the next barrier); true when the row is not a distribution
-    // (handled)
+    // fp64 in thread 0 only, which also leaves the nucleus target in s_tg and
+    // s_th: valid after the next barrier); true when the row is not a
+    // distribution (handled)
     auto finish_sums = [&]() -> bool {
         if (a.K > 0) {
             bq = r / (a.K + 1);
@@ -676,7 +678,9 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         if (tid == 0) {
             S = (double)sh + (double)sl;
-            s_tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
+            const double t = (double)a.top_p * S * (double)FX_SCALE, err = EXACT_CUT ? t * (double)a.sum_err : 0.0;
+            s_tg = all_in ? 0ull : (unsigned long long)ceil(t - err);
+            s_th = all_in ? 0ull : (unsigned long long)ceil(t + err);
         }
         if (!(sh > 0.0f && sh < INFINITY) || !(m < INFINITY) || !(kref < 1e30f)) {
             nonfinite_row<NTC>(a, r);
@@ -684,6 +688,24 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             return true;
         }
         return false;
+    };
+    // replaces S (thread 0) and the target by those of the row's exact mass
+    // (all threads)
+    bool exact_S = false;
+    auto make_exact = [&]() {
+        const unsigned long long fx = exact_mass<DT, NTC, RAGGED>(rc.row(), a.V, a.c, kref, s_redu);
+        if (tid == 0) {
+            S = (double)fx * FX_INV;
+            s_tg = s_th = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * (double)fx);
+        }
+        __syncthreads();
+        exact_S = true;
+    };
+    // hands the row to the general kernel (all threads), whose value histogram
+    // takes S from here
+    auto hand_over = [&]() {
+        if (BF && RAGGED && !exact_S) make_exact();
+        if (tid == 0) fallback_row(a, r, m, kref, S);
     };
 
     if constexpr (BF) {
@@ -806,9 +828,10 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         if (count_on) stream(std::true_type());
         else stream(std::false_type());
         if (finish_sums()) return;
+        if (RAGGED && all_in) make_exact();
         const uint32_t km = __float_as_uint(m) >> 16;
         if (a.force_fb || !(m > 0.0f)) {
-            if (tid == 0) fallback_row(a, r, m, kref, S);
+            hand_over();
             return;
         }
         auto vmass = [&](int idx) { return id_fx(val16(0x8000u + thb0 + (uint32_t)idx), a.c, kref); };
@@ -816,10 +839,11 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         // from the counts of values thc..m (all threads, VPT consecutive
         // values each, from the top).  Returns 0, or 1 when they lie below
         // the counted values, 2 when more ids than the re-read keeps share
-        // the payload's last value ----
+        // the payload's last value (scan_once: 3 when the cut depends on the
+        // error of S) ----
         // (L, vs, vr, j, n_nuc and nge are set when it returns 0)
         int vs = -1, vr = -1, j = 0, n_nuc = -1, nge = 0;
-        auto scan = [&](uint32_t thc) -> int {
+        auto scan_once = [&](uint32_t thc) -> int {
             constexpr int VPT = HW / NTC;
             const int top = (int)(km - thb0) - VPT * tid, lo = (int)(thc - thb0);
             uint32_t cn[VPT];
@@ -882,6 +906,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                         while (q * e1[i] < rem) ++q;
                         while (q > 1ull && (q - 1ull) * e1[i] >= rem) --q;
                         s_j = (int)q;
+                        s_settled = cm + q * e1[i] >= s_th;
                     }
                     cm += mm;
                     cc += cn[i];
@@ -907,6 +932,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             vs = s_vs;
             j = s_j;
             if (!all_in && vs < 0) return 1;
+            if (EXACT_CUT && !all_in && !s_settled) return 3;
             const uint32_t nn = all_in ? (uint32_t)a.V : s_cab + (uint32_t)j;  // (at most V)
             const unsigned long long nuc = s_above + (unsigned long long)j * s_evs;
             n_nuc = all_in ? -1 : (int)nn;
@@ -932,6 +958,13 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                 s_inv_S = inv_mass(s_Snuc);
             }
             return 0;
+        };
+        auto scan = [&](uint32_t thc) -> int {
+            for (;;) {
+                const int f = scan_once(thc);
+                if (f != 3) return f;
+                make_exact();  // (then it is settled)
+            }
         };
         // ---- reading groups of the sketch back ----
         const int ng_all = gpi == 2 ? nit * NTC * 2 : ((nit + (1 << ish) - 1) >> ish) * NTC;
@@ -1139,7 +1172,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             fb = scan(thb0);
         }
         if (fb != 0) {
-            if (tid == 0) fallback_row(a, r, m, kref, S);
+            hand_over();
             return;
         }
         const uint32_t vsb = thb0 + (uint32_t)vs;  // crossing value (bit pattern)
@@ -1150,7 +1183,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             if (!pay_ready) {
                 const int ng = compact(vrb, glist);
                 if (ng > GCAP) {
-                    if (tid == 0) fallback_row(a, r, m, kref, S);
+                    hand_over();
                     return;
                 }
                 if (tid == 0) s_npay = 0;
@@ -1159,7 +1192,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             }
             const int npay = pay_ready ? s_ng : s_npay;
             if (npay != nge) {  // (cannot happen: the counts and the ids agree)
-                if (tid == 0) fallback_row(a, r, m, kref, S);
+                hand_over();
                 return;
             }
             // order them (descending order value)
@@ -1369,9 +1402,10 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             }
         }
         if (finish_sums()) return;
+        if (RAGGED && all_in) make_exact();
         const int nrec = s_nrec;
         if (a.force_fb || nrec > CREC) {
-            if (tid == 0) fallback_row(a, r, m, kref, S);
+            hand_over();
             return;
         }
         const float thc = by_depth ? m - D : thlo;  // every id >= thc was recorded
@@ -1393,10 +1427,9 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         __syncthreads();
         const int nl = s_nl;
         if (nl > LCAP) {
-            if (tid == 0) fallback_row(a, r, m, kref, S);
+            hand_over();
             return;
         }
-        const unsigned long long tg = s_tg;
         // counts of the listed ids in bins of T/8 below m; a bin's ids each
         // carry at least its lower edge's mass, so the first bin where that
         // lower bound of the cumulative mass reaches the target holds or
@@ -1437,7 +1470,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             pm -= lm;
             pc -= lc;
             // 1e-4 covers the fp32 rounding of the bound and of S
-            const float tgf = (float)tg * (1.0f / FX_SCALE) * (1.0f + 1e-4f);
+            const float tgf = (float)s_tg * (1.0f / FX_SCALE) * (1.0f + 1e-4f);
             int hit = -1;
             unsigned ncand = 0u;
 #pragma unroll
@@ -1468,7 +1501,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         __syncthreads();
         if (s_fb || s_n > WCAP) {
-            if (tid == 0) fallback_row(a, r, m, kref, S);
+            hand_over();
             return;
         }
         // candidates: the listed ids in bins up to bsel
@@ -1566,8 +1599,10 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             unsigned long long loc = 0ull, tot;
             for (int i = lo; i < hi; ++i) loc += efx[i];
             const unsigned long long ex = block_exscan_n<NTC>(loc, s_redu, &tot);
-            unsigned long long c = ex;
-            if (!all_in)
+            unsigned long long c;
+            auto find = [&]() {
+                const unsigned long long tg = s_tg;
+                c = ex;
                 for (int i = lo; i < hi; ++i) {
                     const unsigned long long prev = c;
                     c += efx[i];
@@ -1576,7 +1611,17 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
                         s_above = c;
                     }
                 }
-            __syncthreads();
+                __syncthreads();
+            };
+            if (!all_in) {
+                find();
+                if (s_nstar != INT_MAX && s_above < s_th) {  // the cut depends on the error of S
+                    make_exact();
+                    if (tid == 0) s_nstar = INT_MAX;
+                    __syncthreads();
+                    find();
+                }
+            }
             const int nstar = all_in ? n - 1 : s_nstar;  // (INT_MAX: below the list)
             if (nstar != INT_MAX) {
                 const int Lw = min(nstar + 1, a.k);
@@ -1598,7 +1643,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         __syncthreads();
         if (s_nstar == INT_MAX) {
-            if (tid == 0) fallback_row(a, r, m, kref, S);
+            hand_over();
             return;
         }
         // keep the nucleus for the residual step when it fits
@@ -1715,6 +1760,15 @@ void rows_cap_layout(RowArgs &a, int dt, bool ragged) {
             if (ragged && tile == ntile - 2) a.it_partial2 = t / tpi;
         }
     a.inv_ws = (float)(SPB / (double)a.T);
+    // Bound of the relative difference between the row kernel's float32 sum and
+    // the exact 2^-40 one.  Each rounds an id's exponent, at depth d = kref -
+    // z c, by at most d 2^-24 (d 2^-24 ln 2 of its mass), and the mean depth,
+    // weighted by mass, is at most log2(V) + 1 (the masses' entropy less log2
+    // of the total, which is at least 1/2); each has ex2's own error, at most
+    // 2^-22; the float32 sum rounds each mass in at most 8 adds; the exact one
+    // drops less than 2^-40 of every id.
+    a.sum_err = (float)(2.0 * (0.6931472 * ldexp(log2((double)a.V) + 1.0, -24) + ldexp(1.0, -22)) + ldexp(1.0, -21) +
+                        ldexp((double)a.V, -39));
     a.nmin = 2 * a.k + 64 > 256 ? 2 * a.k + 64 : 256;
     // sketch groups: 4 chunks (two per thread and iteration) when they fit,
     // else 8 chunks of 2^sk_ish iterations

@@ -36,9 +36,9 @@ __device__ void finish_row(const RowArgs &a, int r, const char *row, float kref,
                            unsigned long long cut, int flags, const unsigned long long *sorted,
                            int L, double *redd) {
     const int tid = threadIdx.x;
-    // same formulas as the fast row kernel, so a row gets bit-identical
-    // outputs whichever kernel finishes it: p = e * inv_mass(S_nuc), and the
-    // tail from the exact fixed-point sum of the payload masses
+    // same formulas as the single-pass row kernel, so a cut and a nucleus mass
+    // give the same bits in both: p = e * inv_mass(S_nuc), and the tail from
+    // the exact fixed-point sum of the payload masses
     const float inv_S = inv_mass(S_nuc);
     unsigned long long loc = 0ull;
     if (a.k > 0) {
@@ -156,12 +156,12 @@ struct SelState {
 };
 
 // One radix selection.  mode 0: first id where the cumulative mass reaches
-// target_fx (as a double); mode 1: the kk-th id (1-based) by count.
+// ceil(top_p * S); mode 1: the kk-th id (1-based) by count.
 // Returns the order value of the selected id; st->above / above_cnt hold the
 // mass / count strictly before it; when want_S, st->S_fx gets the total mass.
 template <int DT>
 __device__ unsigned long long radix_select(const RowChunks<DT> &rc, float kref, float c, int mode,
-                                           double target, unsigned kk, bool want_S, SelState *st) {
+                                           double top_p, unsigned kk, bool want_S, SelState *st) {
     const int tid = threadIdx.x;
     if (tid == 0) {
         st->prefix = 0ull;
@@ -170,6 +170,7 @@ __device__ unsigned long long radix_select(const RowChunks<DT> &rc, float kref, 
         st->done = 0;
         st->S_fx = 0ull;
     }
+    unsigned long long target = 0ull;  // (thread 0)
     int nbits = 0;
     for (int s = 56; s >= 0; s -= 8) {
         // digits known in advance: the low 16 key bits of a bf16 value are 0,
@@ -204,14 +205,14 @@ __device__ unsigned long long radix_select(const RowChunks<DT> &rc, float kref, 
                 unsigned long long S = 0ull;
                 for (int d = 0; d < 256; ++d) S += st->mass[d];
                 st->S_fx = S;
-                if (mode == 0) target *= (double)S;  // target arrives as top_p
+                if (mode == 0) target = (unsigned long long)ceil(top_p * (double)S);
             }
             int sel = -1;
             int lowest = -1;
             for (int d = 255; d >= 0; --d) {
                 if (st->cnt[d] == 0u) continue;
                 lowest = d;
-                bool hit = mode == 0 ? ((double)(st->above + st->mass[d]) >= target)
+                bool hit = mode == 0 ? (st->above + st->mass[d] >= target)
                                      : (st->above_cnt + st->cnt[d] >= kk);
                 if (hit) {
                     sel = d;
@@ -270,7 +271,7 @@ struct BinState {
     unsigned long long ps[GB_CAP];  // order values of the payload bins
     int nx, np_, bx, bk, ok, nbelow;
     unsigned long long above;       // mass of the bins before the crossing bin
-    double target;
+    unsigned long long target;      // the nucleus target, ceil(top_p * S_fx)
 };
 
 // appends o to arr[*n] for every lane with take (one atomic per warp)
@@ -331,7 +332,7 @@ __device__ bool binned_row(const RowArgs &a, int r, const RowChunks<DT> &rc, flo
             if (W == 0) {  // the first window sees every element: the total
                 unsigned long long S = far_mass;
                 for (int j = 0; j < WN; ++j) S += bs->mass[j];
-                bs->target = (double)a.top_p * (double)S;
+                bs->target = (unsigned long long)ceil((double)a.top_p * (double)S);
                 bs->S_fx = S;
             }
             unsigned long long above = bs->above;
@@ -339,7 +340,7 @@ __device__ bool binned_row(const RowArgs &a, int r, const RowChunks<DT> &rc, flo
             const int wend = W + WN;
             if (!all_in && bs->bx == -2) {
                 for (int d = W; d < wend; ++d) {
-                    if ((double)(above + bs->mass[d - W]) >= bs->target) {
+                    if (above + bs->mass[d - W] >= bs->target) {
                         bs->bx = d;
                         break;
                     }
@@ -423,7 +424,7 @@ __device__ bool binned_row(const RowArgs &a, int r, const RowChunks<DT> &rc, flo
         for (int i = lo; i < hi; ++i) {
             const unsigned long long prev = cum;
             cum += bs->ps[i];
-            if ((double)prev < bs->target && (double)cum >= bs->target) {  // one id crosses
+            if (prev < bs->target && cum >= bs->target) {  // one id crosses
                 bs->bk = i;
                 redd[0] = (double)cum * FX_INV;
             }
@@ -742,7 +743,9 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
 // with the binned path, 158 with this one, 147 with the second read's work
 // done per hit and fewer rows handed over, 153 with the row's exact mass summed
 // in the first read (as the binned path does; with the row kernel's float32 sum
-// 117 of 46080 rows were cut one id away from float64, 34 with the exact one).
+// 117 of 46080 rows were cut one id away from float64, 34 with the exact one;
+// 163 since the row kernel reads the rows it finishes again where the cut
+// depends on that sum's error).
 // What is left is two more reads of those rows by one CTA each.
 constexpr int DH_W = 4096;    // bins
 constexpr int DH_PAD = 32;    // counters of the ids below them, one per lane

@@ -163,6 +163,51 @@ def test_float32_rows_whose_records_overflow(A, orc, B, V):
     assert counters[FALLBACK] == 2 * B and res["checked_seqs"] >= 0.6 * B, (res, counters)
 
 
+# ---------------------------------------------------------------------------
+# the cut is the one of the row's exact mass
+
+
+@pytest.mark.parametrize("dtype,V", [("f32", 20000), ("f32", 20001), ("bf16", 20001), ("bf16", 50003)])
+@pytest.mark.parametrize("n", [256, 510, 2048, 12000])
+@pytest.mark.parametrize("exact", [False, True])
+def test_cut_at_half_of_equal_masses(A, dtype, V, n, exact):
+    # n ids of one value each, top_p = 1/2: exactly n / 2 of them are the
+    # nucleus.  A total wrong in its last bits moves the cut to n / 2 + 1 in
+    # half the rows (half a last bit of float32 is 6e-8, an id's share 1e-4)
+    B, k = 80, 64
+    rng = np.random.default_rng(n)
+    z = np.full((B, 2, V), -np.inf, np.float32)
+    for b in range(B):
+        for i in range(2):
+            ids = rng.choice(V, n, replace=False) if b % 2 else rng.integers(V - n + 1) + np.arange(n)
+            z[b, i, ids] = rng.uniform(0.3, 9.0)
+    zt = _dev(_logits(z, dtype))
+    q = torch.full((B, 1, V), 1.0 / V, device="cuda")
+    xt, u = torch.zeros(B, 1, dtype=torch.int32, device="cuda"), torch.full((B, 2), 0.5, device="cuda")
+    g = A.verify(zt, q, xt, u, 0.7, 0.5, k, exact=exact)
+    p = g["topk_probs"].cpu().numpy().astype(np.float64)
+    assert (np.abs(p * (n // 2) - 1.0) < 1e-6).all(), np.unique(np.round(1.0 / p, 2))
+
+
+@pytest.mark.parametrize("dtype,V,sigma,T,top_p", [
+    ("f32", 40000, 3.0, 0.9, 0.9), ("f32", 40003, 3.0, 0.9, 0.9), ("f32", 40003, 3.0, 0.9, 1.0),
+    ("f32", 40000, 1.0, 1.0, 0.8), ("bf16", 40003, 3.0, 0.9, 0.9), ("bf16", 40003, 3.0, 0.9, 1.0), ("bf16", 40003, 1.0, 1.0, 0.8)])
+@pytest.mark.parametrize("B", [40, 300])               # one wave, and rows that see finished ones
+def test_a_row_is_the_same_whichever_kernel_finishes_it(A, dtype, V, sigma, T, top_p, B):
+    # repeated calls (the rows that overflow the row kernel's areas depend on
+    # what has finished before) and the general kernel alone: the same bits
+    w = gen.make_workload(B, 2, V, dtype, T=T, top_p=top_p, k=24, seed=91, sigma=sigma, rho=0.9)
+    inp = gen.generate(w)
+    z, q, xt, u = (_dev(inp[key]) for key in ("z", "q", "xt", "u"))
+    first = None
+    for run in range(5):
+        g = A.verify(z, q, xt, u, w.T, w.top_p, w.k, exact=run == 4)
+        if first is None:
+            first = g
+        for key in first:
+            assert torch.equal(g[key], first[key]), (key, run)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("B", [20, 50, 250])           # CTAs of 1024, 512 and 256 threads
 @pytest.mark.parametrize("top_p", [0.9, 1.0])
