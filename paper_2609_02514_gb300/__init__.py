@@ -21,7 +21,7 @@ import threading
 
 import torch
 
-__all__ = ["load", "use_checked", "checked_violation", "lib_path", "workspace_bytes", "verify", "sparsify", "cache_build", "cache_lookup",
+__all__ = ["load", "use_checked", "checked_violation", "checked_cache_selects", "lib_path", "workspace_bytes", "verify", "sparsify", "cache_build", "cache_lookup",
            "ROW_NONFINITE", "ROW_BAD_Q", "COUNTERS_OFFSET", "AcespecError"]
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -85,6 +85,17 @@ def checked_violation():
     return None if out[0] == 0 else (int(out[0]), int(out[1]), int(out[2]))
 
 
+def checked_cache_selects():
+    """Rows of q that the checked build's cache_build read again since the
+    last call (their first read's candidates were not enough); clears the count."""
+    lib = load()
+    if not hasattr(lib, "aces_checked_cache_selects"):
+        raise RuntimeError("the product library counts nothing: call use_checked() first")
+    n = ctypes.c_uint(0)
+    _check("aces_checked_cache_selects", lib.aces_checked_cache_selects(ctypes.byref(n)))
+    return int(n.value)
+
+
 def _open(path):
     if path in _libs:
         return _libs[path]
@@ -116,6 +127,8 @@ def _open(path):
     if hasattr(lib, "aces_checked_violation"):
         lib.aces_checked_violation.argtypes = [P]
         lib.aces_checked_violation.restype = I
+        lib.aces_checked_cache_selects.argtypes = [P]
+        lib.aces_checked_cache_selects.restype = I
     _libs[path] = lib
     return lib
 

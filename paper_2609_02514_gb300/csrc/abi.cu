@@ -423,4 +423,14 @@ extern "C" aces_status aces_checked_violation(unsigned long long out[3]) {
     }
     return ACES_OK;
 }
+
+// The rows of q that aces_cache_build read again since the last call, because
+// their first read's candidates were not enough (for the package's tests: not
+// part of the header).  Waits for the device and clears the count.
+extern "C" aces_status aces_checked_cache_selects(unsigned int *n);
+extern "C" aces_status aces_checked_cache_selects(unsigned int *n) {
+    if (!n) return ACES_ERR_INVALID_ARG;
+    if (cudaDeviceSynchronize() != cudaSuccess || check_take_selects(n) != cudaSuccess) return ACES_ERR_CUDA;
+    return ACES_OK;
+}
 #endif

@@ -43,6 +43,7 @@ static inline cudaError_t check_take(unsigned long long out[3]) {
 cudaError_t check_take_rows_cap(unsigned long long out[3]);
 cudaError_t check_take_rows_general(unsigned long long out[3]);
 cudaError_t check_take_cache(unsigned long long out[3]);
+cudaError_t check_take_selects(unsigned int *n);
 cudaError_t check_take_resample(unsigned long long out[3]);
 cudaError_t check_take_kv(unsigned long long out[3]);
 cudaError_t check_take_mask(unsigned long long out[3]);

@@ -1,9 +1,9 @@
 """Branch cache (Sec. III-C) at large fan-outs, against the float64 oracle.
 
-Fan-outs above 8 take the one-pass path: the union of the per-thread top-8
-lists, sorted in shared memory, holds the F_d largest whenever no thread
-dropped an id above the F_d-th entry.  Otherwise the kernel repeats its pass
-eight maxima at a time.  Both must give the oracle's branches bit for bit.
+A row is read once, listing what reaches a threshold found from a sample of
+it; a row whose list does not prove to hold the F_d largest is selected digit
+by digit in further reads.  Both must give the oracle's branches bit for bit
+(tests/test_gpu_checked.py counts the rows of the second kind).
 """
 import dataclasses
 
@@ -45,9 +45,9 @@ def test_large_fanouts_on_the_benchmark_rows(A, orc, F):
     assert (gbt >= 0).mean() > 0.99  # the draft support holds hundreds of ids
 
 
-def test_one_thread_holding_more_than_eight_falls_back_to_repeated_passes(A, orc):
-    # 40 large q values in the chunks of one thread (ids 4 * (256 m) + e):
-    # its list keeps 8 of them, so the union cannot prove the top 32
+def test_the_largest_values_in_the_chunks_of_one_thread(A, orc):
+    # 40 large q values in the chunks that one thread reads when a row has one
+    # CTA (ids 4 * (256 m) + e): they share one of the sample's maxima
     V, K = 32768, 2
     rng = np.random.default_rng(71)
     q = rng.random((1, K, V)).astype(np.float32) * 1e-6
