@@ -422,6 +422,8 @@ struct Workspace {
                                //       in a second pass, [11] bfloat16 rows that published a short
                                //       nucleus, [12] rows finished by the sketch-led pass,
                                //       [13] sequences left to the general kernel's draw,
+                               //       [14] rows the general kernel finished by depth histogram,
+                               //       [15] rows that histogram read twice and did not finish,
                                //       [16..55] how many rows needed each depth (in bins of T/4
                                //       below the row max)
     int *scan_list;            // [B]              (verify only) sequences left to the general kernel's draw

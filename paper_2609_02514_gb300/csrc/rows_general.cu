@@ -464,11 +464,16 @@ __device__ bool binned_row(const RowArgs &a, int r, const RowChunks<DT> &rc, flo
 // the nucleus crossing (first prefix reaching ceil(top_p * S * 2^40)) and the
 // value holding the k-th payload id; the elements of those values (ties are
 // taken in id order, which is the order-value order) are collected and ranked
-// in shared memory.  Returns false, having written nothing, when a needed
-// value lies below the window or a collected set exceeds VH_CAP; the binned
-// path then takes the row.
+// in shared memory.  Declines, having written nothing, when a needed value lies
+// below the window (VH_BELOW: the depth histogram then takes the row) or when a
+// set to collect exceeds VH_CAP (VH_FULL, where the depth histogram's lists
+// would not hold it either: the binned path does).
+enum { VH_DONE, VH_BELOW, VH_FULL };
 constexpr int VH_W = 4096;    // values below the max with a count
 constexpr int VH_CAP = 1024;  // collected ids per set (payload values, crossing value)
+constexpr int DH_XCAP = 1536; // depth histogram: listed ids around the crossing
+constexpr int DH_PCAP = 768;  // listed ids of the payload's bins
+static_assert(DH_PCAP <= VH_CAP, "a payload set too large for the value histogram is too large for the depth histogram");
 constexpr int VH_U = 4;       // 16-byte loads per thread in flight in the counting pass
 
 struct ValHist {
@@ -511,7 +516,7 @@ __device__ __forceinline__ void warp_append_cap(unsigned long long *arr, int *n,
 // S_in: the row's exp-sum in units of 2^kref for a row handed over by the
 // row kernel, 0 otherwise.  *n_fin_out gets the row's count of finite ids
 // when top_p = 1 or S_in = 0 (its only uses), even when the row is declined.
-__device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &rc, float m, float kref, double S_in,
+__device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &rc, float m, float kref, double S_in,
                             unsigned long long *n_fin_out, ValHist *vh, unsigned long long *buf, double *redd,
                             unsigned long long *redu) {
     using E = Elem<ACES_BF16>;
@@ -593,7 +598,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
     const unsigned long long n_fin = block_reduce(nfin, redu, SumU64());  // (its barriers order the counts)
     *n_fin_out = n_fin;
     const double S = have_S ? S_in : block_reduce((double)hi + (double)lo, redd, SumD());
-    if (!(S > 0.0 && S < 1e300)) return false;
+    if (!(S > 0.0 && S < 1e300)) return VH_BELOW;
     const unsigned long long tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
     // ---- prefix scan over the values, PER consecutive values per thread ----
     constexpr int PER = VH_W / NT;
@@ -631,7 +636,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
         }
     }
     __syncthreads();
-    if (vh->dstar == -2) return false;  // the crossing lies below the window
+    if (vh->dstar == -2) return VH_BELOW;  // the crossing lies below the window
     const unsigned long long n_nuc = all_in ? n_fin : vh->cnt_above + (unsigned long long)vh->j;
     const int L = (int)(n_nuc < (unsigned long long)a.k ? n_nuc : (unsigned long long)a.k);
     if (L > 0) {  // the value holding the L-th id (at most one thread finds it)
@@ -650,9 +655,9 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
     }
     __syncthreads();
     const int dstar = vh->dstar, dk = vh->dk;
-    if (dk == -2) return false;  // the L-th id lies below the window
-    if (dk >= 0 && vh->npay_need > (unsigned long long)VH_CAP) return false;
-    if (dstar >= 0 && vh->cnt[dstar] > (uint32_t)VH_CAP) return false;
+    if (dk == -2) return VH_BELOW;  // the L-th id lies below the window
+    if (dk >= 0 && vh->npay_need > (unsigned long long)VH_CAP) return VH_FULL;
+    if (dstar >= 0 && vh->cnt[dstar] > (uint32_t)VH_CAP) return vh->cnt[dstar] > (uint32_t)DH_XCAP ? VH_FULL : VH_BELOW;
     // ---- collect every id of the values up to dk, and those of dstar ----
     // A packed bfloat16 compare per pair of ids (value >= that of dk, or
     // == that of dstar: IEEE order, where -0 == +0 as in the keys) lets a
@@ -723,7 +728,7 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
     }
     if (tid == 0) atomicAdd(&a.ws.fb_count[6], 1);
     finish_row<ACES_BF16>(a, r, row, kref, S_nuc, cut, all_in ? RS_ALL_IN : 0, buf, LL, redd);
-    return true;
+    return VH_DONE;
 }
 
 // ---------------------------------------------------------------------------
@@ -737,8 +742,8 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
 // with bins of T / 200).  A second read sums the exact 2^-40 masses of the ids
 // above that range and lists those inside it and the payload's; the ordered
 // list gives the crossing id.  Returns false, having written nothing, when a
-// list is too long or the payload ends below the bins; the binned path then
-// takes the row (it sums a 64-bit mass per id with shared-memory atomics).  256
+// list would be too long (known after the first read) or the payload ends below
+// the bins; the binned path then takes the row (it sums a 64-bit mass per id with shared-memory atomics).  256
 // rows of 128256 float32 logits, about 200 of them handed over: 297 us a call
 // with the binned path, 158 with this one, 147 with the second read's work
 // done per hit and fewer rows handed over, 153 with the row's exact mass summed
@@ -749,8 +754,6 @@ __device__ bool valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> 
 // What is left is two more reads of those rows by one CTA each.
 constexpr int DH_W = 4096;    // bins
 constexpr int DH_PAD = 32;    // counters of the ids below them, one per lane
-constexpr int DH_XCAP = 1536; // listed ids around the crossing
-constexpr int DH_PCAP = 768;  // listed ids of the payload's bins
 constexpr int DH_U = 4;       // 16-byte loads in flight per thread
 
 struct DepthHist {
@@ -826,6 +829,7 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
     const unsigned long long tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * (double)all_fx);
     __syncthreads();
     // ---- the bins around the crossing and the payload's last ----
+    int b_hi, b_lo, b_k;
     {
         constexpr int PER = DH_W / NT;
         uint32_t cn[PER], lc = 0u;
@@ -881,11 +885,25 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
             if (cc >= ku) atomicMin(&h->b_k, bn);
         }
         __syncthreads();
+        b_hi = h->b_hi;
+        b_lo = h->b_lo;
+        if (b_lo == INT_MAX || (all_in && h->b_k == INT_MAX)) return false;
+        b_k = a.k == 0 ? -1 : (all_in ? h->b_k : min(h->b_k, b_lo));
+        // the lists' lengths (the crossing's in the upper half): a row whose lists
+        // do not fit (values alike: logits that were bfloat16 once) is declined
+        // before the second read.  (256 rows of 128256 equal float32 logits: 2134
+        // us a call with that read, 1942 without.)
+        unsigned long long len = 0ull;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int bn = tid * PER + i;
+            if (!all_in && bn >= b_hi && bn <= b_lo) len += (unsigned long long)cn[i] << 32;
+            if (bn <= b_k) len += cn[i];
+        }
+        // (its barriers: every bin is read, the lists may take the counters' place)
+        len = block_reduce(len, redu, SumU64());
+        if ((len >> 32) > (unsigned long long)DH_XCAP || (uint32_t)len > (uint32_t)DH_PCAP) return false;
     }
-    const int b_hi = h->b_hi, b_lo = h->b_lo;
-    if (b_lo == INT_MAX || (all_in && h->b_k == INT_MAX)) return false;
-    const int b_k = a.k == 0 ? -1 : (all_in ? h->b_k : min(h->b_k, b_lo));
-    __syncthreads();  // (every bin is read: the lists may take the counters' place)
     // ---- exact masses above the range, the ids inside it and the payload's ----
     // (ids are looked at one by one only from a value just below the lowest
     // needed bin: their number per lane, not the row's length, is what costs)
@@ -930,7 +948,10 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
     const unsigned long long n_above = block_reduce((unsigned long long)na, redu, SumU64());
     __syncthreads();
     const int nx = h->nx, np = h->np;
-    if (nx > DH_XCAP || np > DH_PCAP || (!all_in && above >= tg)) return false;
+    if (!all_in && above >= tg) {  // (a bin's bound of a logit far from zero was too tight)
+        if (tid == 0) atomicAdd(&a.ws.fb_count[15], 1);
+        return false;
+    }
     // the payload's ids by rank
     const int lp = np < a.k ? np : a.k;
     rank_order_values<NT>(h->ps, np, reinterpret_cast<uint32_t *>(h->fx), [&](int rank, unsigned long long key) {
@@ -962,13 +983,17 @@ __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, floa
         }
         __syncthreads();
         const int ix = h->ix;
-        if (ix < 0) return false;
+        if (ix < 0) {
+            if (tid == 0) atomicAdd(&a.ws.fb_count[15], 1);
+            return false;
+        }
         S_nuc = (double)h->cum * FX_INV;
         cut = ACES_IN(ix, DH_XCAP) ? h->xs[ix] : 0ull;
         const unsigned long long n_nuc = n_above + (unsigned long long)ix + 1ull;
         if (n_nuc < (unsigned long long)L) L = (int)n_nuc;
     }
     __syncthreads();
+    if (tid == 0) atomicAdd(&a.ws.fb_count[14], 1);
     finish_row<DT>(a, r, rc.row(), kref, S_nuc, cut, all_in ? RS_ALL_IN : 0, buf, L, redd);
     return true;
 }
@@ -1054,13 +1079,14 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
         }
         if constexpr (DT == ACES_BF16) {
             unsigned long long nf = 0ull;
-            bool done = valhist_row(a, r, rc, m, kref, S_in, &nf, &paths.vh, buf, redd, redu);
+            const int vh = valhist_row(a, r, rc, m, kref, S_in, &nf, &paths.vh, buf, redd, redu);
             __syncthreads();
-            if (!done && handed) {
-                done = depth_row<DT>(a, r, rc, m, kref, S_in, &paths.dh, buf, redd, redu);
+            if (vh == VH_DONE) return;
+            if (vh == VH_BELOW && handed) {
+                const bool done = depth_row<DT>(a, r, rc, m, kref, S_in, &paths.dh, buf, redd, redu);
                 __syncthreads();
+                if (done) return;
             }
-            if (done) return;
             n_fin = nf;
         }
         if (binned_row<DT>(a, r, rc, m, kref, n_fin, &paths.bs, buf, redd, redu)) return;

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-FALLBACK, LAZY, SCANNED = 0, 5, 13   # words of the workspace's path counters
+FALLBACK, RADIX, LAZY, SCANNED, DEPTH, DEPTH_LOST = 0, 4, 5, 13, 14, 15   # words of the workspace's path counters
 
 
 @pytest.fixture(scope="module")
@@ -146,7 +146,28 @@ def test_float32_rows_by_depth_histogram(A, orc, V, offset, shift, top_p):
     res, counters, o = _verify(A, orc, w, inp, offset)
     if top_p < 1.0:
         assert counters[FALLBACK] == 12 and (o["n_nuc"] > 4096).any(), counters
-    assert res["checked_seqs"] >= 2, res
+    assert counters[DEPTH] == counters[FALLBACK] and res["checked_seqs"] >= 2, (res, counters)
+
+
+def test_bfloat16_rows_by_depth_histogram(A, orc):
+    # normal logits at T = 1: the crossing lies among negative ones, out of the
+    # value histogram's reach, and no value is shared by many ids
+    w = gen.make_workload(3, 2, 20000, "bf16", T=1.0, top_p=0.9, k=40, seed=92, sigma=1.0)
+    res, counters, _ = _verify(A, orc, w, gen.generate(w))
+    assert counters[FALLBACK] == 9 and counters[DEPTH] == 9 and res["checked_seqs"] >= 1, (res, counters)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_rows_of_alike_values_are_declined_before_the_second_read(A, orc, dtype):
+    # 8 values: thousands of ids of each, more than either list holds; the binned
+    # path (2048 ids a bin) does not hold them either
+    w = gen.make_workload(4, 2, 40000, dtype, T=1.0, top_p=0.8, k=40, seed=93)
+    inp = gen.generate(w)
+    z = np.random.default_rng(93).integers(0, 8, inp["z"].shape).astype(np.float32) * 0.25 + 1.0
+    inp["z"] = _logits(z, dtype)
+    res, counters, _ = _verify(A, orc, w, inp)
+    assert counters[FALLBACK] == 12 and counters[RADIX] == 12, counters
+    assert counters[DEPTH] == 0 and counters[DEPTH_LOST] == 0 and res["checked_seqs"] >= 1, (res, counters)
 
 
 @pytest.mark.parametrize("B", [20, 100, 250])          # CTAs of 1024, 512 and 256 threads
