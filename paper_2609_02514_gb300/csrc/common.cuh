@@ -59,16 +59,15 @@ constexpr int BIN_PER_T = 8;
 // Row-level flags kept in the workspace.
 constexpr int RS_ALL_IN = 1;        // top_p >= 1: every finite id is in the nucleus
 constexpr int RS_NONFINITE = 2;
-// handed to the general kernel: kref holds the row max, c the log2 reference
-// of the row's exp-sum and S_nuc that exp-sum
-constexpr int RS_HANDOFF = 4;
 // the nucleus ends among the ids of one bfloat16 value whose ids were not
 // kept: cut holds that value's 32-bit order key in its high word and j, the
 // number of its ids (in id order) inside the nucleus, in its low word; the
 // draw finds those ids when it reads the row
 constexpr int RS_LAZY = 8;
 
-// Per-row state written by the row kernels and read by the sequence's draw.
+// Per-row state written by the row kernels and read by the sequence's draw.  Of a
+// row handed to the general kernel, until that finishes it: kref holds the row
+// max, c the log2 reference of the row's exp-sum and S_nuc that exp-sum.
 struct RowStat {
     float kref;              // log2 reference: masses are 2^(z*c - kref)
     float c;                 // log2(e) / T
@@ -107,8 +106,8 @@ __device__ __forceinline__ float order_value(unsigned long long o) {
 // stream has exited or executed pdl_trigger(), without waiting for that
 // kernel's completion and memory flush.  Every CTA of such a kernel executes
 // pdl_wait() before it reads anything the previous kernel wrote (and before
-// it exits, so that its completion implies the previous kernel's).  The fast
-// row kernel never triggers early: general-kernel CTAs placed on the first
+// it exits, so that its completion implies the previous kernel's).  The row
+// kernel never triggers early: general-kernel CTAs placed on the first
 // SMs its last wave frees would crowd there and unbalance that persistent
 // grid.  Without the launch attribute both calls are no-ops.
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
@@ -191,19 +190,8 @@ __device__ __forceinline__ float warp_max(float v) {
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
-__device__ __forceinline__ double warp_sum(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w > v ? w : v;
-    }
     return v;
 }
 
@@ -223,23 +211,9 @@ template <class T, class Op>
 __device__ __forceinline__ T block_reduce(T v, T *red, Op op) {
     return block_reduce_n<NT>(v, red, op);
 }
-struct SumD {
-    __device__ double operator()(double v) const { return warp_sum(v); }
-    __device__ double combine(double a, double b) const { return a + b; }
-};
-struct MaxF {
-    __device__ float operator()(float v) const { return warp_max(v); }
-    __device__ float combine(float a, float b) const { return fmaxf(a, b); }
-};
 struct SumU64 {
     __device__ unsigned long long operator()(unsigned long long v) const { return warp_sum(v); }
     __device__ unsigned long long combine(unsigned long long a, unsigned long long b) const { return a + b; }
-};
-struct MaxU64 {
-    __device__ unsigned long long operator()(unsigned long long v) const { return warp_max(v); }
-    __device__ unsigned long long combine(unsigned long long a, unsigned long long b) const {
-        return a > b ? a : b;
-    }
 };
 
 // Exclusive scan over the block of one u64 per thread; `red` holds NTH/32
@@ -259,24 +233,6 @@ __device__ __forceinline__ unsigned long long block_exscan_n(unsigned long long 
     __syncthreads();
     unsigned long long base = 0, all = 0;
     for (int i = 0; i < NTH / 32; ++i) {
-        if (i < wid) base += red[i];
-        all += red[i];
-    }
-    *total = all;
-    return base + inc - v;
-}
-__device__ __forceinline__ double block_exscan(double v, double *red, double *total) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double inc = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        double t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    __syncthreads();
-    if (lane == 31) red[wid] = inc;
-    __syncthreads();
-    double base = 0, all = 0;
-    for (int i = 0; i < NWARP; ++i) {
         if (i < wid) base += red[i];
         all += red[i];
     }

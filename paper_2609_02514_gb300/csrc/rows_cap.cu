@@ -304,7 +304,7 @@ __device__ __forceinline__ void fallback_row(const RowArgs &a, int r, float m, f
     s.c = kref;
     s.S_nuc = S;
     s.cut = 0ull;
-    s.flags = RS_HANDOFF;
+    s.flags = 0;
     s.nnuc = -1;
     a.ws.stats[r] = s;
     const int pos = atomicAdd(a.ws.fb_count, 1);

@@ -457,9 +457,8 @@ __device__ bool binned_row(const RowArgs &a, int r, const RowChunks<DT> &rc, flo
 // 65536 values, and equal values have equal masses, so counting the elements
 // of each value is enough: the values of a window below the row max (at most
 // VH_W of them) get a count, one shared-memory atomic per element and no
-// per-element mass.  The exp-sum S of the whole row comes with a row handed
-// over by the row kernel; otherwise the counting pass sums it in compensated
-// fp32, as the row kernel does.  A prefix scan over the values then gives,
+// per-element mass.  The exp-sum S of the whole row comes with the row, from
+// the row kernel.  A prefix scan over the values then gives,
 // exactly in 2^-40 fixed point (count x the value's mass), the value holding
 // the nucleus crossing (first prefix reaching ceil(top_p * S * 2^40)) and the
 // value holding the k-th payload id; the elements of those values (ties are
@@ -513,16 +512,14 @@ __device__ __forceinline__ void warp_append_cap(unsigned long long *arr, int *n,
 }
 
 // (bfloat16 rows; all threads of the CTA)
-// S_in: the row's exp-sum in units of 2^kref for a row handed over by the
-// row kernel, 0 otherwise.  *n_fin_out gets the row's count of finite ids
-// when top_p = 1 or S_in = 0 (its only uses), even when the row is declined.
-__device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &rc, float m, float kref, double S_in,
+// S: the row's exp-sum in units of 2^kref.  *n_fin_out gets the row's count of
+// finite ids when top_p = 1 (its only use), even when the row is declined.
+__device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &rc, float m, float kref, double S,
                             unsigned long long *n_fin_out, ValHist *vh, unsigned long long *buf, double *redd,
                             unsigned long long *redu) {
     using E = Elem<ACES_BF16>;
     const int tid = threadIdx.x, lane = tid & 31;
     const bool all_in = a.top_p >= 1.0f;
-    const bool have_S = S_in > 0.0;
     const char *row = rc.row();
     const uint32_t km = bkey16(__float_as_uint(m) >> 16);  // m is a bfloat16 value
     for (int i = tid; i < VH_W; i += NT) vh->cnt[i] = 0u;
@@ -534,13 +531,13 @@ __device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &
     }
     // the window: values km - d for d <= D (never -inf, whose key is 0x80)
     uint32_t D = km - 0x81u < (uint32_t)(VH_W - 1) ? km - 0x81u : (uint32_t)(VH_W - 1);
-    if (have_S && !all_in) {
+    if (!all_in) {
         // Every id below a value of mass e_lo = (1 - top_p) S / (16 V) has
         // less mass than that, so all of them together hold less than a
         // sixteenth of the mass outside the nucleus and the crossing lies at
         // or above that value; an id whose fixed-point mass is 0 (below
         // 2^-40) is never needed either.  D is the last value reaching it.
-        const float g = fmaxf(log2f((1.0f - a.top_p) * (float)S_in / (16.0f * (float)a.V)), -41.0f);
+        const float g = fmaxf(log2f((1.0f - a.top_p) * (float)S / (16.0f * (float)a.V)), -41.0f);
         const float vt = (kref + g) / a.c;
         uint32_t lo = 0u, hi = D;  // bval16(km) = m >= vt
         while (lo < hi) {
@@ -551,14 +548,12 @@ __device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &
         D = lo;
     }
     __syncthreads();
-    // ---- pass 1: counts per value (with the finite count and the
-    // compensated exp-sum where they are needed) ----
-    float hi = 0.f, lo = 0.f;
+    // ---- pass 1: counts per value (top_p = 1: and of the finite ids) ----
     unsigned long long nfin = 0ull;
     const int nch = rc.nch;
     // (-inf words outside the row count nowhere)
-    auto count_pass = [&](auto with_sum, auto with_nfin) {
-        constexpr bool WS = decltype(with_sum)::value, WN = decltype(with_nfin)::value;
+    auto count_pass = [&](auto with_nfin) {
+        constexpr bool WN = decltype(with_nfin)::value;
         for (int c0 = tid; c0 < nch; c0 += VH_U * NT) {
             uint4 wu[VH_U];
 #pragma unroll
@@ -566,7 +561,6 @@ __device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &
                 const int cc = c0 + u * NT;
                 wu[u] = cc < nch ? rc.load(cc) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
             }
-            float cs = 0.f;
             uint32_t nf = 0u;
 #pragma unroll
             for (int u = 0; u < VH_U; ++u) {
@@ -576,7 +570,6 @@ __device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const uint32_t b = h ? (wd[q] >> 16) : (wd[q] & 0xFFFFu);
-                        if (WS) cs += ex2(fmaf(__uint_as_float(b << 16), a.c, -kref));  // 0 for -inf
                         if (WN) nf += b != 0xFF80u;
                         const uint32_t d = km - bkey16(b);
                         if (d <= D && ACES_IN(d, VH_W)) atomicAdd(&vh->cnt[d], 1u);
@@ -584,21 +577,12 @@ __device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &
                 }
             }
             if (WN) nfin += nf;
-            if (WS) {
-                const float t = hi + cs;  // Neumaier
-                if (fabsf(hi) >= fabsf(cs)) lo += (hi - t) + cs;
-                else lo += (cs - t) + hi;
-                hi = t;
-            }
         }
     };
-    if (!have_S) count_pass(std::true_type(), std::true_type());
-    else if (all_in) count_pass(std::false_type(), std::true_type());
-    else count_pass(std::false_type(), std::false_type());
+    if (all_in) count_pass(std::true_type());
+    else count_pass(std::false_type());
     const unsigned long long n_fin = block_reduce(nfin, redu, SumU64());  // (its barriers order the counts)
     *n_fin_out = n_fin;
-    const double S = have_S ? S_in : block_reduce((double)hi + (double)lo, redd, SumD());
-    if (!(S > 0.0 && S < 1e300)) return VH_BELOW;
     const unsigned long long tg = all_in ? 0ull : (unsigned long long)ceil((double)a.top_p * S * (double)FX_SCALE);
     // ---- prefix scan over the values, PER consecutive values per thread ----
     constexpr int PER = VH_W / NT;
@@ -732,7 +716,7 @@ __device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &
 }
 
 // ---------------------------------------------------------------------------
-// Depth-histogram path for handed rows (their max m and exp-sum S_in are known):
+// Depth-histogram path (the row's max m and exp-sum S_in are known):
 // the float32 counterpart of the value histogram, and the second try for
 // bfloat16.  One read counts the ids in DH_W equal bins of depth below the
 // max, down to a value the crossing cannot lie below (top_p = 1: to where an
@@ -1012,9 +996,7 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
     unsigned char *scratch = reinterpret_cast<unsigned char *>(&paths);  // (of a finished row)
     __shared__ unsigned long long buf[ACES_MAX_TOPK];
     __shared__ double redd[NWARP];
-    __shared__ float redf[NWARP];
     __shared__ unsigned long long redu[NWARP];
-    __shared__ int s_bad;
     __shared__ int s_nbuf;
     __shared__ DrawPart part;
     __shared__ int pend[DRAW_CL];
@@ -1040,54 +1022,30 @@ __global__ void __launch_bounds__(NT, 2) k_rows_general(const __grid_constant__ 
     // one handed row (all threads)
     auto do_row = [&](int r) {
         const RowChunks<DT> rc(reinterpret_cast<const char *>(a.logits) + (size_t)r * a.V * E::SIZE, a.V);
-        // it comes with its max and its exp-sum (and is finite); the max pass
-        // runs only where the paths need the finite count it takes (top_p = 1
-        // on float32 rows)
+        // it comes with its max and its exp-sum, and is finite
         const RowStat hs = a.ws.stats[r];
-        const bool handed = hs.flags == RS_HANDOFF;
-        float m = hs.kref;
-        unsigned long long n_fin = 0ull;
-        float kref = ceilf(m * a.c);  // masses are 2^(z*c - kref) <= 1
-        // the handed exp-sum in units of 2^kref (its reference is the same
-        // ceil(m c); the power-of-two rescale is exact)
-        const double S_in = handed ? ldexp(hs.S_nuc, (int)(hs.c - kref)) : 0.0;
-        if (DT == ACES_F32 && handed) {
+        const float m = hs.kref;
+        const float kref = ceilf(m * a.c);  // masses are 2^(z*c - kref) <= 1
+        // the exp-sum in units of 2^kref (its reference is the same ceil(m c); the
+        // power-of-two rescale is exact)
+        const double S_in = ldexp(hs.S_nuc, (int)(hs.c - kref));
+        unsigned long long n_fin = 0ull;  // finite ids (top_p = 1)
+        bool depth = true;
+        if constexpr (DT == ACES_BF16) {
+            const int vh = valhist_row(a, r, rc, m, kref, S_in, &n_fin, &paths.vh, buf, redd, redu);
+            __syncthreads();
+            if (vh == VH_DONE) return;
+            depth = vh == VH_BELOW;
+        }
+        if (depth) {
             const bool done = depth_row<DT>(a, r, rc, m, kref, S_in, &paths.dh, buf, redd, redu);
             __syncthreads();
             if (done) return;
         }
-        if (!(handed && (DT == ACES_BF16 || a.top_p < 1.0f))) {
-            // pass 0: max, finite count, invalid values
-            if (tid == 0) s_bad = 0;
-            __syncthreads();
-            float mx = -INFINITY;
-            unsigned long long nfin = 0;
-            int bad = 0;
-            for_each_elem<DT>(rc, [&](int, float v) {
-                if (v != v || v == INFINITY) bad = 1;
-                if (v > -INFINITY) ++nfin;
-                mx = fmaxf(mx, v);
-            });
-            if (bad) s_bad = 1;
-            m = block_reduce(mx, redf, MaxF());
+        if (DT == ACES_F32 && a.top_p >= 1.0f) {
+            unsigned long long nfin = 0ull;
+            for_each_elem<DT>(rc, [&](int, float v) { nfin += v > -INFINITY; });
             n_fin = block_reduce(nfin, redu, SumU64());
-            kref = ceilf(m * a.c);
-            if (s_bad || n_fin == 0ull || !(kref < 1e30f)) {
-                nonfinite_row<NT>(a, r);
-                return;
-            }
-        }
-        if constexpr (DT == ACES_BF16) {
-            unsigned long long nf = 0ull;
-            const int vh = valhist_row(a, r, rc, m, kref, S_in, &nf, &paths.vh, buf, redd, redu);
-            __syncthreads();
-            if (vh == VH_DONE) return;
-            if (vh == VH_BELOW && handed) {
-                const bool done = depth_row<DT>(a, r, rc, m, kref, S_in, &paths.dh, buf, redd, redu);
-                __syncthreads();
-                if (done) return;
-            }
-            n_fin = nf;
         }
         if (binned_row<DT>(a, r, rc, m, kref, n_fin, &paths.bs, buf, redd, redu)) return;
         if (tid == 0) atomicAdd(&a.ws.fb_count[4], 1);
