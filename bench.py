@@ -158,7 +158,7 @@ def measured_peak():
 # device code behind each profiled kernel (its file and the shared device header)
 KERNEL_SOURCES = {
     "aces_verify": ("common.cuh", "draw.cuh", "rows_cap.cu", "rows_general.cu"),
-    "k_cache_build": ("common.cuh", "cache.cu"),
+    "k_cache_build": ("common.cuh", "qrow.cuh", "cache.cu"),
 }
 
 

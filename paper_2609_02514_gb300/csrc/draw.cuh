@@ -37,6 +37,7 @@ constexpr int DRAW_CL = 8;  // CTAs of a draw's cluster, at most
 constexpr int DRAW_CH = 4;  // 16-byte chunks per lane and step of a task
 constexpr int DRAW_SCRATCH = 4 * NUC_CAP * 8;  // bytes of shared memory the draws use, on a 16-byte boundary
 static_assert(DRAW_TASKS * (3 * 8 + 4) <= DRAW_SCRATCH, "the tasks' sums fit");
+static_assert(2 * NUC_CAP * 8 % 16 == 0, "the list's 32-bit keys are read 16 bytes at a time");
 
 // A row of V logits in 16-byte chunks.  A row that does not start on a
 // 16-byte boundary begins `head` elements into chunk 0: element e of chunk c

@@ -127,6 +127,9 @@ struct F32Caps {
 constexpr int RANK_MAX = 512;       // ids ordered by direct ranking (more: bitonic sort)
 static_assert(WS_DEPTH + NSB <= WS_COUNTERS / 4, "the depth histogram fits the counters area");
 static_assert(DRAW_SCRATCH <= SMEM_BF && DRAW_SCRATCH <= SMEM_F32, "the draw's scratch fits");
+// (32-bit keys are read 16 bytes at a time: at hist, and after two lists of RANK_MAX)
+static_assert(HPAD * 4 % 16 == 0 && CREC * 20 % 16 == 0 && F32Caps<2>::CR * 20 % 16 == 0 && 2 * RANK_MAX * 8 % 16 == 0,
+              "the keys of the ranking lie on 16 bytes");
 static_assert(ACES_MAX_V <= 1 << 20 && HW <= 1 << 10 && RANK_MAX <= HW, "a value and an id in 30 bits");
 static_assert(GCAP * 4 <= HW * 4 && PCAP * 8 <= SKG * 2 && "the aliased areas fit");
 static_assert(PCAP <= SK_TMP && SK_TMP + GCAP / 2 <= SKG / 4 && SK_TMP + PCAP <= SKG / 4, "the sketch-led areas fit");

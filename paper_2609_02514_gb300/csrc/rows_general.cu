@@ -18,6 +18,7 @@
 //                selection over the 64-bit order value
 //                O = key(z) << 32 | (2^32 - 1 - id), 8 bits per pass.
 #include <climits>
+#include <cstddef>
 #include <type_traits>
 
 #include <cuda_bf16.h>
@@ -757,6 +758,7 @@ struct DepthHist {
     int ix;
     unsigned long long cum;
 };
+static_assert(offsetof(DepthHist, fx) % 16 == 0, "the payload's 32-bit keys are read 16 bytes at a time");
 
 template <int DT>
 __device__ bool depth_row(const RowArgs &a, int r, const RowChunks<DT> &rc, float m, float kref, double S_in, DepthHist *h,

@@ -72,3 +72,13 @@ def test_traffic_figures_follow_the_kernel_code_not_its_comments():
     assert bench._code_only(src) != bench._code_only(src.replace("x * x", "x + x"))
     for k in bench.KERNEL_SOURCES:
         assert len(bench.kernel_source_hash(k)) == 16
+
+
+def test_a_kernels_hash_covers_every_device_header_it_includes():
+    import re
+    import bench
+    csrc = os.path.join(bench.ROOT, "paper_2609_02514_gb300", "csrc")
+    for kernel, files in bench.KERNEL_SOURCES.items():
+        for f in files:
+            for h in re.findall(r'#include "([^"/]+\.cuh)"', open(os.path.join(csrc, f)).read()):
+                assert h in files, (kernel, f, h)
