@@ -42,7 +42,7 @@ KERNELS_PER_STEP = 4
 VERIFY_KERNELS = ["k_rows_cap", "k_rows_general"]
 # path counters at the start of the workspace (int32 words)
 PATHS = ["rows_on_general_kernel", "timeouts", "rows_value_histogram", "rows_bitonic_order",
-         "general_rows_radix", "rows_cut_left_to_resolve", "general_rows_value_histogram",
+         "general_rows_radix", "rows_cut_left_to_draw", "general_rows_value_histogram",
          "accept_tests_ranked_among_ties", "rows_published_depth", "rows_depth_from_finished_rows",
          "rows_counted_twice", "short_rows_published", "rows_sketch_led"]
 

@@ -385,9 +385,10 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     // one of the row's exact mass, whichever kernel finishes the row: the
     // float32 sum places the target within a bound (sum_err), and where the cut
     // is not the same over that whole range the row is read again for its exact
-    // mass.  (Of 128000 float32 rows 2 to 12 were cut one id away from float64 by
-    // the float32 sum alone.)  Off the grid the mass of top_p = 1 rows is the
-    // exact one too.
+    // mass.  (Rows cut one id away from float64, of 128000 each, by the float32
+    // sum and by the exact one: float32 rows of 50000 logits 11 and 6, of 50003 7
+    // and 9, of 20001 5 and 0; bfloat16 rows of 50003 9 and 6, of 20001 1 and 0.)
+    // Off the grid the mass of top_p = 1 rows is the exact one too.
     constexpr bool EXACT_CUT = !BF || RAGGED;
     extern __shared__ __align__(16) unsigned char smem[];
     // bfloat16: [HPAD dummies, value counts: HW u32 | sketch: SKG u16 | ids >=

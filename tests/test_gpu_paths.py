@@ -4,7 +4,7 @@ The workspace's first ten int32 words count, per call: rows handed to the
 exact general kernel, bounded-wait timeouts (reserved), bfloat16 rows the
 single-pass kernel finished from its value counts, rows whose candidates were
 ordered by bitonic sort (more than 512), rows the general kernel finished by
-radix selection, rows whose nucleus cut was left to the resolve step, rows
+radix selection, rows whose nucleus cut was left to the draw, rows
 the general kernel finished by its bfloat16 value histogram, accept tests
 that ranked the draft token among the ids of the crossing value, rows that
 published their depth, rows that took their depth from finished rows, and
@@ -96,7 +96,7 @@ def test_value_counts_on_the_benchmark_rows(A, orc):
 def test_large_nuclei_leave_the_cut_to_the_resolve_step(A, orc):
     # rows of the 128256-id recipe (nuclei of thousands of ids, k = 32): the
     # crossing value's ids are not among the payload's, so the cut is left to
-    # the resolve step, which finds it for the drawn rows
+    # the draw, which finds it for the drawn rows
     w = gen.make_workload(3, 4, 128256, "bf16", sigma=3.0, rho=0.5, T=1.0, top_p=0.9, k=32, seed=41)
     z = gen.generate(w)["z"]
     counters, res = _run(A, orc, w, z)
@@ -236,7 +236,7 @@ def test_crossing_below_the_counted_values_is_counted_again(A, orc):
     # one id at 16 and 60000 ids at 5 (T = 1) carry about equal mass, so the
     # top_p = 0.9 crossing lies 11 T below the max, beyond D = 10 T: a second
     # pass counts the row from its max down and finds it (k = 1: the payload
-    # is the top id, the crossing value's ids are left to the resolve step)
+    # is the top id, the crossing value's ids are left to the draw)
     V = 65536
     w = gen.make_workload(2, 1, V, "bf16", T=1.0, top_p=0.9, k=1, seed=53)
     rng = np.random.default_rng(53)
