@@ -465,7 +465,7 @@ struct RowArgs {
     int it_partial, it_partial2;  // iterations that read the row's partial last tiles (-1: none)
     float samp_frac;
     float inv_ws;          // sample bins per unit of logit: SPB / T
-    float sum_err;         // bound of the float32 exp-sum's relative distance from the exact one
+    float add_err, sum_err;  // bounds of the float32 exp-sum's relative distance from the exact one
     int nmin;              // float32 first rows: ids the capture must reach
     int sk_gpi, sk_ish;    // bfloat16 sketch: groups per thread and iteration (2: 4 chunks each; 1: 8
                            // chunks of 2^sk_ish iterations)

@@ -341,7 +341,7 @@ __device__ __forceinline__ unsigned long long id_fx(float v, float c, float kref
 // 2^-40 units, exactly (a second read of the row; all NTC threads).
 template <int DT, int NTC, bool RAGGED>
 __device__ __noinline__ unsigned long long exact_mass(const char *row, int V, float c, float kref, unsigned long long *red) {
-    constexpr int EPC = Elem<DT>::EPC, U = 4;  // loads in flight
+    constexpr int EPC = Elem<DT>::EPC, U = 32 / EPC;  // loads in flight (32 ids: more code is slower the first time)
     const RowChunks<DT, RAGGED> rc(row, V);
     const uint32_t ni = Elem<DT>::NEG_INF_WORD;
     unsigned long long sum = 0ull;
@@ -367,6 +367,15 @@ __device__ __noinline__ unsigned long long exact_mass(const char *row, int V, fl
     return block_reduce_n<NTC>(sum, red, SumU64());
 }
 
+// sum_err (see rows_cap_layout) of a row whose nucleus, P of its mass S, has n
+// ids: they bound the masses' entropy and with it the mean depth (about 7
+// instead of 18 bits for 900 of 128256 ids, P = 0.95, S = 15)
+__device__ __noinline__ float sharp_err(float sum_err, float P, int n, int V, float S) {
+    const float h = -P * log2f(P) - (1.0f - P) * log2f(1.0f - P), lv = log2f((float)V);
+    const float depth = h + P * log2f((float)n) + (1.0f - P) * lv - log2f(S) + 0.01f;
+    return sum_err - 2.0f * 0.6931472f * ldexpf(fmaxf(lv + 1.0f - fmaxf(depth, 0.0f), 0.0f), -24);
+}
+
 // NTC: threads per CTA, 1024 / NTC CTAs per SM
 // (RAGGED: rows off the 16-byte grid; a build of its own, as the edges cost
 // the other one registers: 128 x 17 rows of 128256 205 -> 213 us)
@@ -383,9 +392,9 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     constexpr bool BF = DT == ACES_BF16;
     // The cut of float32 rows, and of bfloat16 rows off the 16-byte grid, is the
     // one of the row's exact mass, whichever kernel finishes the row: the
-    // float32 sum places the target within a bound (sum_err), and where the cut
-    // is not the same over that whole range the row is read again for its exact
-    // mass.  (Rows cut one id away from float64, of 128000 each, by the float32
+    // float32 sum places the target within a bound, and where the cut is not the
+    // same over that whole range (sharpen) the row is read again for its exact
+    // mass, which takes one SM about 5 us for 128256 logits.  (Rows cut one id away from float64, of 128000 each, by the float32
     // sum and by the exact one: float32 rows of 50000 logits 11 and 6, of 50003 7
     // and 9, of 20001 5 and 0; bfloat16 rows of 50003 9 and 6, of 20001 1 and 0.)
     // Off the grid the mass of top_p = 1 rows is the exact one too.
@@ -608,6 +617,15 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     float v_need = 0.0f;  // the crossing (top_p = 1: the payload's end), for the hints
     bool short_row = false;  // (bfloat16) few ids reach the crossing: published for later rows' pass
 
+    // the nucleus target's range from S, known up to the relative error err (thread 0)
+    auto set_target = [&](float err) {
+        const double t = (double)a.top_p * S * (double)FX_SCALE;
+        s_tg = all_in ? 0ull : (unsigned long long)ceil(t - t * (double)err);
+        s_th = all_in ? 0ull : (unsigned long long)ceil(t + t * (double)err);
+    };
+    // every mass was summed against the final reference kref: the one of the
+    // sample's max, with which all threads start
+    auto one_ref = [&]() { return have && kref == ceilf(m1 * a.c); };
     // reduces the row max, the reference and the exp-sum S (fp32 two-sum tree,
     // fp64 in thread 0 only, which also leaves the nucleus target in s_tg and
     // s_th: valid after the next barrier); true when the row is not a
@@ -682,9 +700,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         if (tid == 0) {
             S = (double)sh + (double)sl;
-            const double t = (double)a.top_p * S * (double)FX_SCALE, err = EXACT_CUT ? t * (double)a.sum_err : 0.0;
-            s_tg = all_in ? 0ull : (unsigned long long)ceil(t - err);
-            s_th = all_in ? 0ull : (unsigned long long)ceil(t + err);
+            set_target(EXACT_CUT ? (one_ref() ? a.add_err : a.sum_err) : 0.0f);
         }
         if (!(sh > 0.0f && sh < INFINITY) || !(m < INFINITY) || !(kref < 1e30f)) {
             nonfinite_row<NTC>(a, r);
@@ -695,7 +711,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     };
     // replaces S (thread 0) and the target by those of the row's exact mass
     // (all threads)
-    bool exact_S = false;
+    bool exact_S = false, sharp = false;
     auto make_exact = [&]() {
         const unsigned long long fx = exact_mass<DT, NTC, RAGGED>(rc.row(), a.V, a.c, kref, s_redu);
         if (tid == 0) {
@@ -704,6 +720,18 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         }
         __syncthreads();
         exact_S = true;
+    };
+    // the cut lies inside the target's range: the range that a nucleus of n ids
+    // leaves, then the exact target (all threads)
+    auto sharpen = [&](int n) {
+        __syncthreads();  // (the range has been read)
+        if (sharp || one_ref()) {
+            make_exact();
+            return;
+        }
+        sharp = true;
+        if (tid == 0) set_target(sharp_err(a.sum_err, a.top_p, n, a.V, (float)S));
+        __syncthreads();
     };
     // hands the row to the general kernel (all threads), whose value histogram
     // takes S from here
@@ -726,6 +754,7 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
         // SK_TMP * 4 slots)
         const int sk_slots = a.sk_gpi == 2 ? nit * NTC * 2 : ((nit + (1 << a.sk_ish) - 1) >> a.sk_ish) * NTC;
         const bool skm = s_skm != 0 && sk_slots <= SK_TMP * 4;
+        if (EXACT_CUT && have) raise_ref(m1);  // (one reference for all threads)
         if (have && m1 > 0.0f && !skm) {
             const float t = m1 - D;
             int lo = t > 0.0f ? (int)__bfloat16_as_ushort(__float2bfloat16_rd(t)) : 1;
@@ -967,7 +996,10 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             for (;;) {
                 const int f = scan_once(thc);
                 if (f != 3) return f;
-                make_exact();  // (then it is settled)
+                // (then it is settled; a sharper range first, as for float32 rows, costs
+                // more than it saves here)
+                __syncthreads();
+                make_exact();
             }
         };
         // ---- reading groups of the sketch back ----
@@ -1619,8 +1651,8 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
             };
             if (!all_in) {
                 find();
-                if (s_nstar != INT_MAX && s_above < s_th) {  // the cut depends on the error of S
-                    make_exact();
+                while (s_nstar != INT_MAX && s_above < s_th) {  // the cut depends on the error of S (at most twice)
+                    sharpen(s_nstar + 1);
                     if (tid == 0) s_nstar = INT_MAX;
                     __syncthreads();
                     find();
@@ -1764,15 +1796,16 @@ void rows_cap_layout(RowArgs &a, int dt, bool ragged) {
             if (ragged && tile == ntile - 2) a.it_partial2 = t / tpi;
         }
     a.inv_ws = (float)(SPB / (double)a.T);
-    // Bound of the relative difference between the row kernel's float32 sum and
-    // the exact 2^-40 one.  Each rounds an id's exponent, at depth d = kref -
-    // z c, by at most d 2^-24 (d 2^-24 ln 2 of its mass), and the mean depth,
-    // weighted by mass, is at most log2(V) + 1 (the masses' entropy less log2
-    // of the total, which is at least 1/2); each has ex2's own error, at most
-    // 2^-22; the float32 sum rounds each mass in at most 8 adds; the exact one
-    // drops less than 2^-40 of every id.
-    a.sum_err = (float)(2.0 * (0.6931472 * ldexp(log2((double)a.V) + 1.0, -24) + ldexp(1.0, -22)) + ldexp(1.0, -21) +
-                        ldexp((double)a.V, -39));
+    // Bounds of the relative difference between the row kernel's float32 sum and
+    // the exact 2^-40 one.  The float32 sum rounds each mass in at most 8 adds and
+    // the exact one drops less than 2^-40 of every id (add_err; the total is at
+    // least 1/2).  Unless both take an id's mass against the same reference, each
+    // rounds its exponent, at depth d = kref - z c, by at most d 2^-24 (d 2^-24 ln
+    // 2 of its mass), and each has ex2's own error, at most 2^-22; the mean depth,
+    // weighted by mass, is the masses' entropy less log2 of the total: at most
+    // log2(V) + 1 (sum_err).
+    a.add_err = (float)(ldexp(1.0, -21) + ldexp((double)a.V, -39));
+    a.sum_err = a.add_err + (float)(2.0 * (0.6931472 * ldexp(log2((double)a.V) + 1.0, -24) + ldexp(1.0, -22)));
     a.nmin = 2 * a.k + 64 > 256 ? 2 * a.k + 64 : 256;
     // sketch groups: 4 chunks (two per thread and iteration) when they fit,
     // else 8 chunks of 2^sk_ish iterations

@@ -734,7 +734,7 @@ __device__ int valhist_row(const RowArgs &a, int r, const RowChunks<ACES_BF16> &
 // done per hit and fewer rows handed over, 153 with the row's exact mass summed
 // in the first read (as the binned path does; with the row kernel's float32 sum
 // 117 of 46080 rows were cut one id away from float64, 34 with the exact one;
-// 163 since the row kernel reads the rows it finishes again where the cut
+// 157 since the row kernel reads the rows it finishes again where the cut
 // depends on that sum's error).
 // What is left is two more reads of those rows by one CTA each.
 constexpr int DH_W = 4096;    // bins
