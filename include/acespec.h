@@ -178,14 +178,15 @@ aces_status aces_verify_noalloc(const void *target_logits, aces_dtype dt, const 
  * that aces_verify keeps for rows its single-pass kernel cannot settle (it
  * reads each row two to four times).  A reference for checking the fast path;
  * not meant for serving.  The results are the same bits, with two exceptions
- * on rows that are on the 16-byte grid (V * element size a multiple of 16 and
- * target_logits 16-byte aligned), where the single-pass kernel's sum of a
- * row's mass is a float32 one, within about 1e-7 of the exact one:
+ * where the single-pass kernel's sum of a row's mass is a float32 one, within
+ * about 1e-7 of the general kernel's exact one:
  *   - float32 rows with top_p = 1 may differ in the last bit of their
- *     probabilities and tail (in aces_verify itself, too, such a row takes
- *     one kernel or the other depending on the rows that finished before it);
- *   - bfloat16 rows with more than 1024 ids of the value at which the nucleus
- *     ends may have a nucleus one id longer or shorter.
+ *     probabilities and tail, and in a draw or an accept test that such a bit
+ *     decides (in aces_verify itself, too, such a row takes one kernel or the
+ *     other depending on the rows that finished before it);
+ *   - bfloat16 rows on the 16-byte grid (V a multiple of 8, target_logits
+ *     16-byte aligned) with more than 1024 ids of the value at which the
+ *     nucleus ends may have a nucleus one id longer or shorter.
  */
 aces_status aces_verify_exact(const void *target_logits, aces_dtype dt, const float *draft_probs,
                               const int32_t *draft_tokens, const float *uniforms, int B, int K, int V,
