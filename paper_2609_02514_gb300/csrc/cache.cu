@@ -133,7 +133,7 @@ __device__ __noinline__ int cache_row_select(const float *qr, int V, int xd, int
 // and F = 4 (a sorted list of four per thread and no threshold: 583, and 700 on
 // wider support, where its insertions diverge), 645 with F = 64 (1000 with lists
 // of eight and a 2048-entry sort a row); 64 rows of full support with F = 64 52
-// us on clusters of eight.  One sequence of 16 x 128256 takes 10 us on clusters of
+// us on clusters of eight.  One sequence of 16 x 128256 takes 9 us on clusters of
 // eight (22 with a CTA a row).  Short rows with wide fan-outs, whose slice is
 // its own sample: 64 x 8 rows of 8000 with F = 256 24 us (102 with the lists).
 __global__ void __launch_bounds__(NTC, 4) k_cache_build(CacheArgs a) {
@@ -209,14 +209,6 @@ __global__ void __launch_bounds__(NTC, 4) k_cache_build(CacheArgs a) {
     };
     load();
     // ---- a threshold from the sample ----
-    // Positive floats order like their bits; negative q (and the padding) are
-    // at most 0 as integers.
-    int mx = 0;
-#pragma unroll
-    for (int u = 0; u < CLD; ++u) mx = max(mx, max(max((int)w[u].x, (int)w[u].y), max((int)w[u].z, (int)w[u].w)));
-    smax[tid] = (uint32_t)mx;
-    if (CL > 1) cl.sync();  // (the first CTA's counter is set before another adds to it)
-    else __syncthreads();
     // Of the `want` largest the sample, a share f of the slice, holds want * f on
     // average; its rank-r value with r four deviations above that is below the
     // want-th largest but for about one row in 10^4 whose ids come in no order,
@@ -224,6 +216,8 @@ __global__ void __launch_bounds__(NTC, 4) k_cache_build(CacheArgs a) {
     // values: the rank among the NTC maxima is corrected for values that share a
     // thread (and r for how their number varies, which is all of r's variance
     // when the sample is the whole slice).
+    int need = 0;      // (warp 0, while its loads are under way)
+    float room = 0.0f;
     if (tid < 32) {
         int ns = 0;  // chunks of the sample, two of its tiles a lane
 #pragma unroll
@@ -237,8 +231,21 @@ __global__ void __launch_bounds__(NTC, 4) k_cache_build(CacheArgs a) {
         const float var = wf * (1.0f - f) + NTC * (exp2f(1.4427f * x) - 1.0f - x);
         const float r = wf + 4.0f * sqrtf(fmaxf(var, 0.0f)) + (f < 1.0f ? 4.0f : 1.0f);
         const auto maxima = [](float values) { return NTC * (1.0f - exp2f(-1.4427f * values / NTC)); };
-        int need = min((int)ceilf(maxima(r)), NTC);
-        if (sure) need = max(need, (int)ceilf(want) + 1);
+        need = min((int)ceilf(maxima(r)), NTC);
+        if (sure) need = (int)ceilf(want) + 1;
+        // the most maxima that may reach the threshold: those of many more values
+        // than asked for and than direct ranking takes, or than the list holds
+        room = maxima(f * fminf(0.75f * CCAP / CL, fmaxf(0.75f * RANK_MAX / CL, 1.5f * r / f)));
+    }
+    // Positive floats order like their bits; negative q (and the padding) are
+    // at most 0 as integers.
+    int mx = 0;
+#pragma unroll
+    for (int u = 0; u < CLD; ++u) mx = max(mx, max(max((int)w[u].x, (int)w[u].y), max((int)w[u].z, (int)w[u].w)));
+    smax[tid] = (uint32_t)mx;
+    if (CL > 1) cl.sync();  // (the first CTA's counter is set before another adds to it)
+    else __syncthreads();
+    if (tid < 32) {
         uint32_t v[NTC / 32], thr = 0u;
         int cnt = NTC, bit = 30;
 #pragma unroll
@@ -256,10 +263,8 @@ __global__ void __launch_bounds__(NTC, 4) k_cache_build(CacheArgs a) {
         };
         // the largest threshold (its exponent and four bits) that `need` maxima reach
         for (; bit >= 19; --bit) try_bit();
-        // more bits while the values that reach it are many more than asked for and
-        // than direct ranking takes, or than the list holds (values alike: 64 x 8
-        // uniform rows of 256000, F = 8: 425 us without, 109)
-        const float room = maxima(f * fminf(0.75f * CCAP / CL, fmaxf(0.75f * RANK_MAX / CL, 1.5f * r / f)));
+        // more bits while too many do (values alike: 64 x 8 uniform rows of 256000, F
+        // = 8: 425 us without, 109)
         if (thr > 0u)
             for (; bit >= 0 && (float)cnt > room; --bit) try_bit();
         if (tid == 0) {
