@@ -430,9 +430,10 @@ __global__ void __launch_bounds__(NTC, 1024 / NTC) k_rows_cap(RowArgs a) {
     // one of the row's exact mass, whichever kernel finishes the row: the
     // float32 sum places the target within a bound, and where the cut is not the
     // same over that whole range (sharpen) the row is read again for its exact
-    // mass, which takes one SM about 5 us for 128256 logits.  (Rows cut one id away from float64, of 128000 each, by the float32
-    // sum and by the exact one: float32 rows of 50000 logits 11 and 6, of 50003 7
-    // and 9, of 20001 5 and 0; bfloat16 rows of 50003 9 and 6, of 20001 1 and 0.)
+    // mass: 5 to 12 us more on a call of one wave.  (Rows cut one id away from
+    // float64, of 128000 each, by the float32 sum and by the exact one: float32
+    // rows of 50000 logits 11 and 6, of 50003 7 and 9, of 20001 5 and 0; bfloat16
+    // rows of 50003 9 and 6, of 20001 1 and 0.)
     constexpr bool EXACT_CUT = !BF || RAGGED;
     extern __shared__ __align__(16) unsigned char smem[];
     // bfloat16: [HPAD dummies, value counts: HW u32 | sketch: SKG u16 | ids >=
